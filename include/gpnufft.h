@@ -98,7 +98,12 @@ typedef struct gp_plan_opts {
   int tile;
   int transform;          /* 0 auto (3 for d = 2 when nf = 2^a; 2 for d = 1 in FP64;
                                else 1);
-                             1 full-grid cuFFT R2C/C2R;
+                             1 full-grid cuFFT R2C/C2R; for d = 3 with a 7-smooth nf
+                               <= 2048 (every grid the plan chooses itself), the
+                               library's own transforms over the box of cells the
+                               plan's points and queries can reach, and from them to
+                               the modes |n_a| <= M (then info.bytes_resident is well
+                               below gp_plan_params' estimate);
                              2 pruned: custom shared-memory row FFTs keeping modes 0..M,
                                cuFFT along the first axis (d <= 2, nf = 2^a);
                              3 pruned, transposed (d = 2, nf = 2^a): custom row FFTs

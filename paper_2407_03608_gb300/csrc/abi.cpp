@@ -495,10 +495,14 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   plan->grid_elems = ps.G;
   plan->spec_elems = ps.S;
   plan->n_freq = ps.nfreq;
+  const bool box3 = !ps.tr3 && !ps.rowfft && box3_supported(d, h.nf);
+  // box transforms keep A' on the octant |n_a| = 0..M only
+  plan->box3.on = box3;
+  if (box3) plan->n_freq = (h.M + 1) * (h.M + 1) * (h.M + 1);
   plan->tr3 = ps.tr3;
   plan->rowfft = ps.rowfft;
   plan->lean = ps.lean;
-  const long long a_bytes = ps.a_bytes;
+  const long long a_bytes = (long long)(C * (C + 1) / 2) * plan->n_freq * (long long)rs;
   GPN_CHECK(o.max_bytes <= 0 || ps.est <= o.max_bytes, GP_ENOMEM,
             "plan needs about " + std::to_string(ps.est) + " device bytes, above max_bytes");
 
@@ -523,6 +527,17 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   // full-grid transforms: room for a spectrum in each grid buffer (cuFFT work areas)
   const long long grid_pitch = (!plan->tr3 && !plan->rowfft) ? std::max(G, 2 * S) : G;
   plan->grid_bytes = (size_t)C * grid_rhs * grid_pitch * rs;
+  GridView& v = plan->view;
+  v.cstride = G;
+  v.rstride = (long long)C * G;
+  for (long long q = d - 1, s = 1; q >= 0; --q, s *= h.nf) {
+    v.stride[q] = s;
+    v.ext[q] = (int)h.nf;
+  }
+  if (box3) {
+    box3_setup(*plan);
+    plan->grid_bytes = (size_t)v.rstride * grid_rhs * rs;
+  }
   plan->grid = plan->alloc(plan->grid_bytes);
   GPN_CUDA(cudaMemsetAsync(plan->grid, 0, plan->grid_bytes, st));
   plan->grid_out = plan->alloc(plan->grid_bytes);
@@ -540,12 +555,12 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
       tr3_setup(*plan);
     else
       build_twiddles(*plan);
-  } else {
+  } else if (!box3) {
     plan->spec = plan->alloc((size_t)C * grid_rhs * S * 2 * rs);
   }
   plan->interp_cc = (int)std::max<size_t>(
       1, std::min<size_t>((size_t)C, kInterpSmemBudget / interp_stage_bytes(d, h.tile, h.width, rs)));
-  if (d >= 2) make_tensor_map(*plan);
+  if (d >= 2 && !box3) make_tensor_map(*plan);
   plan->dev_status = (int*)plan->alloc(sizeof(int));
   GPN_CUDA(cudaMemsetAsync(plan->dev_status, 0, sizeof(int), st));
   GPN_CUDA(cudaMallocHost(&plan->host_status, sizeof(int)));
@@ -567,7 +582,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
     if (o.precision != GP_DF64) plan->t3_plan(1);   // float-float columns are the library's own kernel
   } else if (plan->rowfft) {
     if (d == 2) plan->col_plan(1);
-  } else {
+  } else if (!box3) {
     // the widest batch first, so that the shared cuFFT work area is sized once
     plan->fwd_plan(plan->grid_rhs);
     plan->inv_plan(plan->grid_rhs);

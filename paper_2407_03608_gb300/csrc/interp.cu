@@ -39,8 +39,7 @@ struct InterpArgs {
   int nbins[kMaxDim];
   long long n;
   const T* grid;
-  long long nf;
-  long long G;
+  GridView v;    // layout of the grid
   int width;
   T beta;
   T inv_halfw;
@@ -98,7 +97,7 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
   int P = 1;
 #pragma unroll
   for (int q = 0; q < D - 1; ++q) P *= W;
-  const T* grid_r = a.grid + (size_t)r * C * a.G;
+  const T* grid_r = a.grid + r * a.v.rstride;
   double* out_r = a.out + (size_t)r * a.n;
   const double* alpha_r = a.alpha ? a.alpha + (size_t)r * a.n : nullptr;
 
@@ -148,7 +147,8 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
         rem /= E;
         int soff = 0;
         long long goff = 0;
-        bool in = (long long)base[D - 1] + last < a.nf;
+        const int gx = base[D - 1] + last - a.v.lo[D - 1];
+        bool in = gx >= 0 && gx < a.v.ext[D - 1];
         int lcoord[kMaxDim];
 #pragma unroll
         for (int q = D - 2; q >= 0; --q) {
@@ -158,13 +158,13 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
         const int k = rem;
 #pragma unroll
         for (int q = 0; q < D - 1; ++q) {
-          const long long gq = (long long)base[q] + lcoord[q];
-          in = in && gq < a.nf;
+          const int gq = base[q] + lcoord[q] - a.v.lo[q];
+          in = in && gq >= 0 && gq < a.v.ext[q];
           soff = soff * E + lcoord[q];
-          goff = goff * a.nf + gq;
+          goff += gq * a.v.stride[q];
         }
-        goff = goff * a.nf + base[D - 1] + last;
-        st[(size_t)k * SV + soff * EP + last] = in ? grid_r[(size_t)(c0 + k) * a.G + goff] : T(0);
+        goff += gx * a.v.stride[D - 1];
+        st[(size_t)k * SV + soff * EP + last] = in ? grid_r[(c0 + k) * a.v.cstride + goff] : T(0);
       }
       __syncthreads();
     }
@@ -357,8 +357,7 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
   a.bins = ps.active_bins;
   a.n = ps.n;
   a.grid = (const T*)plan.grid_out;
-  a.nf = g.nf;
-  a.G = plan.grid_elems;
+  a.v = plan.view;
   a.width = g.width;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);
@@ -381,7 +380,11 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
   switch (g.d) {
     case 1: launch_c<T, 1, false>(a, plan.tmap_out, grid, smem, st); break;
     case 2: launch_c<T, 2, true>(a, plan.tmap_out, grid, smem, st); break;
-    default: launch_c<T, 3, true>(a, plan.tmap_out, grid, smem, st);
+    default:
+      if (plan.box3.on)
+        launch_c<T, 3, false>(a, plan.tmap_out, grid, smem, st);
+      else
+        launch_c<T, 3, true>(a, plan.tmap_out, grid, smem, st);
   }
   GPN_CUDA(cudaGetLastError());
 }

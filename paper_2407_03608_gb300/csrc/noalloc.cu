@@ -73,8 +73,7 @@ struct QueryArgs {
   double bary[kMaxChannels];
   int C;
   const T* grid;       // inverse-transformed fine grids, channel k at k * G
-  long long nf;
-  long long G;
+  GridView v;            // layout of the grid
   int width;
   T beta;
   T inv_halfw;
@@ -116,7 +115,7 @@ __global__ void __launch_bounds__(256) k_query_interp(QueryArgs<T> a) {
       // The plan centres the box on the grid with a margin of at least width/2 + 2 cells
       // per side, so for a query inside the box the support lies inside the grid and
       // this test never rejects it; it only guards the grid reads below.
-      ok = ok && l0d >= 0.0 && l0d + W <= (double)a.nf;
+      ok = ok && l0d >= (double)a.v.lo[q] && l0d + W <= (double)(a.v.lo[q] + a.v.ext[q]);
       l0[q] = ok ? (long long)l0d : 0;
       xi[q] = ok ? (T)(g - l0d) : T(0);
     }
@@ -149,13 +148,13 @@ __global__ void __launch_bounds__(256) k_query_interp(QueryArgs<T> a) {
 #pragma unroll
       for (int q = 0; q < D; ++q) {
         wgt *= shfl_val(pq[q], iq[q]);
-        off = off * a.nf + l0[q] + iq[q];
+        off += (l0[q] + iq[q] - a.v.lo[q]) * a.v.stride[q];
       }
       if (valid) {
         const T* gp = a.grid + off;
 #pragma unroll
         for (int k = 0; k < CMAX; ++k)
-          if (k < a.C) madd(acc[k], wgt, ldg_val(gp + (size_t)k * a.G));
+          if (k < a.C) madd(acc[k], wgt, ldg_val(gp + k * a.v.cstride));
       }
     }
 #pragma unroll
@@ -230,8 +229,7 @@ void query_impl(Plan& plan, const double* x, const double* fa, const double* fb,
     a.bary[k] = plan.tb.bary[k];
   }
   a.grid = (const T*)plan.grid_out;
-  a.nf = g.nf;
-  a.G = plan.grid_elems;
+  a.v = plan.view;
   a.width = g.width;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);

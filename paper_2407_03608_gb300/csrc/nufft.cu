@@ -29,7 +29,7 @@ struct ATensorArgs {
   int C;
   int J;
   int d;
-  int quad;             // 1: d = 2 quadrant layout [pair][m_1][m_0], m_a = 0..M
+  int quad;             // 1: m_a = 0..M on every axis, [pair][m_1][m_0] (d = 2), [pair][m_0][m_1][m_2] (d = 3)
 };
 
 __global__ void k_build_a_f32(ATensorArgs<float> a);
@@ -41,7 +41,12 @@ __device__ void build_a_body(const ATensorArgs<T>& a) {
   if (f >= a.n_freq) return;
   long long m[kMaxDim];
   long long rest = f;
-  if (a.quad) {
+  if (a.quad && a.d == 3) {
+    for (int q = 2; q >= 0; --q) {
+      m[q] = rest % (a.M + 1);
+      rest /= a.M + 1;
+    }
+  } else if (a.quad) {
     m[0] = rest % (a.M + 1);
     m[1] = rest / (a.M + 1);
   } else {
@@ -88,15 +93,15 @@ void build_a_tensor(Plan& plan, cudaStream_t st) {
     e = cudaMemcpyAsync(etab, plan.tb.etab.data(), sizeof(double) * plan.tb.etab.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(vt, plan.tb.vt.data(), sizeof(double) * J, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    int nb = blocks_for(plan.n_freq, 128);
+    const int nb = blocks_for(plan.n_freq, 128), quad = plan.tr3 || plan.box3.on;
     if (plan.precision == GP_FP32) {
-      ATensorArgs<float> a{etab, vt, (float*)plan.a_tensor, plan.n_freq, h.M, C, J, h.d, plan.tr3 ? 1 : 0};
+      ATensorArgs<float> a{etab, vt, (float*)plan.a_tensor, plan.n_freq, h.M, C, J, h.d, quad};
       k_build_a_f32<<<nb, 128, 0, st>>>(a);
     } else if (plan.precision == GP_DF64) {
-      ATensorArgs<dd> a{etab, vt, (dd*)plan.a_tensor, plan.n_freq, h.M, C, J, h.d, plan.tr3 ? 1 : 0};
+      ATensorArgs<dd> a{etab, vt, (dd*)plan.a_tensor, plan.n_freq, h.M, C, J, h.d, quad};
       k_build_a_dd<<<nb, 128, 0, st>>>(a);
     } else {
-      ATensorArgs<double> a{etab, vt, (double*)plan.a_tensor, plan.n_freq, h.M, C, J, h.d, plan.tr3 ? 1 : 0};
+      ATensorArgs<double> a{etab, vt, (double*)plan.a_tensor, plan.n_freq, h.M, C, J, h.d, quad};
       k_build_a_f64<<<nb, 128, 0, st>>>(a);
     }
     e = cudaGetLastError();
@@ -179,7 +184,8 @@ void run_fft_forward(Plan& plan, int R, cudaStream_t st) {
   // the row-kernel paths mark between their rows and cuFFT's columns themselves
   if (plan.tr3) return tr3_forward(plan, R, st);
   if (plan.rowfft) return rowfft_forward(plan, R, st);
-  prof_mark(plan, 0, st);                          // all of the phase is cuFFT
+  prof_mark(plan, 0, st);                          // all of the phase is cuFFT (or the box transforms)
+  if (plan.box3.on) return box3_forward(plan, R, st);
   cufftHandle h = plan.fwd_plan(R);
   GPN_CUFFT(cufftSetStream(h, st));
   if (plan.precision == GP_FP32)
@@ -191,6 +197,11 @@ void run_fft_forward(Plan& plan, int R, cudaStream_t st) {
 void run_fft_inverse(Plan& plan, int R, cudaStream_t st) {
   if (plan.tr3) return tr3_inverse(plan, R, st);
   if (plan.rowfft) return rowfft_inverse(plan, R, st);
+  if (plan.box3.on) {
+    box3_inverse(plan, R, st);
+    prof_mark(plan, 1, st);
+    return;
+  }
   cufftHandle h = plan.inv_plan(R);
   GPN_CUFFT(cufftSetStream(h, st));
   if (plan.precision == GP_FP32)

@@ -8,6 +8,7 @@
 #include <cufft.h>
 
 #include "common.h"
+#include "fft_mixed.h"
 #include "params.h"
 
 namespace gpn {
@@ -44,6 +45,27 @@ struct GridGeom {
   int tile;
   int C;                 // channels = n_sigma + 1
   long long M;
+};
+
+// Where a fine-grid value lies: right-hand side r, channel k and cell (c_0, .., c_{d-1}) at
+// r rstride + k cstride + sum_a (c_a - lo_a) stride_a, for lo_a <= c_a < lo_a + ext_a.
+struct GridView {
+  long long rstride = 0, cstride = 0, stride[kMaxDim] = {0, 0, 0};
+  int lo[kMaxDim] = {0, 0, 0}, ext[kMaxDim] = {1, 1, 1};
+};
+
+// 3-D transforms over the occupied box (fft3d.cu)
+struct Box3 {
+  bool on = false;
+  int lo[3] = {0, 0, 0}, ext[3] = {0, 0, 0};   // box cells per axis
+  int Cp = 0;                                  // channel pitch of the grids (even)
+  long long Qp = 0;                            // row pitch of the spectra ((M + 1) C, padded)
+  long long size_a = 0, size_b = 0;            // complex values per right-hand side
+  void* buf_a = nullptr;
+  void* buf_b = nullptr;
+  void* tw = nullptr;
+  fft::MixedPlan fft;
+  int cols = 1, rows = 1, pairs = 1;           // columns / rows and channel pairs a block
 };
 
 // Per-phase event timing of matvecs (diagnostic, off by default).
@@ -157,6 +179,8 @@ struct Plan {
   // transposed pruned path (transform 3, d = 2): fx, fy, fz hold [cr][M+1][nf] columns,
   // the A' tensor is stored on the quadrant [pair][m][|n1|]
   bool tr3 = false;
+  Box3 box3;                            // d = 3 over the occupied box
+  GridView view;                        // layout of grid and grid_out
   int t3_rb = 1;                        // grid rows per CTA of the row kernels
   void* tw_half = nullptr;              // two-level twiddle tables of the row kernels
   void* col_tw = nullptr;               // pass tables of the float-float column transforms
@@ -292,6 +316,13 @@ void tr3_setup(Plan& plan);
 void tr3_forward(Plan& plan, int R, cudaStream_t st);
 void tr3_diag(Plan& plan, int R, cudaStream_t st);
 void tr3_inverse(Plan& plan, int R, cudaStream_t st);
+
+// 3-D transforms and step 3 over the occupied box (fft3d.cu)
+bool box3_supported(int d, long long nf);
+void box3_setup(Plan& plan);
+void box3_forward(Plan& plan, int R, cudaStream_t st);
+void box3_diag(Plan& plan, int R, cudaStream_t st);
+void box3_inverse(Plan& plan, int R, cudaStream_t st);
 
 // Full matvec in sorted order: out = (K~ + shift I) alpha.
 void matvec_sorted(Plan& plan, const double* alpha_sorted, double* out_sorted, int R, double shift, cudaStream_t st);
