@@ -537,6 +537,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   if (box3) {
     box3_setup(*plan);
     plan->grid_bytes = (size_t)v.rstride * grid_rhs * rs;
+    if (spread3d_supported(*plan)) build_spread3d_tiles(*plan, bstart);
   }
   plan->grid = plan->alloc(plan->grid_bytes);
   GPN_CUDA(cudaMemsetAsync(plan->grid, 0, plan->grid_bytes, st));

@@ -132,6 +132,8 @@ struct Plan {
   long long n_active_tiles = 0;
   int* sp2_tiles = nullptr;             // 2-D register-accumulating spread: active 16 x TY tiles
   long long n_sp2_tiles = 0;
+  int* sp3_tiles = nullptr;             // 3-D register-accumulating spread: active tiles
+  long long n_sp3_tiles = 0;
   int interp_cc = 1;                    // channels per interp staging chunk
   CUtensorMap tmap_out;                 // TMA descriptor of grid_out (d >= 2)
   int* dev_status = nullptr;            // set by kernels whose bounded waits ran out
@@ -255,6 +257,10 @@ bool spread2d_supported(const Plan& plan);
 int spread2d_rows(const Plan& plan);
 void build_spread2d_tiles(Plan& plan, const std::vector<int>& bstart);
 void launch_spread2d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st);
+// 3-D spreading with register accumulators on the box grids
+bool spread3d_supported(const Plan& plan);
+void build_spread3d_tiles(Plan& plan, const std::vector<int>& bstart);
+void launch_spread3d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st);
 // Steps (2b)+(3)+(4a): deconvolve, apply A', zero outside the mode box (in spec).
 void launch_diag(Plan& plan, int R, cudaStream_t st);
 // Exact diagonal correction: plan.dcorr[p] = K_pp - K~_pp (points.cu).
