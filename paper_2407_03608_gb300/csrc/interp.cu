@@ -39,7 +39,8 @@ struct InterpArgs {
   int nbins[kMaxDim];
   long long n;
   const T* grid;
-  GridView v;    // layout of the grid
+  long long nf;
+  long long G;
   int width;
   T beta;
   T inv_halfw;
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
   int P = 1;
 #pragma unroll
   for (int q = 0; q < D - 1; ++q) P *= W;
-  const T* grid_r = a.grid + r * a.v.rstride;
+  const T* grid_r = a.grid + (size_t)r * C * a.G;
   double* out_r = a.out + (size_t)r * a.n;
   const double* alpha_r = a.alpha ? a.alpha + (size_t)r * a.n : nullptr;
 
@@ -147,8 +148,7 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
         rem /= E;
         int soff = 0;
         long long goff = 0;
-        const int gx = base[D - 1] + last - a.v.lo[D - 1];
-        bool in = gx >= 0 && gx < a.v.ext[D - 1];
+        bool in = (long long)base[D - 1] + last < a.nf;
         int lcoord[kMaxDim];
 #pragma unroll
         for (int q = D - 2; q >= 0; --q) {
@@ -158,13 +158,13 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
         const int k = rem;
 #pragma unroll
         for (int q = 0; q < D - 1; ++q) {
-          const int gq = base[q] + lcoord[q] - a.v.lo[q];
-          in = in && gq >= 0 && gq < a.v.ext[q];
+          const long long gq = (long long)base[q] + lcoord[q];
+          in = in && gq < a.nf;
           soff = soff * E + lcoord[q];
-          goff += gq * a.v.stride[q];
+          goff = goff * a.nf + gq;
         }
-        goff += gx * a.v.stride[D - 1];
-        st[(size_t)k * SV + soff * EP + last] = in ? grid_r[(c0 + k) * a.v.cstride + goff] : T(0);
+        goff = goff * a.nf + base[D - 1] + last;
+        st[(size_t)k * SV + soff * EP + last] = in ? grid_r[(size_t)(c0 + k) * a.G + goff] : T(0);
       }
       __syncthreads();
     }
@@ -357,7 +357,8 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
   a.bins = ps.active_bins;
   a.n = ps.n;
   a.grid = (const T*)plan.grid_out;
-  a.v = plan.view;
+  a.nf = g.nf;
+  a.G = plan.grid_elems;
   a.width = g.width;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);
@@ -380,11 +381,7 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
   switch (g.d) {
     case 1: launch_c<T, 1, false>(a, plan.tmap_out, grid, smem, st); break;
     case 2: launch_c<T, 2, true>(a, plan.tmap_out, grid, smem, st); break;
-    default:
-      if (plan.box3.on)
-        launch_c<T, 3, false>(a, plan.tmap_out, grid, smem, st);
-      else
-        launch_c<T, 3, true>(a, plan.tmap_out, grid, smem, st);
+    default: launch_c<T, 3, true>(a, plan.tmap_out, grid, smem, st);
   }
   GPN_CUDA(cudaGetLastError());
 }
@@ -414,6 +411,7 @@ size_t interp_stage_bytes(int d, int tile, int width, size_t rs) {
 void launch_interp(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
                    int R, cudaStream_t st) {
   if (ps.n == 0) return;
+  if (plan.box3.on) return launch_interp3d(plan, ps, alpha_sorted, shift, out_sorted, R, st);
   if (plan.precision == GP_FP32)
     interp_impl<float>(plan, ps, alpha_sorted, shift, out_sorted, R, st);
   else if (plan.precision == GP_DF64)

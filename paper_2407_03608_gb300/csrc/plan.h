@@ -284,6 +284,10 @@ void launch_step3_lean(Plan& plan, int R, cudaStream_t st);
 void launch_interp(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
                    int R, cudaStream_t st);
 
+// ... on the 3-D box grids (interp3d.cu)
+void launch_interp3d(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
+                     int R, cudaStream_t st);
+
 // Static scratch of gp_posterior_mean_noalloc (one array per device): a rejected-
 // query counter in the first kNoAllocHeaderBytes, then float64 staging for host
 // queries (x: Nq*d, the two fields: 2*Nq) and for a host output (Nq).
