@@ -512,6 +512,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   if (o.diag_correct) build_diag_correction(*plan, w, sig, st);
   GPN_CHECK(o.near_radius >= 0.0 && std::isfinite(o.near_radius), GP_EINVAL, "near_radius must be >= 0");
   if (o.near_radius > 0.0) build_near_field(*plan, o.near_radius, x.ptr, w, sig, st);
+  if (d == 1) line_points_setup(*plan, st);
   build_active_tiles(*plan, bstart);
   if (spread2d_supported(*plan)) build_spread2d_tiles(*plan, bstart);
   GPN_CHECK(o.precision != GP_DF64 || plan->sp2_tiles, GP_EUNSUPPORTED,
@@ -547,17 +548,27 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
     set_data_extent(*plan);
     const size_t rows = d == 2 ? (size_t)h.nf : 1;
     const size_t fbytes = rows * C * (size_t)grid_rhs * (h.M + 1) * 2 * rs;
-    plan->fx = plan->alloc(fbytes);
-    plan->fy = plan->alloc(fbytes);
-    plan->fz = plan->alloc(fbytes);
+    if (d == 1) {
+      // one allocation, which the split transforms use as a whole
+      plan->fx = plan->alloc(3 * fbytes);
+      plan->fy = (char*)plan->fx + fbytes;
+      plan->fz = (char*)plan->fy + fbytes;
+    } else {
+      plan->fx = plan->alloc(fbytes);
+      plan->fy = plan->alloc(fbytes);
+      plan->fz = plan->alloc(fbytes);
+    }
     GPN_CUDA(cudaMemsetAsync(plan->fx, 0, fbytes, st));
     GPN_CUDA(cudaMemsetAsync(plan->fz, 0, fbytes, st));
     if (plan->tr3)
       tr3_setup(*plan);
+    else if (line_supported(d, h.nf, o.precision, 3 * (h.M + 1)))
+      line_setup(*plan, plan->fx);
     else
       build_twiddles(*plan);
   } else if (!box3) {
     plan->spec = plan->alloc((size_t)C * grid_rhs * S * 2 * rs);
+    if (!plan->lean && line_supported(d, h.nf, o.precision, S)) line_setup(*plan, plan->spec);
   }
   plan->interp_cc = (int)std::max<size_t>(
       1, std::min<size_t>((size_t)C, kInterpSmemBudget / interp_stage_bytes(d, h.tile, h.width, rs)));
@@ -583,7 +594,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
     if (o.precision != GP_DF64) plan->t3_plan(1);   // float-float columns are the library's own kernel
   } else if (plan->rowfft) {
     if (d == 2) plan->col_plan(1);
-  } else if (!box3) {
+  } else if (!box3 && !plan->line) {
     // the widest batch first, so that the shared cuFFT work area is sized once
     plan->fwd_plan(plan->grid_rhs);
     plan->inv_plan(plan->grid_rhs);

@@ -310,9 +310,9 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
 
 // ---- transforms -----------------------------------------------------------------------------
 
-// threads a block: 64 registers a thread in FP32, 128 in float64
+// threads a block: 128 registers a thread in FP32, 255 in float64
 template <typename T>
-constexpr int kLineThreads = sizeof(T) == 4 ? 1024 : 512;
+constexpr int kLineThreads = sizeof(T) == 4 ? 512 : 256;
 constexpr int kMaxSplit = 8;
 // blocks of a launch: at most four an SM
 constexpr int kLineBlocks = 4 * 152;

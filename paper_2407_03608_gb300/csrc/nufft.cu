@@ -183,6 +183,11 @@ cufftHandle Plan::inv_plan(int R) {
 void run_fft_forward(Plan& plan, int R, cudaStream_t st) {
   // the row-kernel paths mark between their rows and cuFFT's columns themselves
   if (plan.tr3) return tr3_forward(plan, R, st);
+  if (plan.line) {
+    line_forward(plan, R, st);
+    prof_mark(plan, 0, st);
+    return;
+  }
   if (plan.rowfft) return rowfft_forward(plan, R, st);
   prof_mark(plan, 0, st);                          // all of the phase is cuFFT (or the box transforms)
   if (plan.box3.on) return box3_forward(plan, R, st);
@@ -196,6 +201,10 @@ void run_fft_forward(Plan& plan, int R, cudaStream_t st) {
 
 void run_fft_inverse(Plan& plan, int R, cudaStream_t st) {
   if (plan.tr3) return tr3_inverse(plan, R, st);
+  if (plan.line) {
+    prof_mark(plan, 1, st);
+    return line_inverse(plan, R, st);
+  }
   if (plan.rowfft) return rowfft_inverse(plan, R, st);
   if (plan.box3.on) {
     box3_inverse(plan, R, st);

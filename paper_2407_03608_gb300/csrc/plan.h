@@ -30,7 +30,7 @@ struct PointSet {
   int* active_bins = nullptr;                          // bins holding at least one point
   long long n_active_bins = 0;
   // kernel values psi(j - xi_a), j < width, per axis [n][width] (real_t, sorted order):
-  // tabulated once for the 2-D float64 and float-float plans, whose kernel values cost
+  // tabulated once for the 1-D and 2-D float64 and float-float plans, whose kernel values cost
   // a float64 or float-float exponential each; null otherwise (the kernels evaluate psi)
   void* psi[kMaxDim] = {nullptr, nullptr, nullptr};
 };
@@ -183,6 +183,14 @@ struct Plan {
   bool tr3 = false;
   Box3 box3;                            // d = 3 over the occupied box
   GridView view;                        // layout of grid and grid_out
+  // d = 1 (line1d.cu): cell groups the points reach, and the split transforms
+  int* line_start = nullptr;            // per group of 32 cells: the run of points reaching it
+  int line_group0 = 0, line_groups = 0;
+  bool line = false;
+  void* line_spec = nullptr;            // [r][C][nf/2] complex
+  void* line_tw = nullptr;              // exp(-2 pi i k / nf)
+  void* line_ptw[4] = {nullptr, nullptr, nullptr, nullptr};   // pass twiddles of nf/2, nf/4, nf/8, nf/16
+  int line_lo = 0, line_hi = 0;         // cells the transforms read and write
   int t3_rb = 1;                        // grid rows per CTA of the row kernels
   void* tw_half = nullptr;              // two-level twiddle tables of the row kernels
   void* col_tw = nullptr;               // pass tables of the float-float column transforms
@@ -197,8 +205,8 @@ struct Plan {
   cufftHandle inv_plan(int R);
 };
 
-// Kernel values tabulated per point (PointSet::psi): the 2-D float64 and float-float plans
-inline bool psi_tabulated(int d, int precision) { return d == 2 && precision != GP_FP32; }
+// Kernel values tabulated per point (PointSet::psi): the 1-D and 2-D float64 and float-float plans
+inline bool psi_tabulated(int d, int precision) { return d <= 2 && precision != GP_FP32; }
 inline bool psi_tabulated(const Plan& p) { return psi_tabulated(p.geom.d, p.precision); }
 
 // Hyperparameters, layout and device footprint of a plan (host only; abi.cpp).
@@ -333,6 +341,17 @@ void box3_setup(Plan& plan);
 void box3_forward(Plan& plan, int R, cudaStream_t st);
 void box3_diag(Plan& plan, int R, cudaStream_t st);
 void box3_inverse(Plan& plan, int R, cudaStream_t st);
+
+// One-dimensional plans (line1d.cu)
+bool line_supported(int d, long long nf, int precision, long long pitch);
+void line_points_setup(Plan& plan, cudaStream_t st);
+void line_setup(Plan& plan, void* spec);
+void line_forward(Plan& plan, int R, cudaStream_t st);
+void line_diag(Plan& plan, int R, cudaStream_t st);
+void line_inverse(Plan& plan, int R, cudaStream_t st);
+void launch_spread1d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st);
+void launch_interp1d(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
+                     int R, cudaStream_t st);
 
 // Full matvec in sorted order: out = (K~ + shift I) alpha.
 void matvec_sorted(Plan& plan, const double* alpha_sorted, double* out_sorted, int R, double shift, cudaStream_t st);

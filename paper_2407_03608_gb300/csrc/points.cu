@@ -114,18 +114,19 @@ __global__ void k_cells(const double* __restrict__ x, long long n, CellArgs ca, 
     lin = lin * ca.nb[a] + b;
   }
   if (!ok) atomicAdd(bad, 1ull);
-  key[i] = (int)lin;
+  key[i] = ca.d == 1 ? l0_out[i] : (int)lin;   // d = 1: sorted by cell within the bins
   idx[i] = (int)i;
 }
 
-// bin_start[b] = first sorted position whose key >= b (lower bound).
-__global__ void k_bin_start(const int* __restrict__ keys, long long n, long long nbins, int* __restrict__ start) {
+// bin_start[b] = first sorted position whose key >= b unit (lower bound; unit: keys a bin).
+__global__ void k_bin_start(const int* __restrict__ keys, long long n, long long nbins, int unit,
+                            int* __restrict__ start) {
   long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (b > nbins) return;
   long long lo = 0, hi = n;
   while (lo < hi) {
     long long mid = (lo + hi) >> 1;
-    if (keys[mid] < b)
+    if (keys[mid] < b * unit)
       lo = mid + 1;
     else
       hi = mid;
@@ -313,14 +314,15 @@ void build_pointset(Plan& plan, PointSet& ps, const double* x_dev, const double*
     if (n > 0) k_cells<<<blocks_for(n, 256), 256, 0, st>>>(x_dev, n, ca, l0_tmp, xi_tmp, keys, idx, bad);
     chk(cudaGetLastError());
     int end_bit = 1;
-    while ((1ll << end_bit) <= ps.nbins_total) ++end_bit;
+    while ((1ll << end_bit) <= (d == 1 ? h.nf : ps.nbins_total)) ++end_bit;
     if (n > 0) {
       chk(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, keys, keys_sorted, idx, ps.perm, (int)n, 0, end_bit, st));
       chk(cudaMalloc(&cub_tmp, std::max<size_t>(cub_bytes, 16)));
       chk(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, keys, keys_sorted, idx, ps.perm, (int)n, 0, end_bit,
                                           st));
     }
-    k_bin_start<<<blocks_for(ps.nbins_total + 1, 256), 256, 0, st>>>(keys_sorted, n, ps.nbins_total, ps.bin_start);
+    k_bin_start<<<blocks_for(ps.nbins_total + 1, 256), 256, 0, st>>>(keys_sorted, n, ps.nbins_total,
+                                                                 d == 1 ? h.tile : 1, ps.bin_start);
     chk(cudaGetLastError());
     ChebArgs cb{};
     cb.C = plan.geom.C;
