@@ -752,9 +752,7 @@ int gp_matvec(gp_plan_t plan, const double* alpha, double* out, int R, double sh
     const size_t cnt = (size_t)p->N * R;
     const double* a = dev_input(alpha, p->stage_in, cnt, st);
     DevOut o(out, p->stage_out, cnt);
-    gather_sorted(p->pts, a, p->vec_a, R, st);
-    matvec_sorted(*p, p->vec_a, p->vec_b, R, shift, st);
-    scatter_sorted(p->pts, p->vec_b, o.dev, R, st);
+    matvec_caller(*p, a, o.dev, R, shift, st);
     GPN_CUDA(cudaGetLastError());
     o.finish(*p, st);
     return GP_OK;

@@ -411,7 +411,7 @@ size_t interp_stage_bytes(int d, int tile, int width, size_t rs) {
 void launch_interp(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
                    int R, cudaStream_t st) {
   if (ps.n == 0) return;
-  if (plan.geom.d == 1) return launch_interp1d(plan, ps, alpha_sorted, shift, out_sorted, R, st);
+  if (plan.geom.d == 1) return launch_interp1d(plan, ps, alpha_sorted, shift, out_sorted, nullptr, R, st);
   if (plan.box3.on) return launch_interp3d(plan, ps, alpha_sorted, shift, out_sorted, R, st);
   if (plan.precision == GP_FP32)
     interp_impl<float>(plan, ps, alpha_sorted, shift, out_sorted, R, st);

@@ -24,7 +24,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "fft_mixed.h"
+#include "fft_core.h"
 #include "kernels.h"
 
 namespace gpn {
@@ -32,7 +32,6 @@ namespace gpn {
 namespace {
 
 using fft::cpx;
-using fft::MixedPlan;
 
 template <typename T>
 struct alignas(2 * sizeof(T)) RawC {
@@ -50,18 +49,20 @@ __device__ __forceinline__ void store_c(cpx<T>* p, cpx<T> v) {
 
 // ---- spreading --------------------------------------------------------------------------
 
-constexpr int kCells = 32;      // cells a block
-constexpr int kWarps = 8;
+constexpr int kSpreadThreads = 256;
+constexpr int kChunk = 128;     // points staged at a time
 
 template <typename T>
 struct Spread1Args {
   const int* l0;
+  const int* perm;       // sorted position -> caller index, when alpha is in the caller's order
   const T* xi;
   const T* psi;          // tabulated kernel values [n][width] (null: evaluate)
   const T* wk;           // [n][C]
-  const int* start;      // per cell group: first point reaching it, first point past it
-  int group0;            // first cell group launched
-  const double* alpha;   // sorted order, n x R column-major
+  const int* start;      // start[c]: first sorted point with l0 >= c, c <= nf
+  int cell0, cell1;      // cells the points reach
+  int cells;             // cells a block
+  const double* alpha;   // n x R column-major
   long long n;
   T* grid;               // [r][k][nf]
   long long nf;
@@ -69,118 +70,93 @@ struct Spread1Args {
   T beta, inv_halfw;
 };
 
+// One thread takes one (cell, channel) pair, one block a run of `cells` cells.  The points that
+// reach the run are one contiguous run of the cell-sorted points; the block stages their kernel
+// values and w_k alpha in shared memory, kChunk points at a time, and every thread walks the
+// points that reach its own cell (again contiguous), so that every multiply-add is a needed
+// one.  The order of the sums is the points' order (results do not depend on scheduling), and
+// every cell the points reach is written, so the grid needs no clearing.
 template <typename T>
-__host__ __device__ constexpr int wk_pitch(int nc) {
-  return (nc + (int)(16 / sizeof(T)) - 1) / (int)(16 / sizeof(T)) * (int)(16 / sizeof(T));
-}
-
-// One block takes 32 cells, one a lane, and all channels in registers (NC = C, or 32 with the
-// extra ones zero).  The points that reach the group are dealt to the warps in runs of up to 32:
-// a warp tabulates its run's kernel values and w_k alpha in shared memory, then walks the run,
-// every lane adding the point's value at its cell.  The warps' sums are added in order (results
-// do not depend on scheduling) and every cell is written, so the grid needs no clearing.
-template <typename T, int NC>
-__global__ void __launch_bounds__(32 * kWarps) k_spread1d(Spread1Args<T> a) {
-  constexpr int WP = wk_pitch<T>(NC), VW = (int)(16 / sizeof(T));
-  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-  const int W = a.width, PS = W | 1, C = a.C, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = blockIdx.y;
+__global__ void __launch_bounds__(kSpreadThreads) k_spread1d(Spread1Args<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* s_wk = reinterpret_cast<T*>(smem_raw) + warp * 32 * (WP + PS + VW);   // [32][WP], then [32][PS]
-  T* s_psi = s_wk + 32 * WP;
-  const int g = a.group0 + blockIdx.x, cell = g * kCells + lane;
-  const int p0 = a.start[2 * g], p1 = a.start[2 * g + 1];
-  // points a warp takes at a time: an even share, so that short runs occupy every warp
-  const int run = min(32, (p1 - p0 + kWarps - 1) / kWarps);
+  const int W = a.width, C = a.C, r = blockIdx.y, tid = threadIdx.x;
+  T* s_wk = reinterpret_cast<T*>(smem_raw);   // [kChunk][C]
+  T* s_psi = s_wk + kChunk * C;               // [kChunk][W]
+  T* s_amp = s_psi + kChunk * W;              // [kChunk]: alpha, converted once a point
+  int* s_l0 = reinterpret_cast<int*>(s_amp + kChunk);
+  const int c0 = a.cell0 + blockIdx.x * a.cells, c1 = min(c0 + a.cells, a.cell1);
+  const int p0 = a.start[max(0, c0 - W + 1)], p1 = a.start[c1];
+  const int ci = tid / C, k = tid - ci * C, cell = c0 + ci;
+  const int pi = tid / W, j = tid - pi * W, pstep = kSpreadThreads / W;
+  const bool on = ci < a.cells && cell < c1;
+  const int q0 = on ? a.start[max(0, cell - W + 1)] : 0, q1 = on ? a.start[cell + 1] : 0;
   const double* alpha = a.alpha + (size_t)r * a.n;
-  T acc[NC];
-#pragma unroll
-  for (int k = 0; k < NC; ++k) acc[k] = T(0);
-  for (int q0 = p0 + warp * run; q0 < p1; q0 += kWarps * run) {
-    const int m = min(run, p1 - q0);
-    const int l0 = lane < m ? a.l0[q0 + lane] : 0;
-    for (int i = lane; i < m * W; i += 32) {
-      const int q = i / W, j = i - q * W;
-      s_psi[q * PS + j] =
-          a.psi ? a.psi[(size_t)q0 * W + i] : psi_at<T>(j, a.xi[q0 + q], a.beta, a.inv_halfw);
+  T acc = T(0);
+  for (int base = p0; base < p1; base += kChunk) {
+    const int m = min(kChunk, p1 - base);
+    for (int i = tid; i < m; i += kSpreadThreads) {
+      s_l0[i] = a.l0[base + i];
+      s_amp[i] = (T)alpha[a.perm ? a.perm[base + i] : base + i];
     }
-    for (int i = lane; i < m * C; i += 32) {
-      const int q = i / C, k = i - q * C;
-      s_wk[q * WP + k] = a.wk[(size_t)q0 * C + i] * (T)alpha[q0 + q];
-    }
-    if (C < NC)
-      for (int q = lane; q < m; q += 32)
-        for (int k = C; k < NC; ++k) s_wk[q * WP + k] = T(0);
-    __syncwarp();
-    for (int q = 0; q < m; ++q) {
-      const int j = cell - __shfl_sync(0xffffffffu, l0, q);
-      const T ps = (unsigned)j < (unsigned)W ? s_psi[q * PS + j] : T(0);
-      T w[WP];
-#pragma unroll
-      for (int v = 0; v < WP / VW; ++v) {
-        const V u = reinterpret_cast<const V*>(s_wk + q * WP)[v];
-        w[VW * v] = u.x;
-        w[VW * v + 1] = u.y;
-        if constexpr (VW == 4) {
-          w[VW * v + 2] = u.z;
-          w[VW * v + 3] = u.w;
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < NC; ++k) acc[k] += ps * w[k];
-    }
-    __syncwarp();
+    if (pi < pstep)
+      for (int q = pi; q < m; q += pstep)
+        s_psi[q * W + j] = a.psi ? a.psi[(size_t)(base + q) * W + j]
+                                 : psi_at<T>(j, a.xi[base + q], a.beta, a.inv_halfw);
+    __syncthreads();
+    if (ci < a.cells)
+      for (int q = ci; q < m; q += a.cells) s_wk[q * C + k] = a.wk[(size_t)(base + q) * C + k] * s_amp[q];
+    __syncthreads();
+    const int e = min(q1 - base, m);
+    T part = T(0);   // a chunk's sum on its own: dense cells add their points in two levels
+#pragma unroll 4
+    for (int q = max(q0 - base, 0); q < e; ++q) part += s_psi[q * W + (cell - s_l0[q])] * s_wk[q * C + k];
+    acc += part;
+    __syncthreads();
   }
+  // the run's sums leave through shared memory, cells fastest
+  T* s_out = reinterpret_cast<T*>(smem_raw);
+  if (on) s_out[k * a.cells + ci] = acc;
   __syncthreads();
-  T* red = reinterpret_cast<T*>(smem_raw);   // [warp][NC][32]
-#pragma unroll
-  for (int k = 0; k < NC; ++k) red[(warp * NC + k) * 32 + lane] = acc[k];
-  __syncthreads();
-  if (cell >= a.nf) return;
-  for (int k = warp; k < C; k += kWarps) {
-    T s = T(0);
-#pragma unroll
-    for (int q = 0; q < kWarps; ++q) s += red[(q * NC + k) * 32 + lane];
-    a.grid[((size_t)r * C + k) * a.nf + cell] = s;
-  }
-}
-
-template <typename T, int NC>
-void spread_launch(const Spread1Args<T>& a, dim3 grid, cudaStream_t st) {
-  const size_t tab = 32 * (size_t)(wk_pitch<T>(NC) + (a.width | 1) + (int)(16 / sizeof(T)));
-  const size_t smem = kWarps * sizeof(T) * std::max<size_t>(tab, 32 * NC);
-  GPN_CUDA(cudaFuncSetAttribute(k_spread1d<T, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_spread1d<T, NC><<<grid, 32 * kWarps, smem, st>>>(a);
-}
-
-template <typename T, int NC>
-void spread_dispatch(const Spread1Args<T>& a, dim3 grid, cudaStream_t st) {
-  if constexpr (NC > 16) {
-    spread_launch<T, 32>(a, grid, st);
-  } else {
-    if (a.C == NC)
-      spread_launch<T, NC>(a, grid, st);
-    else
-      spread_dispatch<T, NC + 1>(a, grid, st);
+  const int nc = c1 - c0;
+  for (int i = tid; i < nc * C; i += kSpreadThreads) {
+    const int kk = i / nc, c = i - kk * nc;
+    a.grid[((size_t)r * C + kk) * a.nf + c0 + c] = s_out[kk * a.cells + c];
   }
 }
 
 template <typename T>
-void spread_impl(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st) {
+void spread_impl(Plan& plan, const double* alpha, const int* perm, int R, cudaStream_t st) {
   const GridGeom& g = plan.geom;
   const PointSet& ps = plan.pts;
-  Spread1Args<T> a{ps.cell0[0],      (const T*)ps.xi[0], (const T*)ps.psi[0], (const T*)ps.wk,
-                   plan.line_start,  plan.line_group0,   alpha_sorted,        ps.n,
-                   (T*)plan.grid,    g.nf,               g.width,             g.C,
-                   es_beta_arg<T>(g.beta), (T)(2.0 / g.width)};
-  spread_dispatch<T, 1>(a, dim3((unsigned)plan.line_groups, (unsigned)R), st);
+  Spread1Args<T> a{};
+  a.l0 = ps.cell0[0];
+  a.perm = perm;
+  a.xi = (const T*)ps.xi[0];
+  a.psi = (const T*)ps.psi[0];
+  a.wk = (const T*)ps.wk;
+  a.start = plan.line_start;
+  a.cell0 = plan.line_cell0;
+  a.cell1 = plan.line_cell1;
+  a.cells = std::max(1, kSpreadThreads / g.C);
+  a.alpha = alpha;
+  a.n = ps.n;
+  a.grid = (T*)plan.grid;
+  a.nf = g.nf;
+  a.width = g.width;
+  a.C = g.C;
+  a.beta = es_beta_arg<T>(g.beta);
+  a.inv_halfw = (T)(2.0 / g.width);
+  const size_t smem = kChunk * ((g.C + g.width + 1) * sizeof(T) + sizeof(int));
+  GPN_CUDA(cudaFuncSetAttribute(k_spread1d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int blocks = (a.cell1 - a.cell0 + a.cells - 1) / a.cells;
+  k_spread1d<T><<<dim3((unsigned)blocks, (unsigned)R), kSpreadThreads, smem, st>>>(a);
   GPN_CUDA(cudaGetLastError());
 }
 
-// start[2g], start[2g + 1]: the sorted points whose support meets cells [32 g, 32 g + 32)
-__global__ void k_line_start(const int* __restrict__ l0, int n, int W, int groups, int* __restrict__ start) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2 * groups) return;
-  const int c = (i / 2) * kCells + (i % 2 ? kCells : 1 - W);   // first l0 past the group / reaching it
+// start[c], c = 0 .. nf: first sorted point with l0 >= c
+__global__ void k_line_start(const int* __restrict__ l0, int n, int cells, int* __restrict__ start) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c > cells) return;
   int lo = 0, hi = n;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -189,7 +165,7 @@ __global__ void k_line_start(const int* __restrict__ l0, int n, int W, int group
     else
       hi = mid;
   }
-  start[i] = lo;
+  start[c] = lo;
 }
 
 // ---- interpolation ------------------------------------------------------------------------
@@ -197,6 +173,7 @@ __global__ void k_line_start(const int* __restrict__ l0, int n, int W, int group
 template <typename T>
 struct Interp1Args {
   const int* l0;
+  const int* perm;       // sorted position -> caller index, when alpha and out are in the caller's order
   const T* xi;
   const T* psi;
   const T* wk;
@@ -213,12 +190,23 @@ struct Interp1Args {
 
 template <typename T>
 __device__ __forceinline__ void finish_point(const Interp1Args<T>& a, long long p, int r, double res) {
-  if (a.alpha) res += (a.dcorr ? a.shift + a.dcorr[p] : a.shift) * a.alpha[(size_t)r * a.n + p];
-  a.out[(size_t)r * a.n + p] = res;
+  const long long i = (size_t)r * a.n + (a.perm ? a.perm[p] : p);
+  if (a.alpha) res += (a.dcorr ? a.shift + a.dcorr[p] : a.shift) * a.alpha[i];
+  a.out[i] = res;
 }
 
+// sum + w b, the product exact: in float64, or for FP32 plans in float-float (conversions to
+// float64 run on its pipe, at a sixteenth of the FP32 rate)
+__device__ __forceinline__ void add_product(double& sum, double w, double b) { sum += w * b; }
+__device__ __forceinline__ void add_product(dd& sum, float w, float b) {
+  const float p = ffops::mul(w, b);
+  sum += dd(p, ffops::fma(w, b, -p));
+}
+template <typename T>
+using SumOf = typename std::conditional<sizeof(T) == 4, dd, double>::type;
+
 // Sixteen lanes a point: lane j holds psi(j), lane k sums channel k (k + 16, ...) over the W
-// cells; the products w_k beta_k are added in float64.  For point sets too small to fill the
+// cells; the products w_k beta_k are added exactly (see add_product).  For point sets too small to fill the
 // chip with a thread a point (and for float64, whose kernel values it spreads over the lanes).
 template <typename T>
 __global__ void __launch_bounds__(128) k_interp1d_lanes(Interp1Args<T> a) {
@@ -229,19 +217,23 @@ __global__ void __launch_bounds__(128) k_interp1d_lanes(Interp1Args<T> a) {
   const T* g = a.grid + (size_t)r * a.C * a.nf + a.l0[q];
   T pj = T(0);
   if (gl < W) pj = a.psi ? a.psi[q * W + gl] : psi_at<T>(gl, a.xi[q], a.beta, a.inv_halfw);
-  double part = 0.0;
+  SumOf<T> part(0.0);
   for (int k0 = 0; k0 < a.C; k0 += 16) {
     const bool in = k0 + gl < a.C;
     const int k = in ? k0 + gl : a.C - 1;
     const T* gk = g + (size_t)k * a.nf;
-    T s = T(0);
-#pragma unroll 4
-    for (int j = 0; j < W; ++j) s += __shfl_sync(0xffffffffu, pj, j, 16) * __ldg(gk + j);
-    if (in) part += (double)(a.wk[q * a.C + k] * s);
+    const T w = in ? a.wk[q * a.C + k] : T(0);
+    T v[kMaxWidth], s = T(0);   // every cell is loaded before the first sum
+#pragma unroll
+    for (int j = 0; j < kMaxWidth; ++j) v[j] = j < W ? __ldg(gk + j) : T(0);
+#pragma unroll
+    for (int j = 0; j < kMaxWidth; ++j)
+      if (j < W) s += __shfl_sync(0xffffffffu, pj, j, 16) * v[j];
+    add_product(part, w, s);
   }
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o, 16);
-  if (on && gl == 0) finish_point(a, p, r, part);
+  for (int o = 8; o > 0; o >>= 1) part += shfl_xor_val(part, o);
+  if (on && gl == 0) finish_point(a, p, r, (double)part);
 }
 
 // A thread a point, NC = C channels in registers (32 with the extra ones unused): neighbouring
@@ -262,11 +254,11 @@ __global__ void __launch_bounds__(128) k_interp1d(Interp1Args<T> a) {
     for (int k = 0; k < NC; ++k)
       if (NC <= 16 || k < C) acc[k] += ps * __ldg(g + (size_t)k * a.nf + j);
   }
-  double res = 0.0;
+  SumOf<T> res(0.0);
 #pragma unroll
   for (int k = 0; k < NC; ++k)
-    if (NC <= 16 || k < C) res += (double)a.wk[p * C + k] * (double)acc[k];
-  finish_point(a, p, r, res);
+    if (NC <= 16 || k < C) add_product(res, a.wk[p * C + k], acc[k]);
+  finish_point(a, p, r, (double)res);
 }
 
 template <typename T, int NC>
@@ -282,10 +274,11 @@ void interp_dispatch(const Interp1Args<T>& a, dim3 grid, cudaStream_t st) {
 }
 
 template <typename T>
-void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted, int R,
+void interp_impl(Plan& plan, const PointSet& ps, const double* alpha, double shift, double* out, const int* perm, int R,
                  cudaStream_t st) {
   const GridGeom& g = plan.geom;
   Interp1Args<T> a{ps.cell0[0],
+                   perm,
                    (const T*)ps.xi[0],
                    (const T*)ps.psi[0],
                    (const T*)ps.wk,
@@ -296,10 +289,10 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
                    g.C,
                    es_beta_arg<T>(g.beta),
                    (T)(2.0 / g.width),
-                   alpha_sorted,
+                   alpha,
                    shift,
                    (&ps == &plan.pts) ? plan.dcorr : nullptr,
-                   out_sorted};
+                   out};
   // a thread a point once the points fill half of the chip's threads (152 SMs x 1024)
   if (ps.n * R >= 152ll * 1024)
     interp_dispatch<T, 1>(a, dim3((unsigned)((ps.n + 127) / 128), (unsigned)R), st);
@@ -310,12 +303,18 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
 
 // ---- transforms -----------------------------------------------------------------------------
 
-// threads a block: 128 registers a thread in FP32, 255 in float64
-template <typename T>
-constexpr int kLineThreads = sizeof(T) == 4 ? 512 : 256;
 constexpr int kMaxSplit = 8;
-// blocks of a launch: at most four an SM
-constexpr int kLineBlocks = 4 * 152;
+// blocks wanted in a launch: three quarters of the SMs
+constexpr int kLineBlocks = 114;
+
+// The passes of the N-point sub-transform: one of radix r0 (2 or 4, or 1: none), then np of
+// radix R; a thread holds NB butterflies of radix R.  The passes run as one loop over the same
+// code: a block runs each pass once, so unrolled passes would be bound by instruction fetches
+// (measured: 31 us for 512-point float64 sub-transforms with unrolled radix-8 passes, an
+// estimated 7 us of which is arithmetic).
+struct LinePlan {
+  int N = 0, R = 0, NB = 0, r0 = 1, np = 0;
+};
 
 template <typename T>
 struct LineArgs {
@@ -323,7 +322,7 @@ struct LineArgs {
   cpx<T>* out;
   const cpx<T>* tw;      // exp(-2 pi i k / nf), k < nf
   const cpx<T>* ptw;     // pass twiddles of the h / S point transform
-  MixedPlan m;
+  int N, r0, np;
   int h;
   int lo, hi;            // pairs of the row that hold data or are read by the interpolation
 };
@@ -335,23 +334,40 @@ __device__ __forceinline__ cpx<T> quarter_turns(cpx<T> a, int q) {
   return q & 2 ? cpx<T>{-a.x, -a.y} : a;
 }
 
-template <bool INV, bool HELD, typename T, typename In, typename Out, typename Sync>
-__device__ __forceinline__ void line_pass(int R, int N, int J, int Ns, int jl, const cpx<T>* tw, In in, Out out,
-                                          Sync sync) {
-  switch (R) {
-    case 16: fft::mixed_pass<16, INV, HELD>(N, J, Ns, jl, tw, in, out, sync); break;
-    case 8: fft::mixed_pass<8, INV, HELD>(N, J, Ns, jl, tw, in, out, sync); break;
-    case 4: fft::mixed_pass<4, INV, HELD>(N, J, Ns, jl, tw, in, out, sync); break;
-    default: fft::mixed_pass<2, INV, HELD>(N, J, Ns, jl, tw, in, out, sync);
+// one Stockham pass in place, NB butterflies a thread (J threads)
+template <int R, int NB, bool INV, typename T>
+__device__ __forceinline__ void line_pass(cpx<T>* s, int N, int J, int Ns, int t, const cpx<T>* tw) {
+  const int nbf = N / R;
+  cpx<T> v[NB][R];
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[b][r] = load_c(s + t + b * J + r * nbf);
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int j = t + b * J, k = j & (Ns - 1);
+    if (Ns > 1) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) {
+        cpx<T> w = load_c(tw + (r - 1) * Ns + k);
+        if (INV) w.y = -w.y;
+        v[b][r] = fft::cmul(v[b][r], w);
+      }
+    }
+    fft::dft<INV, R>(v[b]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) store_c(s + (j - k) * R + k + r * Ns, v[b][r]);
   }
+  __syncthreads();
 }
 
-// blockIdx = (output residue q, channel and right-hand side)
-template <typename T, bool INV, int S>
-__global__ void __launch_bounds__(kLineThreads<T>, 1) k_line(LineArgs<T> a) {
+// blockIdx = (output residue q, channel and right-hand side); N / (R NB) threads
+template <typename T, bool INV, int S, int R, int NB>
+__global__ void __launch_bounds__(512) k_line(LineArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* s = reinterpret_cast<cpx<T>*>(smem_raw);
-  const int N = a.m.N, J = a.m.J, jl = threadIdx.x, q = blockIdx.x;
+  const int N = a.N, J = blockDim.x, t = threadIdx.x, q = blockIdx.x;
   const cpx<T>* src = a.in + (size_t)blockIdx.y * a.h;
   cpx<T>* dst = a.out + (size_t)blockIdx.y * a.h;
   auto twid = [&](int i) {
@@ -359,45 +375,44 @@ __global__ void __launch_bounds__(kLineThreads<T>, 1) k_line(LineArgs<T> a) {
     if (INV) w.y = -w.y;
     return w;
   };
-  auto at = [&](int j) {
-    return INV || (j >= a.lo && j < a.hi) ? load_c(src + j) : cpx<T>{T(0), T(0)};
-  };
   const cpx<T> w8 = S == 8 ? twid(q * (a.h / 4)) : cpx<T>{T(1), T(0)};   // W_8^q
-  auto sums = [&](int n) -> cpx<T> {
-    if constexpr (S == 1) return at(n);
-    cpx<T> z[S], u;
+#pragma unroll 2
+  for (int n = t; n < N; n += J) {
+    cpx<T> z[S];
 #pragma unroll
-    for (int i = 0; i < S; ++i) z[i] = at(n + i * N);
-    // W_S^{i q}: the halves pair up with the sign (-1)^q, the quarters with quarter turns
-#pragma unroll
-    for (int i = 0; i < S / 2; ++i) z[i] = q & 1 ? z[i] - z[i + S / 2] : z[i] + z[i + S / 2];
-    if constexpr (S == 2) u = z[0];
-    if constexpr (S == 4) u = z[0] + quarter_turns<INV>(z[1], q & 3);
-    if constexpr (S == 8) {
-      const cpx<T> u0 = z[0] + quarter_turns<INV>(z[2], q & 3), u1 = z[1] + quarter_turns<INV>(z[3], q & 3);
-      u = u0 + (q & 1 ? fft::cmul(u1, w8) : quarter_turns<INV>(u1, q / 2));
+    for (int i = 0; i < S; ++i) {
+      const int j = n + i * N;
+      z[i] = INV || (j >= a.lo && j < a.hi) ? load_c(src + j) : cpx<T>{T(0), T(0)};
     }
-    return q == 0 ? u : fft::cmul(u, twid(2 * n * q));
-  };
-  auto put = [&](int k, cpx<T> v) {
-    const int j = q + S * k;
-    if (!INV || (j >= a.lo && j < a.hi)) store_c(dst + j, v);
-  };
-  line_pass<INV, false, T>(a.m.R[0], N, J, 1, jl, a.ptw, sums, [&](int n, cpx<T> v) { store_c(s + n, v); }, [] {});
+    // W_S^{i q}: the halves pair up with the sign (-1)^q, the quarters with quarter turns
+    if constexpr (S > 1) {
+      const cpx<T> w = twid(2 * n * q);
+#pragma unroll
+      for (int i = 0; i < S / 2; ++i) z[i] = q & 1 ? z[i] - z[i + S / 2] : z[i] + z[i + S / 2];
+      if constexpr (S == 4) z[0] = z[0] + quarter_turns<INV>(z[1], q & 3);
+      if constexpr (S == 8) {
+        const cpx<T> u0 = z[0] + quarter_turns<INV>(z[2], q & 3), u1 = z[1] + quarter_turns<INV>(z[3], q & 3);
+        z[0] = u0 + (q & 1 ? fft::cmul(u1, w8) : quarter_turns<INV>(u1, q / 2));
+      }
+      z[0] = fft::cmul(z[0], w);
+    }
+    store_c(s + n, z[0]);
+  }
   __syncthreads();
-  int ns = a.m.R[0];
-  for (int p = 1; p + 1 < a.m.np; ++p) {
-    line_pass<INV, true, T>(a.m.R[p], N, J, ns, jl, a.ptw + a.m.tw[p], [&](int n) { return load_c(s + n); },
-                            [&](int n, cpx<T> v) { store_c(s + n, v); }, [] { __syncthreads(); });
-    __syncthreads();
-    ns *= a.m.R[p];
+  const cpx<T>* tw = a.ptw;
+  int ns = a.r0;
+  if (a.r0 == 2) line_pass<2, R * NB / 2, INV, T>(s, N, J, 1, t, tw);
+  if (a.r0 == 4) line_pass<4, (R * NB > 4 ? R * NB / 4 : 1), INV, T>(s, N, J, 1, t, tw);
+#pragma unroll 1
+  for (int p = 0; p < a.np; ++p) {
+    line_pass<R, NB, INV, T>(s, N, J, ns, t, tw);
+    if (ns > 1) tw += (R - 1) * ns;
+    ns *= R;
   }
-  if (a.m.np == 1) {
-    for (int n = jl; n < N; n += blockDim.x) put(n, load_c(s + n));
-    return;
+  for (int n = t; n < N; n += J) {
+    const int j = q + S * n;
+    if (!INV || (j >= a.lo && j < a.hi)) store_c(dst + j, load_c(s + n));
   }
-  line_pass<INV, false, T>(a.m.R[a.m.np - 1], N, J, ns, jl, a.ptw + a.m.tw[a.m.np - 1],
-                           [&](int n) { return load_c(s + n); }, put, [] {});
 }
 
 // ---- step 3 on the pairs (k, h - k) -----------------------------------------------------------
@@ -410,10 +425,10 @@ struct LineDiagArgs {
   const cpx<T>* tw;      // exp(-2 pi i k / nf)
   const T* A;            // packed upper triangle [p][f], f = 0..M
   long long n_freq;
-  int h, M, C, R;
+  int h, M, C;
 };
 
-// blockDim = (kDiagK pairs, C channels)
+// blockIdx = (pair group, right-hand side), blockDim = (kDiagK pairs, C channels)
 template <typename T>
 __global__ void __launch_bounds__(1024) k_line_diag(LineDiagArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -422,86 +437,104 @@ __global__ void __launch_bounds__(1024) k_line_diag(LineDiagArgs<T> a) {
   cpx<T>* s_hi = s_lo + C * kDiagK;                     // X[h - k]
   const int k = blockIdx.x * kDiagK + tx, kn = h - k;
   const bool on = k <= h / 2, lo = on && k <= a.M, hi = on && kn <= a.M;
-  const cpx<T> w = on ? load_c(a.tw + k) : cpx<T>{T(1), T(0)}, wn{-w.x, w.y};   // W_nf^{h-k} = -conj W_nf^k
+  const cpx<T> w = on ? load_c(a.tw + k) : cpx<T>{T(1), T(0)};
   const int rowp = c * C - c * (c - 1) / 2;
-  for (int r = 0; r < a.R; ++r) {
-    cpx<T>* Z = a.Z + ((size_t)r * C + c) * h;
-    cpx<T> zk{T(0), T(0)}, zn{T(0), T(0)};
-    if (lo) {
-      zk = load_c(Z + k);
-      zn = load_c(Z + (kn & (h - 1)));
-    }
-    store_c(s_lo + c * kDiagK + tx, fft::r2c_split(zk, zn, w));
-    if (hi) store_c(s_hi + c * kDiagK + tx, fft::r2c_split(zn, zk, wn));
-    __syncthreads();
-    cpx<T> a0{T(0), T(0)}, a1{T(0), T(0)};
-    if (lo) {
-      for (int l = 0; l < C; ++l) {
-        const int p = l >= c ? rowp + (l - c) : l * C - l * (l - 1) / 2 + (c - l);
-        const T* Ap = a.A + (size_t)p * a.n_freq;
-        const T v = __ldg(Ap + k);
-        const cpx<T> b = load_c(s_lo + l * kDiagK + tx);
-        a0.x += v * b.x;
-        a0.y += v * b.y;
-        if (hi) {
-          const T vn = __ldg(Ap + kn);
-          const cpx<T> bn = load_c(s_hi + l * kDiagK + tx);
-          a1.x += vn * bn.x;
-          a1.y += vn * bn.y;
-        }
+  cpx<T>* Z = a.Z + ((size_t)blockIdx.y * C + c) * h;
+  cpx<T> zk{T(0), T(0)}, zn{T(0), T(0)};
+  if (lo) {
+    zk = load_c(Z + k);
+    zn = load_c(Z + (kn & (h - 1)));
+  }
+  // with c = conj Z[h-k], e = Z[k] + c, o = Z[k] - c, p = W^k o: X[k] = (e - i p) / 2 and
+  // X[h-k] = conj(e + i p) / 2
+  {
+    const cpx<T> e{zk.x + zn.x, zk.y - zn.y}, o{zk.x - zn.x, zk.y + zn.y}, p = fft::cmul(w, o);
+    store_c(s_lo + c * kDiagK + tx, {T(0.5) * (e.x + p.y), T(0.5) * (e.y - p.x)});
+    if (hi) store_c(s_hi + c * kDiagK + tx, {T(0.5) * (e.x - p.y), -T(0.5) * (e.y + p.x)});
+  }
+  __syncthreads();
+  cpx<T> a0{T(0), T(0)}, a1{T(0), T(0)};
+  if (lo) {
+#pragma unroll 5
+    for (int l = 0; l < C; ++l) {
+      const int p = l >= c ? rowp + (l - c) : l * C - l * (l - 1) / 2 + (c - l);
+      const T* Ap = a.A + (size_t)p * a.n_freq;
+      const T v = __ldg(Ap + k);
+      const cpx<T> b = load_c(s_lo + l * kDiagK + tx);
+      a0.x += v * b.x;
+      a0.y += v * b.y;
+      if (hi) {
+        const T vn = __ldg(Ap + kn);
+        const cpx<T> bn = load_c(s_hi + l * kDiagK + tx);
+        a1.x += vn * bn.x;
+        a1.y += vn * bn.y;
       }
     }
-    if (on) {
-      store_c(Z + k, fft::c2r_merge(a0, a1, w));
-      if (k != 0 && kn != k) store_c(Z + kn, fft::c2r_merge(a1, a0, wn));
-    }
-    __syncthreads();   // the next right-hand side refills the modes
+  }
+  if (on) {
+    // with c = conj a1, e = a0 + c, o = a0 - c, p = conj(W^k) o: Z[k] = e + i p, Z[h-k] = conj(e - i p)
+    const cpx<T> e{a0.x + a1.x, a0.y - a1.y}, o{a0.x - a1.x, a0.y + a1.y}, p = fft::cmul(fft::conj(w), o);
+    store_c(Z + k, {e.x - p.y, e.y + p.x});
+    if (k != 0 && kn != k) store_c(Z + kn, {e.x + p.y, p.x - e.y});
   }
 }
 
-// the passes of the h / S point transform: radix 8 (16 for long ones) and a last 4 or 2
-MixedPlan line_passes(int n) {
-  MixedPlan m;
+// Radix 4 up to 1024 points (256 threads), radix 8 above in FP32 and four butterflies of radix
+// 4 a thread in float64 (whose radix-8 butterflies would not fit the registers)
+LinePlan line_passes(int n, int precision) {
+  LinePlan m;
   m.N = n;
-  const int big = n >= 2048 ? 16 : 8;
-  for (int rest = n; rest > 1; ++m.np) {
-    int r = big;
-    while (rest % r) r /= 2;
-    if (m.np == fft::kMaxPasses) return MixedPlan{};
-    m.R[m.np] = r;
-    rest /= r;
+  m.R = precision == GP_FP32 && n > 1024 ? 8 : 4;
+  m.NB = n <= 1024 ? 1 : (m.R == 8 ? (n <= 4096 ? 1 : 2) : 4);
+  int rest = n;
+  while (rest % m.R == 0) {
+    rest /= m.R;
+    ++m.np;
   }
-  m.J = std::max(1, n / big);
-  int off = 0, ns = 1;
-  for (int p = 0; p < m.np; ++p) {
-    m.tw[p] = off;
-    if (p > 0) off += (m.R[p] - 1) * ns;
-    ns *= m.R[p];
-  }
+  m.r0 = rest;
+  const size_t bytes = (precision == GP_FP32 ? 8 : 16) * (size_t)n;
+  if (n < 4 || n / (m.R * m.NB) > 512 || bytes > (size_t(128) << 10)) m.N = 0;
   return m;
 }
+bool passes_fit(int n, int precision) { return line_passes(n, precision).N > 0; }
 
-template <typename T>
-bool passes_fit(int n) {
-  const MixedPlan m = line_passes(n);
-  return m.np > 0 && m.J <= kLineThreads<T> && sizeof(cpx<T>) * (size_t)n <= (size_t(128) << 10);
+// the pass twiddles W_{Ns R}^{r k}, [r - 1][k], k < Ns, as interleaved (re, im)
+std::vector<double> line_tables(const LinePlan& m) {
+  std::vector<double> t;
+  int ns = m.r0;
+  for (int p = 0; p < m.np; ++p, ns *= m.R)
+    if (ns > 1)
+      for (int r = 1; r < m.R; ++r)
+        for (int k = 0; k < ns; ++k) {
+          const double th = 6.283185307179586476925286766559 * (double)(r * k) / ((double)ns * m.R);
+          t.push_back(std::cos(th));
+          t.push_back(-std::sin(th));
+        }
+  return t;
 }
-bool passes_fit(int n, int precision) { return precision == GP_FP32 ? passes_fit<float>(n) : passes_fit<double>(n); }
 
-// blocks a transform is split over: as many as keep the launch within kLineBlocks, more where
-// the sub-transform would not fit a block, fewer where it would drop below 64 points
+// Blocks a transform is split over: the fewest that give kLineBlocks blocks (every block reads
+// the whole sequence, so S multiplies the reads from L2), more where the sub-transform would
+// not fit a block, fewer where it would drop below 64 points.  Measured at N = 1e5 FP32 with
+// 40 sequences of 32768: 29 us with S = 8.
 int line_split(const Plan& plan, int CR) {
   const int h = (int)(plan.geom.nf / 2);
-  int S = kMaxSplit;
-  while (S > 1 && ((long long)CR * S > kLineBlocks || h / S < 64) && passes_fit(h / (S / 2), plan.precision)) S /= 2;
+  int S = 1;
+  while (S < kMaxSplit && (!passes_fit(h / S, plan.precision) || ((long long)CR * S < kLineBlocks && h / S >= 128)))
+    S *= 2;
   return S;
 }
 
 template <typename T, bool INV, int S>
-void line_launch(const LineArgs<T>& a, int CR, cudaStream_t st) {
-  const size_t smem = sizeof(cpx<T>) * (size_t)a.m.N;
-  GPN_CUDA(cudaFuncSetAttribute(k_line<T, INV, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_line<T, INV, S><<<dim3(S, (unsigned)CR), a.m.J, smem, st>>>(a);
+void line_launch(const LineArgs<T>& a, const LinePlan& m, int CR, cudaStream_t st) {
+  const size_t smem = sizeof(cpx<T>) * (size_t)a.N;
+  void (*k)(LineArgs<T>) = nullptr;
+  if constexpr (sizeof(T) == 4)
+    k = m.R == 4 ? k_line<T, INV, S, 4, 1> : (m.NB == 1 ? k_line<T, INV, S, 8, 1> : k_line<T, INV, S, 8, 2>);
+  else
+    k = m.NB == 1 ? k_line<T, INV, S, 4, 1> : k_line<T, INV, S, 4, 4>;
+  GPN_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k<<<dim3(S, (unsigned)CR), m.N / (m.R * m.NB), smem, st>>>(a);
 }
 
 template <typename T, bool INV>
@@ -515,14 +548,17 @@ void line_run(Plan& plan, int R, cudaStream_t st) {
   a.out = (cpx<T>*)(INV ? plan.grid_out : plan.line_spec);
   a.tw = (const cpx<T>*)plan.line_tw;
   a.ptw = (const cpx<T>*)plan.line_ptw[si];
-  a.m = line_passes(a.h / S);
+  const LinePlan m = line_passes(a.h / S, plan.precision);
+  a.N = m.N;
+  a.r0 = m.r0;
+  a.np = m.np;
   a.lo = plan.line_lo / 2;
   a.hi = (plan.line_hi + 1) / 2;
   switch (S) {
-    case 1: line_launch<T, INV, 1>(a, CR, st); break;
-    case 2: line_launch<T, INV, 2>(a, CR, st); break;
-    case 4: line_launch<T, INV, 4>(a, CR, st); break;
-    default: line_launch<T, INV, 8>(a, CR, st);
+    case 1: line_launch<T, INV, 1>(a, m, CR, st); break;
+    case 2: line_launch<T, INV, 2>(a, m, CR, st); break;
+    case 4: line_launch<T, INV, 4>(a, m, CR, st); break;
+    default: line_launch<T, INV, 8>(a, m, CR, st);
   }
   GPN_CUDA(cudaGetLastError());
 }
@@ -537,9 +573,8 @@ void line_diag_impl(Plan& plan, int R, cudaStream_t st) {
   a.h = (int)(plan.geom.nf / 2);
   a.M = (int)plan.geom.M;
   a.C = plan.geom.C;
-  a.R = R;
   const size_t smem = 2 * sizeof(cpx<T>) * kDiagK * a.C;
-  k_line_diag<T><<<(unsigned)(a.h / 2 / kDiagK + 1), dim3(kDiagK, a.C), smem, st>>>(a);
+  k_line_diag<T><<<dim3((unsigned)(a.h / 2 / kDiagK + 1), (unsigned)R), dim3(kDiagK, a.C), smem, st>>>(a);
   GPN_CUDA(cudaGetLastError());
 }
 
@@ -556,24 +591,23 @@ void* upload(Plan& plan, const std::vector<double>& v) {
 // Plans whose transforms run here: nf = 2^a whose eighth fits a block.  `pitch`: complex
 // values per channel of the buffer the spectra can live in.
 bool line_supported(int d, long long nf, int precision, long long pitch) {
-  if (d != 1 || nf < 16 || (nf & (nf - 1)) || nf / 2 > pitch || precision == GP_DF64) return false;
-  return nf / 2 / kMaxSplit <= (1 << 20) && passes_fit((int)std::max<long long>(2, nf / 2 / kMaxSplit), precision);
+  if (d != 1 || nf < 64 || (nf & (nf - 1)) || nf / 2 > pitch || precision == GP_DF64) return false;
+  return nf / 2 / kMaxSplit <= (1 << 20) && passes_fit((int)(nf / 2 / kMaxSplit), precision);
 }
 
-// the cell groups the points reach (every 1-D plan spreads with k_spread1d)
+// where each cell's points start (every 1-D plan spreads with k_spread1d)
 void line_points_setup(Plan& plan, cudaStream_t st) {
   const PointSet& ps = plan.pts;
-  const int n = (int)ps.n, W = plan.geom.width;
+  const int n = (int)ps.n, cells = (int)plan.geom.nf;
   int first = 0, last = 0;
   GPN_CUDA(cudaMemcpyAsync(&first, ps.cell0[0], sizeof(int), cudaMemcpyDeviceToHost, st));
   GPN_CUDA(cudaMemcpyAsync(&last, ps.cell0[0] + n - 1, sizeof(int), cudaMemcpyDeviceToHost, st));
-  const int groups = (int)((plan.geom.nf + kCells - 1) / kCells);
-  plan.line_start = (int*)plan.alloc(sizeof(int) * 2 * groups);
-  k_line_start<<<blocks_for(2 * groups, 256), 256, 0, st>>>(ps.cell0[0], n, W, groups, plan.line_start);
+  plan.line_start = (int*)plan.alloc(sizeof(int) * ((size_t)cells + 1));
+  k_line_start<<<blocks_for(cells + 1, 256), 256, 0, st>>>(ps.cell0[0], n, cells, plan.line_start);
   GPN_CUDA(cudaGetLastError());
   GPN_CUDA(cudaStreamSynchronize(st));
-  plan.line_group0 = first / kCells;
-  plan.line_groups = (last + W - 1) / kCells - plan.line_group0 + 1;
+  plan.line_cell0 = first;
+  plan.line_cell1 = last + plan.geom.width;   // at most nf: no support leaves the grid
 }
 
 // twiddles, pass tables of every split, and the cells the transforms read and write (the
@@ -597,8 +631,8 @@ void line_setup(Plan& plan, void* spec) {
   plan.line_tw = f32 ? upload<float>(plan, tw) : upload<double>(plan, tw);
   for (int si = 0; si < 4; ++si) {
     const int n = (int)(h.nf / 2) >> si;
-    if (n < 2 || !passes_fit(n, plan.precision)) continue;
-    const std::vector<double> t = fft::mixed_tables(line_passes(n));
+    if (n < 4 || !passes_fit(n, plan.precision)) continue;
+    const std::vector<double> t = line_tables(line_passes(n, plan.precision));
     plan.line_ptw[si] = f32 ? upload<float>(plan, t) : upload<double>(plan, t);
   }
 }
@@ -624,19 +658,19 @@ void line_diag(Plan& plan, int R, cudaStream_t st) {
     line_diag_impl<double>(plan, R, st);
 }
 
-void launch_spread1d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st) {
+void launch_spread1d(Plan& plan, const double* alpha, const int* perm, int R, cudaStream_t st) {
   if (plan.precision == GP_FP32)
-    spread_impl<float>(plan, alpha_sorted, R, st);
+    spread_impl<float>(plan, alpha, perm, R, st);
   else
-    spread_impl<double>(plan, alpha_sorted, R, st);
+    spread_impl<double>(plan, alpha, perm, R, st);
 }
 
-void launch_interp1d(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
+void launch_interp1d(Plan& plan, const PointSet& ps, const double* alpha, double shift, double* out, const int* perm,
                      int R, cudaStream_t st) {
   if (plan.precision == GP_FP32)
-    interp_impl<float>(plan, ps, alpha_sorted, shift, out_sorted, R, st);
+    interp_impl<float>(plan, ps, alpha, shift, out, perm, R, st);
   else
-    interp_impl<double>(plan, ps, alpha_sorted, shift, out_sorted, R, st);
+    interp_impl<double>(plan, ps, alpha, shift, out, perm, R, st);
 }
 
 }  // namespace gpn

@@ -252,7 +252,9 @@ void PhaseProfile::destroy() {
 
 namespace {
 // steps (1)-(5) for R <= grid_rhs right-hand sides (one pass through the grids)
-void matvec_block(Plan& plan, const double* alpha_sorted, double* out_sorted, int R, double shift, cudaStream_t st) {
+// (perm: 1-D plans without a near field, alpha and out in the caller's order)
+void matvec_block(Plan& plan, const double* alpha_sorted, double* out_sorted, const int* perm, int R, double shift,
+                  cudaStream_t st) {
   PhaseProfile& pf = plan.prof;
   const bool rec = pf.on;
   if (rec) {
@@ -265,7 +267,10 @@ void matvec_block(Plan& plan, const double* alpha_sorted, double* out_sorted, in
     GPN_CUDA(cudaEventRecord(pf.ev[0], st));
     pf.in_matvec = true;
   }
-  launch_spread(plan, alpha_sorted, R, st);
+  if (perm)
+    launch_spread1d(plan, alpha_sorted, perm, R, st);
+  else
+    launch_spread(plan, alpha_sorted, R, st);
   if (rec) GPN_CUDA(cudaEventRecord(pf.ev[1], st));
   run_fft_forward(plan, R, st);
   if (rec) GPN_CUDA(cudaEventRecord(pf.ev[2], st));
@@ -273,8 +278,12 @@ void matvec_block(Plan& plan, const double* alpha_sorted, double* out_sorted, in
   if (rec) GPN_CUDA(cudaEventRecord(pf.ev[3], st));
   run_fft_inverse(plan, R, st);
   if (rec) GPN_CUDA(cudaEventRecord(pf.ev[4], st));
-  launch_interp(plan, plan.pts, alpha_sorted, shift, out_sorted, R, st);
-  launch_near_apply(plan, alpha_sorted, out_sorted, R, st);
+  if (perm) {
+    launch_interp1d(plan, plan.pts, alpha_sorted, shift, out_sorted, perm, R, st);
+  } else {
+    launch_interp(plan, plan.pts, alpha_sorted, shift, out_sorted, R, st);
+    launch_near_apply(plan, alpha_sorted, out_sorted, R, st);
+  }
   if (rec) {
     pf.in_matvec = false;
     GPN_CUDA(cudaEventRecord(pf.ev[5], st));
@@ -285,12 +294,25 @@ void matvec_block(Plan& plan, const double* alpha_sorted, double* out_sorted, in
 
 // Columns beyond the grids' rhs_block run in blocks, one after the other on the stream
 // (each block is one recorded pass when the phases are profiled).
-void matvec_sorted(Plan& plan, const double* alpha_sorted, double* out_sorted, int R, double shift, cudaStream_t st) {
+static void matvec_blocks(Plan& plan, const double* alpha, double* out, const int* perm, int R, double shift,
+                          cudaStream_t st) {
   const size_t n = (size_t)plan.N;
   for (int r0 = 0; r0 < R; r0 += plan.grid_rhs) {
     const int rc = std::min(plan.grid_rhs, R - r0);
-    matvec_block(plan, alpha_sorted + (size_t)r0 * n, out_sorted + (size_t)r0 * n, rc, shift, st);
+    matvec_block(plan, alpha + (size_t)r0 * n, out + (size_t)r0 * n, perm, rc, shift, st);
   }
+}
+
+void matvec_sorted(Plan& plan, const double* alpha_sorted, double* out_sorted, int R, double shift, cudaStream_t st) {
+  matvec_blocks(plan, alpha_sorted, out_sorted, nullptr, R, shift, st);
+}
+
+// 1-D plans read and write the caller's order themselves: two launches of nine fewer.
+void matvec_caller(Plan& plan, const double* alpha, double* out, int R, double shift, cudaStream_t st) {
+  if (plan.line_start && plan.near_nnz == 0) return matvec_blocks(plan, alpha, out, plan.pts.perm, R, shift, st);
+  gather_sorted(plan.pts, alpha, plan.vec_a, R, st);
+  matvec_sorted(plan, plan.vec_a, plan.vec_b, R, shift, st);
+  scatter_sorted(plan.pts, plan.vec_b, out, R, st);
 }
 
 double time_matvecs(Plan& plan, cudaStream_t st) {

@@ -183,9 +183,9 @@ struct Plan {
   bool tr3 = false;
   Box3 box3;                            // d = 3 over the occupied box
   GridView view;                        // layout of grid and grid_out
-  // d = 1 (line1d.cu): cell groups the points reach, and the split transforms
-  int* line_start = nullptr;            // per group of 32 cells: the run of points reaching it
-  int line_group0 = 0, line_groups = 0;
+  // d = 1 (line1d.cu): where each cell's points start, and the split transforms
+  int* line_start = nullptr;            // first sorted point with l0 >= c, c = 0..nf
+  int line_cell0 = 0, line_cell1 = 0;   // cells the points reach
   bool line = false;
   void* line_spec = nullptr;            // [r][C][nf/2] complex
   void* line_tw = nullptr;              // exp(-2 pi i k / nf)
@@ -349,12 +349,16 @@ void line_setup(Plan& plan, void* spec);
 void line_forward(Plan& plan, int R, cudaStream_t st);
 void line_diag(Plan& plan, int R, cudaStream_t st);
 void line_inverse(Plan& plan, int R, cudaStream_t st);
-void launch_spread1d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st);
-void launch_interp1d(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
+// (perm: alpha and out are in the caller's order; null: in sorted order)
+void launch_spread1d(Plan& plan, const double* alpha, const int* perm, int R, cudaStream_t st);
+void launch_interp1d(Plan& plan, const PointSet& ps, const double* alpha, double shift, double* out, const int* perm,
                      int R, cudaStream_t st);
 
 // Full matvec in sorted order: out = (K~ + shift I) alpha.
 void matvec_sorted(Plan& plan, const double* alpha_sorted, double* out_sorted, int R, double shift, cudaStream_t st);
+// The same in the caller's order (vec_a and vec_b hold the sorted vectors where the kernels
+// need them).
+void matvec_caller(Plan& plan, const double* alpha, double* out, int R, double shift, cudaStream_t st);
 // Milliseconds per matvec (R = 1, CUDA events, after two untimed ones) on a fixed input.
 double time_matvecs(Plan& plan, cudaStream_t st);
 

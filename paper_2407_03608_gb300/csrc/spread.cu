@@ -398,7 +398,7 @@ size_t spread_smem_bytes(int d, int tile, int C, size_t rs, int width) {
 
 void launch_spread(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st) {
   if (plan.sp2_tiles) return launch_spread2d(plan, alpha_sorted, R, st);
-  if (plan.line_start) return launch_spread1d(plan, alpha_sorted, R, st);
+  if (plan.line_start) return launch_spread1d(plan, alpha_sorted, nullptr, R, st);
   if (plan.sp3_tiles) return launch_spread3d(plan, alpha_sorted, R, st);
   const GridGeom& g = plan.geom;
   if (g.d == 1 && plan.precision == GP_FP64 && plan.n_active_tiles < 152) {
