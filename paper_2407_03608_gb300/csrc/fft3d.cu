@@ -9,10 +9,13 @@
 // of all channels is contiguous, so a transform along any axis runs over adjacent columns,
 // and the x transform takes two real channels as one complex sequence.
 //   grid  [r][z][y][x][Cp]     box cells (real), Cp = C rounded up to even
-//   X1    [r][z][y][q]         after the x transform, q = m_x C + k, pitch Qp
+//   X1    [r][z][y][q]         after the x transform, q = m_x Cs + k, pitch Qp
 //   X2    [r][z][n_y + M][q]   after y
 //   X3    [r][n_z + M][n_y + M][q]   after z: the mode box step 3 works on in place
-// and the same arrays backwards.  X1 and X3 share one buffer, X2 is the other.
+// and the same arrays backwards.  X1 and X3 share one buffer, X2 is the other.  The spectra
+// are made of 16-byte elements: one complex float64 value, or in FP32 those of two adjacent
+// channels, {re, re, im, im} (Cs = C rounded up to even), which the passes transform with
+// packed instructions (fft_mixed.h).
 //
 // Each block transforms B adjacent columns through shared memory, [n][b] with b fastest,
 // with the mixed-radix passes of fft_mixed.h: the first pass reads its inputs straight from
@@ -20,6 +23,8 @@
 // through shared memory twice.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "fft_mixed.h"
@@ -29,33 +34,45 @@ namespace gpn {
 
 namespace {
 
-using fft::cpx;
+using fft::cv;
+using fft::f2;
 using fft::MixedPlan;
+using fft::Span;
+using fft::vset;
 
-// threads of a transform block: two blocks an SM keep 64 registers a thread in FP32 (16
-// values in flight) and 128 in float64
-template <typename T>
-constexpr int kBoxThreads = sizeof(T) == 4 ? 512 : 256;
+// threads of a transform block: two blocks an SM keep 64 registers a thread (up to 10 elements
+// of four words in flight)
+constexpr int kBoxThreads = 512;
 
+// the element type of a plan's arithmetic, and the values it holds
 template <typename T>
-struct alignas(2 * sizeof(T)) RawC {
-  T x, y;
-};
+using VecOf = typename std::conditional<sizeof(T) == 4, f2, double>::type;
 template <typename T>
-__device__ __forceinline__ cpx<T> load_c(const cpx<T>* p) {
-  const RawC<T> v = *reinterpret_cast<const RawC<T>*>(p);
-  return {v.x, v.y};
+constexpr int kLanes = fft::Elem<VecOf<T>>::lanes;
+
+template <typename V>
+__device__ __forceinline__ cv<V> load_v(const cv<V>* p) {
+  const float4 u = *reinterpret_cast<const float4*>(p);
+  cv<V> v;
+  memcpy(&v, &u, 16);
+  return v;
 }
-template <typename T>
-__device__ __forceinline__ void store_c(cpx<T>* p, cpx<T> v) {
-  *reinterpret_cast<RawC<T>*>(p) = RawC<T>{v.x, v.y};
+template <typename V>
+__device__ __forceinline__ void store_v(cv<V>* p, cv<V> v) {
+  float4 u;
+  memcpy(&u, &v, 16);
+  *reinterpret_cast<float4*>(p) = u;
+}
+template <typename V>
+__device__ __forceinline__ cv<V> zero_v() {
+  return {vset<V>(0), vset<V>(0)};
 }
 
-template <typename T>
+template <typename V>
 struct BoxColsArgs {
-  const cpx<T>* in;
-  cpx<T>* out;
-  const cpx<T>* tw;
+  const cv<V>* in;
+  cv<V>* out;
+  const cv<V>* tw;
   MixedPlan m;
   int B;                                  // columns a block
   int lo, ext, M;                         // box window along the axis, modes
@@ -65,40 +82,41 @@ struct BoxColsArgs {
 
 // Transforms along y and z.  Forward: box cells [lo, lo + ext) to the modes -M..M; inverse
 // back.  blockIdx = (column group, outer index, right-hand side).
-template <typename T, bool INV>
-__global__ void __launch_bounds__(kBoxThreads<T>, 2) k_box_cols(BoxColsArgs<T> a) {
+template <typename V, bool INV>
+__global__ void __launch_bounds__(kBoxThreads, 2) k_box_cols(BoxColsArgs<V> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<T>* s = reinterpret_cast<cpx<T>*>(smem_raw);
-  const int B = a.B, b = threadIdx.x % B, jl = threadIdx.x / B, N = a.m.N, J = a.m.J, M = a.M;
+  const int B = a.B, jl = threadIdx.x / B, b = threadIdx.x - jl * B, N = a.m.N, J = a.m.J, M = a.M;
   const long long col = blockIdx.x * (long long)B + b;
-  const cpx<T>* src = a.in + blockIdx.z * a.in_r + blockIdx.y * a.in_o + col;
-  cpx<T>* dst = a.out + blockIdx.z * a.out_r + blockIdx.y * a.out_o + col;
-  cpx<T>* sb = s + b;
+  const cv<V>* src = a.in + blockIdx.z * a.in_r + blockIdx.y * a.in_o + col;
+  cv<V>* dst = a.out + blockIdx.z * a.out_r + blockIdx.y * a.out_o + col;
+  cv<V>* sb = reinterpret_cast<cv<V>*>(smem_raw) + b;
   // element n of the sequence: its place along the axis in the window or mode array, or -1
   auto window = [&](int n) { return (unsigned)(n - a.lo) < (unsigned)a.ext ? n - a.lo : -1; };
   auto mode = [&](int n) { return n <= M ? n + M : (n >= N - M ? n - N + M : -1); };
   const long long in_s = a.in_s, out_s = a.out_s;
-  fft::mixed_pass_any<INV, false, T>(
-      a.m.R[0], N, J, 1, jl, a.tw,
+  const auto from_smem = [&](int n) { return load_v(sb + n * B); };
+  const auto to_smem = [&](int n, cv<V> v) { store_v(sb + n * B, v); };
+  fft::mixed_pass_any<INV, false, V>(
+      a.m.R[0], N, J, jl, Span<V>{1, 0, a.tw},
       [&](int n) {
         const int i = INV ? mode(n) : window(n);
-        return i >= 0 ? load_c(src + i * in_s) : cpx<T>{T(0), T(0)};
+        return i >= 0 ? load_v(src + i * in_s) : zero_v<V>();
       },
-      [&](int n, cpx<T> v) { store_c(sb + n * B, v); }, [] {});
+      to_smem, [] {});
   __syncthreads();
   int ns = a.m.R[0];
   for (int p = 1; p + 1 < a.m.np; ++p) {
-    fft::mixed_pass_any<INV, true, T>(
-        a.m.R[p], N, J, ns, jl, a.tw + a.m.tw[p], [&](int n) { return load_c(sb + n * B); },
-        [&](int n, cpx<T> v) { store_c(sb + n * B, v); }, [] { __syncthreads(); });
+    fft::mixed_pass_any<INV, true, V>(a.m.R[p], N, J, jl, Span<V>{ns, a.m.inv_ns[p], a.tw + a.m.tw[p]}, from_smem,
+                                      to_smem, [] { __syncthreads(); });
     __syncthreads();
     ns *= a.m.R[p];
   }
-  fft::mixed_pass_any<INV, false, T>(
-      a.m.R[a.m.np - 1], N, J, ns, jl, a.tw + a.m.tw[a.m.np - 1], [&](int n) { return load_c(sb + n * B); },
-      [&](int n, cpx<T> v) {
+  const int p = a.m.np - 1;
+  fft::mixed_pass_any<INV, false, V>(
+      a.m.R[p], N, J, jl, Span<V>{ns, a.m.inv_ns[p], a.tw + a.m.tw[p]}, from_smem,
+      [&](int n, cv<V> v) {
         const int i = INV ? window(n) : mode(n);
-        if (i >= 0) store_c(dst + i * out_s, v);
+        if (i >= 0) store_v(dst + i * out_s, v);
       },
       [] {});
 }
@@ -106,106 +124,132 @@ __global__ void __launch_bounds__(kBoxThreads<T>, 2) k_box_cols(BoxColsArgs<T> a
 template <typename T>
 struct BoxRowsArgs {
   T* grid;                // box cells [row][x][Cp]
-  cpx<T>* X;              // [row][q]
-  const cpx<T>* tw;
+  cv<VecOf<T>>* X;        // [row][q / lanes]
+  const cv<VecOf<T>>* tw;
   MixedPlan m;
-  int YB, PB;             // rows and channel pairs a block
+  int YB, PB;             // rows and channel groups a block
   int pitch;              // shared-memory elements per sequence element
   int lo, ext, M;
-  int C, Cp;
-  long long Qp;
-  long long nrows;        // R E_0 E_1
+  int Cp;                 // channel pitch of the grid
+  int Ce;                 // elements per mode of X (Cs / lanes)
+  long long Qe;           // elements per row of X
+  long long nrows;        // E_0 E_1
 };
 
-// Transforms along x.  A sequence is the pair of channels (2p, 2p + 1) of one row as real and
-// imaginary part; its transform Z gives X_2p[m] = (Z[m] + conj Z[N-m]) / 2 and
-// X_2p+1[m] = (Z[m] - conj Z[N-m]) / 2i.  blockIdx = (row group, pair group).
+// the channels of group p at a cell: 2 lanes of them, the first half as real parts, the second
+// (zero past the pitch) as imaginary parts
 template <typename T>
-__global__ void __launch_bounds__(kBoxThreads<T>, 2) k_box_rows_fwd(BoxRowsArgs<T> a) {
+__device__ __forceinline__ cv<VecOf<T>> load_group(const T* cell, int p, int Cp) {
+  using V = VecOf<T>;
+  constexpr int L = kLanes<T>;
+  const V* c = reinterpret_cast<const V*>(cell) + 2 * p;
+  return {c[0], (2 * p + 1) * L < Cp ? c[1] : vset<V>(0)};
+}
+template <typename T>
+__device__ __forceinline__ void store_group(T* cell, int p, int Cp, cv<VecOf<T>> v) {
+  using V = VecOf<T>;
+  constexpr int L = kLanes<T>;
+  V* c = reinterpret_cast<V*>(cell) + 2 * p;
+  c[0] = v.x;
+  if ((2 * p + 1) * L < Cp) c[1] = v.y;
+}
+
+// Transforms along x.  A sequence takes channel group p of one row: with lanes L, channels
+// 2 L p .. as real parts and the L after them as imaginary parts, so that one complex transform
+// Z serves 2 L real rows: X_a[m] = (Z[m] + conj Z[N-m]) / 2 for the first channels and
+// X_b[m] = (Z[m] - conj Z[N-m]) / 2i for the second.  blockIdx = (row group, channel groups).
+template <typename T>
+__global__ void __launch_bounds__(kBoxThreads, 2) k_box_rows_fwd(BoxRowsArgs<T> a) {
+  using V = VecOf<T>;
+  constexpr int L = kLanes<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<T>* s = reinterpret_cast<cpx<T>*>(smem_raw);
-  const int PB = a.PB, B = a.YB * PB, b = threadIdx.x % B, jl = threadIdx.x / B;
-  const int N = a.m.N, J = a.m.J, M = a.M, P = a.Cp / 2;
+  cv<V>* s = reinterpret_cast<cv<V>*>(smem_raw);
+  const int PB = a.PB, B = a.YB * PB, jl = threadIdx.x / B, b = threadIdx.x - jl * B;
+  const int N = a.m.N, J = a.m.J, M = a.M, Cp = a.Cp, pitch = a.pitch;
   const int yb = b / PB, p = blockIdx.y * PB + (b - yb * PB);
   const long long row = blockIdx.x * (long long)a.YB + yb;
-  const bool valid = row < a.nrows && p < P;
-  const cpx<T>* src = reinterpret_cast<const cpx<T>*>(a.grid) + (valid ? row : 0) * (long long)a.ext * P + p;
-  cpx<T>* sb = s + b;
-  const int pitch = a.pitch;
-  fft::mixed_pass_any<false, false, T>(
-      a.m.R[0], N, J, 1, jl, a.tw,
+  const bool valid = row < a.nrows && 2 * p * L < Cp;
+  const T* src = a.grid + (valid ? row : 0) * (long long)a.ext * Cp;
+  cv<V>* sb = s + b;
+  const auto from_smem = [&](int n) { return load_v(sb + n * pitch); };
+  const auto to_smem = [&](int n, cv<V> v) { store_v(sb + n * pitch, v); };
+  fft::mixed_pass_any<false, false, V>(
+      a.m.R[0], N, J, jl, Span<V>{1, 0, a.tw},
       [&](int n) {
         const int i = n - a.lo;
-        return valid && (unsigned)i < (unsigned)a.ext ? load_c(src + (long long)i * P) : cpx<T>{T(0), T(0)};
+        return valid && (unsigned)i < (unsigned)a.ext ? load_group(src + i * Cp, p, Cp) : zero_v<V>();
       },
-      [&](int n, cpx<T> v) { store_c(sb + n * pitch, v); }, [] {});
+      to_smem, [] {});
   __syncthreads();
   int ns = a.m.R[0];
   for (int q = 1; q < a.m.np; ++q) {
-    fft::mixed_pass_any<false, true, T>(
-        a.m.R[q], N, J, ns, jl, a.tw + a.m.tw[q], [&](int n) { return load_c(sb + n * pitch); },
-        [&](int n, cpx<T> v) { store_c(sb + n * pitch, v); }, [] { __syncthreads(); });
+    fft::mixed_pass_any<false, true, V>(a.m.R[q], N, J, jl, Span<V>{ns, a.m.inv_ns[q], a.tw + a.m.tw[q]}, from_smem,
+                                        to_smem, [] { __syncthreads(); });
     __syncthreads();
     ns *= a.m.R[q];
   }
-  // the two channels of every (row, mode, pair), pairs fastest: adjacent in X
-  const int pc = threadIdx.x % PB, m0 = threadIdx.x / PB, mstep = blockDim.x / PB;
-  const int k = 2 * (blockIdx.y * PB + pc);
-  if (k >= a.C || m0 >= mstep) return;
+  // the two elements of every (row, mode, group), groups fastest: adjacent in X
+  const int m0 = threadIdx.x / PB, pc = threadIdx.x - m0 * PB, mstep = blockDim.x / PB;
+  const int e = 2 * (blockIdx.y * PB + pc);
+  if (e >= a.Ce || m0 >= mstep) return;
+  const V half = vset<V>(T(0.5));
   for (int y = 0; y < a.YB; ++y) {
     const long long r = blockIdx.x * (long long)a.YB + y;
     if (r >= a.nrows) break;
-    cpx<T>* dst = a.X + r * a.Qp + k;
-    const cpx<T>* sy = s + y * PB + pc;
+    cv<V>* dst = a.X + r * a.Qe + e;
+    const cv<V>* sy = s + y * PB + pc;
     for (int m = m0; m <= M; m += mstep) {
-      const cpx<T> z = load_c(sy + m * pitch), w = load_c(sy + (m == 0 ? 0 : N - m) * pitch);
-      cpx<T>* o = dst + (long long)m * a.C;
-      store_c(o, {T(0.5) * (z.x + w.x), T(0.5) * (z.y - w.y)});
-      if (k + 1 < a.C) store_c(o + 1, {T(0.5) * (z.y + w.y), T(0.5) * (w.x - z.x)});
+      const cv<V> z = load_v(sy + m * pitch), w = load_v(sy + (m == 0 ? 0 : N - m) * pitch);
+      cv<V>* o = dst + m * a.Ce;
+      store_v(o, {fft::vmul(half, fft::vadd(z.x, w.x)), fft::vmul(half, fft::vsub(z.y, w.y))});
+      if (e + 1 < a.Ce) store_v(o + 1, {fft::vmul(half, fft::vadd(z.y, w.y)), fft::vmul(half, fft::vsub(w.x, z.x))});
     }
   }
 }
 
-// The inverse: Z[m] = X_2p[m] + i X_2p+1[m], Z[N-m] = conj(X_2p[m]) + i conj(X_2p+1[m]) (the
-// imaginary part of mode 0 is dropped, as a C2R transform does), zero elsewhere.
+// The inverse: Z[m] = X_a[m] + i X_b[m], Z[N-m] = conj(X_a[m]) + i conj(X_b[m]) (the imaginary
+// part of mode 0 is dropped, as a C2R transform does), zero elsewhere.
 template <typename T>
-__global__ void __launch_bounds__(kBoxThreads<T>, 2) k_box_rows_inv(BoxRowsArgs<T> a) {
+__global__ void __launch_bounds__(kBoxThreads, 2) k_box_rows_inv(BoxRowsArgs<T> a) {
+  using V = VecOf<T>;
+  constexpr int L = kLanes<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<T>* s = reinterpret_cast<cpx<T>*>(smem_raw);
-  const int PB = a.PB, B = a.YB * PB, b = threadIdx.x % B, jl = threadIdx.x / B;
-  const int N = a.m.N, J = a.m.J, M = a.M, P = a.Cp / 2;
+  cv<V>* s = reinterpret_cast<cv<V>*>(smem_raw);
+  const int PB = a.PB, B = a.YB * PB, jl = threadIdx.x / B, b = threadIdx.x - jl * B;
+  const int N = a.m.N, J = a.m.J, M = a.M, Cp = a.Cp, pitch = a.pitch;
   const int yb = b / PB, p = blockIdx.y * PB + (b - yb * PB);
   const long long row = blockIdx.x * (long long)a.YB + yb;
-  const bool valid = row < a.nrows && p < P, two = 2 * p + 1 < a.C;
-  const cpx<T>* src = a.X + (valid ? row : 0) * a.Qp + 2 * p;
-  cpx<T>* dst = reinterpret_cast<cpx<T>*>(a.grid) + (valid ? row : 0) * (long long)a.ext * P + p;
-  cpx<T>* sb = s + b;
-  const int pitch = a.pitch;
-  fft::mixed_pass_any<true, false, T>(
-      a.m.R[0], N, J, 1, jl, a.tw,
+  const bool valid = row < a.nrows && 2 * p * L < Cp, two = 2 * p + 1 < a.Ce;
+  const cv<V>* src = a.X + (valid ? row : 0) * a.Qe + 2 * p;
+  T* dst = a.grid + (valid ? row : 0) * (long long)a.ext * Cp;
+  cv<V>* sb = s + b;
+  const auto from_smem = [&](int n) { return load_v(sb + n * pitch); };
+  const auto to_smem = [&](int n, cv<V> v) { store_v(sb + n * pitch, v); };
+  fft::mixed_pass_any<true, false, V>(
+      a.m.R[0], N, J, jl, Span<V>{1, 0, a.tw},
       [&](int n) {
         const bool up = n <= M, down = n >= N - M;
-        if (!valid || !(up || down)) return cpx<T>{T(0), T(0)};
-        const cpx<T>* x = src + (long long)(up ? n : N - n) * a.C;
-        const cpx<T> u = load_c(x), v = two ? load_c(x + 1) : cpx<T>{T(0), T(0)};
-        if (n == 0) return cpx<T>{u.x, v.x};
-        return up ? cpx<T>{u.x - v.y, u.y + v.x} : cpx<T>{u.x + v.y, v.x - u.y};
+        if (!valid || !(up || down)) return zero_v<V>();
+        const cv<V>* x = src + (up ? n : N - n) * a.Ce;
+        const cv<V> u = load_v(x), v = two ? load_v(x + 1) : zero_v<V>();
+        if (n == 0) return cv<V>{u.x, v.x};
+        return up ? fft::add_turn<true>(v, u) : cv<V>{fft::vadd(u.x, v.y), fft::vsub(v.x, u.y)};
       },
-      [&](int n, cpx<T> v) { store_c(sb + n * pitch, v); }, [] {});
+      to_smem, [] {});
   __syncthreads();
   int ns = a.m.R[0];
   for (int q = 1; q + 1 < a.m.np; ++q) {
-    fft::mixed_pass_any<true, true, T>(
-        a.m.R[q], N, J, ns, jl, a.tw + a.m.tw[q], [&](int n) { return load_c(sb + n * pitch); },
-        [&](int n, cpx<T> v) { store_c(sb + n * pitch, v); }, [] { __syncthreads(); });
+    fft::mixed_pass_any<true, true, V>(a.m.R[q], N, J, jl, Span<V>{ns, a.m.inv_ns[q], a.tw + a.m.tw[q]}, from_smem,
+                                       to_smem, [] { __syncthreads(); });
     __syncthreads();
     ns *= a.m.R[q];
   }
-  fft::mixed_pass_any<true, false, T>(
-      a.m.R[a.m.np - 1], N, J, ns, jl, a.tw + a.m.tw[a.m.np - 1], [&](int n) { return load_c(sb + n * pitch); },
-      [&](int n, cpx<T> v) {
+  const int q = a.m.np - 1;
+  fft::mixed_pass_any<true, false, V>(
+      a.m.R[q], N, J, jl, Span<V>{ns, a.m.inv_ns[q], a.tw + a.m.tw[q]}, from_smem,
+      [&](int n, cv<V> v) {
         const int i = n - a.lo;
-        if (valid && (unsigned)i < (unsigned)a.ext) store_c(dst + (long long)i * P, v);
+        if (valid && (unsigned)i < (unsigned)a.ext) store_group(dst + i * Cp, p, Cp, v);
       },
       [] {});
 }
@@ -227,14 +271,24 @@ constexpr int kDiagM = 64;
 
 template <typename T>
 struct BoxDiagArgs {
-  cpx<T>* X;              // [r][nz + M][ny + M][q]
+  cv<VecOf<T>>* X;        // [r][nz + M][ny + M][q / lanes]
   const T* A;             // [pair][|nz|][|ny|][m], the octant (null: lean)
   const T* tab;           // lean factors [j][m][CP]
   const T* sqv;           // sqrt(v~_j)
   long long n_freq;       // (M + 1)^3
-  long long Qp, xr;       // row pitch and right-hand-side stride of X
+  long long Qe, xr;       // row pitch and right-hand-side stride of X, in elements
   int M, C, CP, J, R;
 };
+
+// channel k of the elements at e: its real and imaginary part
+template <typename T>
+__device__ __forceinline__ T& re_of(cv<VecOf<T>>* e, int k) {
+  return reinterpret_cast<T*>(e)[kLanes<T> == 2 ? k / 2 * 4 + k % 2 : 2 * k];
+}
+template <typename T>
+__device__ __forceinline__ T& im_of(cv<VecOf<T>>* e, int k) {
+  return reinterpret_cast<T*>(e)[kLanes<T> == 2 ? k / 2 * 4 + 2 + k % 2 : 2 * k + 1];
+}
 
 // rows of the sign combinations of (|nz|, |ny|); returns their number
 __device__ __forceinline__ int sign_rows(int nz, int ny, int M, long long (&row)[4]) {
@@ -262,8 +316,9 @@ __device__ __forceinline__ void stage_factors(const BoxDiagArgs<T>& a, T* s_em, 
 template <typename T, int NC, bool LEAN>
 __global__ void __launch_bounds__(kDiagM) k_box_diag(BoxDiagArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int PITCH = NC | 1, NP = NC * (NC + 1) / 2;
-  cpx<T>* s_b = reinterpret_cast<cpx<T>*>(smem_raw);           // [4][kDiagM][PITCH]
+  using V = VecOf<T>;
+  constexpr int L = kLanes<T>, NE = (NC + L - 1) / L, PITCH = NE | 1, NP = NC * (NC + 1) / 2;
+  cv<V>* s_b = reinterpret_cast<cv<V>*>(smem_raw);             // [4][kDiagM][PITCH]
   const int ny = blockIdx.y, nz = blockIdx.z, m0 = blockIdx.x * kDiagM, t = threadIdx.x;
   const int Mp = a.M + 1, nm = min(kDiagM, Mp - m0);
   long long row[4];
@@ -307,38 +362,54 @@ __global__ void __launch_bounds__(kDiagM) k_box_diag(BoxDiagArgs<T> a) {
     for (int p = 0; p < NP; ++p) av[p] = __ldg(Am + (size_t)p * a.n_freq);
   }
   for (int r = 0; r < a.R; ++r) {
-    cpx<T>* Xr = a.X + r * a.xr + (size_t)m0 * NC;
+    cv<V>* Xr = a.X + r * a.xr + (size_t)m0 * NE;
     for (int s = 0; s < ns; ++s)
-      for (int e = t; e < nm * NC; e += kDiagM) {
-        const int f = e / NC;
-        s_b[(s * kDiagM + f) * PITCH + (e - f * NC)] = load_c(Xr + row[s] * a.Qp + e);
+      for (int e = t; e < nm * NE; e += kDiagM) {
+        const int f = e / NE;
+        store_v(s_b + (s * kDiagM + f) * PITCH + (e - f * NE), load_v(Xr + row[s] * a.Qe + e));
       }
     __syncthreads();
     if (t < nm) {
       for (int s = 0; s < ns; ++s) {
-        cpx<T>* sb = s_b + (s * kDiagM + t) * PITCH;
-        cpx<T> b[NC];
+        cv<V>* sb = s_b + (s * kDiagM + t) * PITCH;
+        T bx[NE * L], by[NE * L];
 #pragma unroll
-        for (int k = 0; k < NC; ++k) b[k] = load_c(sb + k);
+        for (int e = 0; e < NE; ++e) {
+          cv<V> v = load_v(sb + e);
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-          cpx<T> o{T(0), T(0)};
-#pragma unroll
-          for (int l = 0; l < NC; ++l) {
-            const int lo = k < l ? k : l, hi = k < l ? l : k;
-            const T w = av[lo * NC - lo * (lo - 1) / 2 + (hi - lo)];
-            o.x += w * b[l].x;
-            o.y += w * b[l].y;
+          for (int l = 0; l < L; ++l) {
+            bx[e * L + l] = re_of<T>(&v, l);
+            by[e * L + l] = im_of<T>(&v, l);
           }
-          store_c(sb + k, o);
+        }
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+          cv<V> o = zero_v<V>();
+#pragma unroll
+          for (int q = 0; q < L; ++q) {
+            const int k = e * L + q;
+            T ox = T(0), oy = T(0);
+            if (k < NC) {
+#pragma unroll
+              for (int l = 0; l < NC; ++l) {
+                const int lo = k < l ? k : l, hi = k < l ? l : k;
+                const T w = av[lo * NC - lo * (lo - 1) / 2 + (hi - lo)];
+                ox += w * bx[l];
+                oy += w * by[l];
+              }
+            }
+            re_of<T>(&o, q) = ox;
+            im_of<T>(&o, q) = oy;
+          }
+          store_v(sb + e, o);
         }
       }
     }
     __syncthreads();
     for (int s = 0; s < ns; ++s)
-      for (int e = t; e < nm * NC; e += kDiagM) {
-        const int f = e / NC;
-        store_c(Xr + row[s] * a.Qp + e, s_b[(s * kDiagM + f) * PITCH + (e - f * NC)]);
+      for (int e = t; e < nm * NE; e += kDiagM) {
+        const int f = e / NE;
+        store_v(Xr + row[s] * a.Qe + e, load_v(s_b + (s * kDiagM + f) * PITCH + (e - f * NE)));
       }
     __syncthreads();
   }
@@ -349,9 +420,11 @@ __global__ void __launch_bounds__(kDiagM) k_box_diag(BoxDiagArgs<T> a) {
 template <typename T, bool LEAN>
 __global__ void __launch_bounds__(kDiagM) k_box_diag_wide(BoxDiagArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int C = a.C, PITCH = C | 1;
-  cpx<T>* s_b = reinterpret_cast<cpx<T>*>(smem_raw);           // [kDiagM][PITCH]
-  cpx<T>* s_o = s_b + kDiagM * PITCH;                          // [kDiagM][PITCH]
+  using V = VecOf<T>;
+  constexpr int L = kLanes<T>;
+  const int C = a.C, E = (C + L - 1) / L, PITCH = E | 1;
+  cv<V>* s_b = reinterpret_cast<cv<V>*>(smem_raw);             // [kDiagM][PITCH]
+  cv<V>* s_o = s_b + kDiagM * PITCH;                           // [kDiagM][PITCH]
   T* s_em = reinterpret_cast<T*>(s_o + kDiagM * PITCH);        // lean: [J][CP]
   const int ny = blockIdx.y, nz = blockIdx.z, m0 = blockIdx.x * kDiagM, t = threadIdx.x;
   const int Mp = a.M + 1, nm = min(kDiagM, Mp - m0);
@@ -361,45 +434,46 @@ __global__ void __launch_bounds__(kDiagM) k_box_diag_wide(BoxDiagArgs<T> a) {
   const int m = m0 + min(t, nm - 1);
   for (int r = 0; r < a.R; ++r)
     for (int s = 0; s < ns; ++s) {
-      cpx<T>* Xs = a.X + r * a.xr + row[s] * a.Qp + (size_t)m0 * C;
-      for (int e = t; e < nm * C; e += kDiagM) s_b[e / C * PITCH + e % C] = load_c(Xs + e);
+      cv<V>* Xs = a.X + r * a.xr + row[s] * a.Qe + (size_t)m0 * E;
+      for (int e = t; e < nm * E; e += kDiagM) store_v(s_b + e / E * PITCH + e % E, load_v(Xs + e));
       __syncthreads();
-      const cpx<T>* b = s_b + t * PITCH;
-      cpx<T>* o = s_o + t * PITCH;
+      cv<V>* b = s_b + t * PITCH;
+      cv<V>* o = s_o + t * PITCH;
       if (t < nm) {
+        for (int e = 0; e < E; ++e) store_v(o + e, zero_v<V>());
         if constexpr (LEAN) {
-          for (int k = 0; k < C; ++k) store_c(o + k, {T(0), T(0)});
           for (int j = 0; j < a.J; ++j) {
             const T* tm = a.tab + ((size_t)j * Mp + m) * a.CP;
             const T* em = s_em + j * a.CP;
-            cpx<T> u{T(0), T(0)};
+            T ux = T(0), uy = T(0);
             for (int l = 0; l < C; ++l) {
               const T g = em[l] * __ldg(tm + l);
-              u.x += g * b[l].x;
-              u.y += g * b[l].y;
+              ux += g * re_of<T>(b, l);
+              uy += g * im_of<T>(b, l);
             }
             for (int k = 0; k < C; ++k) {
               const T g = em[k] * __ldg(tm + k);
-              o[k].x += g * u.x;
-              o[k].y += g * u.y;
+              re_of<T>(o, k) += g * ux;
+              im_of<T>(o, k) += g * uy;
             }
           }
         } else {
           const T* Am = a.A + ((size_t)nz * Mp + ny) * Mp + m;
           for (int k = 0; k < C; ++k) {
-            cpx<T> v{T(0), T(0)};
+            T vx = T(0), vy = T(0);
             for (int l = 0; l < C; ++l) {
               const int lo = k < l ? k : l, hi = k < l ? l : k;
               const T w = __ldg(Am + (size_t)(lo * C - lo * (lo - 1) / 2 + (hi - lo)) * a.n_freq);
-              v.x += w * b[l].x;
-              v.y += w * b[l].y;
+              vx += w * re_of<T>(b, l);
+              vy += w * im_of<T>(b, l);
             }
-            store_c(o + k, v);
+            re_of<T>(o, k) = vx;
+            im_of<T>(o, k) = vy;
           }
         }
       }
       __syncthreads();
-      for (int e = t; e < nm * C; e += kDiagM) store_c(Xs + e, s_o[e / C * PITCH + e % C]);
+      for (int e = t; e < nm * E; e += kDiagM) store_v(Xs + e, load_v(s_o + e / E * PITCH + e % E));
       __syncthreads();
     }
 }
@@ -407,12 +481,13 @@ __global__ void __launch_bounds__(kDiagM) k_box_diag_wide(BoxDiagArgs<T> a) {
 template <typename T, int NC, bool LEAN>
 void diag_launch(const BoxDiagArgs<T>& a, dim3 grid, cudaStream_t st) {
   if constexpr (NC > 12) {
-    const size_t smem = 2 * sizeof(cpx<T>) * kDiagM * (a.C | 1) + (LEAN ? sizeof(T) * a.J * a.CP : 0);
+    const int E = (a.C + kLanes<T> - 1) / kLanes<T>;
+    const size_t smem = 2 * 16 * kDiagM * (E | 1) + (LEAN ? sizeof(T) * a.J * a.CP : 0);
     GPN_CUDA(cudaFuncSetAttribute(k_box_diag_wide<T, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_box_diag_wide<T, LEAN><<<grid, kDiagM, smem, st>>>(a);
   } else if (a.C == NC) {
-    const size_t smem =
-        std::max<size_t>(4 * sizeof(cpx<T>) * kDiagM * (NC | 1), LEAN ? sizeof(T) * a.J * a.CP : 0);
+    const int E = (NC + kLanes<T> - 1) / kLanes<T>;
+    const size_t smem = std::max<size_t>(4 * 16 * kDiagM * (E | 1), LEAN ? sizeof(T) * a.J * a.CP : 0);
     GPN_CUDA(cudaFuncSetAttribute(k_box_diag<T, NC, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_box_diag<T, NC, LEAN><<<grid, kDiagM, smem, st>>>(a);
   } else {
@@ -424,12 +499,12 @@ template <typename T>
 void box_diag_impl(Plan& plan, int R, cudaStream_t st) {
   const Box3& bx = plan.box3;
   BoxDiagArgs<T> a{};
-  a.X = (cpx<T>*)bx.buf_a;
+  a.X = (cv<VecOf<T>>*)bx.buf_a;
   a.A = (const T*)plan.a_tensor;
   a.tab = (const T*)plan.lean_tab;
   a.sqv = (const T*)plan.lean_sqv;
   a.n_freq = plan.n_freq;
-  a.Qp = bx.Qp;
+  a.Qe = bx.Qe;
   a.xr = bx.size_a;
   a.M = (int)plan.geom.M;
   a.C = plan.geom.C;
@@ -446,10 +521,11 @@ void box_diag_impl(Plan& plan, int R, cudaStream_t st) {
 
 template <typename T, bool INV>
 void box_cols(Plan& plan, int axis, int R, cudaStream_t st) {
+  using V = VecOf<T>;
   const Box3& bx = plan.box3;
-  const long long W = 2 * plan.geom.M + 1, Qp = bx.Qp;
-  BoxColsArgs<T> a{};
-  a.tw = (const cpx<T>*)bx.tw;
+  const long long W = 2 * plan.geom.M + 1, Qe = bx.Qe;
+  BoxColsArgs<V> a{};
+  a.tw = (const cv<V>*)bx.tw;
   a.m = bx.fft;
   a.B = bx.cols;
   a.lo = bx.lo[axis];
@@ -459,34 +535,34 @@ void box_cols(Plan& plan, int axis, int R, cudaStream_t st) {
   // forward strides (the inverse swaps in and out): y takes buf_a [z][y][q] to buf_b
   // [z][ny][q]; z takes buf_b [z][(ny, q)] to buf_a [nz][(ny, q)]
   if (axis == 1) {
-    ncols = Qp;
+    ncols = Qe;
     outer = bx.ext[0];
-    a.in_o = (long long)bx.ext[1] * Qp;
-    a.out_o = W * Qp;
-    a.in_s = a.out_s = Qp;
-    a.in = (const cpx<T>*)bx.buf_a;
-    a.out = (cpx<T>*)bx.buf_b;
+    a.in_o = (long long)bx.ext[1] * Qe;
+    a.out_o = W * Qe;
+    a.in_s = a.out_s = Qe;
+    a.in = (const cv<V>*)bx.buf_a;
+    a.out = (cv<V>*)bx.buf_b;
     a.in_r = bx.size_a;
     a.out_r = bx.size_b;
   } else {
-    ncols = W * Qp;
+    ncols = W * Qe;
     outer = 1;
-    a.in_s = a.out_s = W * Qp;
-    a.in = (const cpx<T>*)bx.buf_b;
-    a.out = (cpx<T>*)bx.buf_a;
+    a.in_s = a.out_s = W * Qe;
+    a.in = (const cv<V>*)bx.buf_b;
+    a.out = (cv<V>*)bx.buf_a;
     a.in_r = bx.size_b;
     a.out_r = bx.size_a;
   }
   if (INV) {
-    const cpx<T>* in = a.in;
+    const cv<V>* in = a.in;
     a.in = a.out;
-    a.out = const_cast<cpx<T>*>(in);
+    a.out = const_cast<cv<V>*>(in);
     std::swap(a.in_o, a.out_o);
     std::swap(a.in_r, a.out_r);
   }
-  const size_t smem = sizeof(cpx<T>) * (size_t)a.m.N * a.B;
-  GPN_CUDA(cudaFuncSetAttribute(k_box_cols<T, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_box_cols<T, INV><<<dim3((unsigned)(ncols / a.B), (unsigned)outer, (unsigned)R), a.m.J * a.B, smem, st>>>(a);
+  const size_t smem = 16 * (size_t)a.m.N * a.B;
+  GPN_CUDA(cudaFuncSetAttribute(k_box_cols<V, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_box_cols<V, INV><<<dim3((unsigned)(ncols / a.B), (unsigned)outer, (unsigned)R), a.m.J * a.B, smem, st>>>(a);
   GPN_CUDA(cudaGetLastError());
 }
 
@@ -494,27 +570,28 @@ template <typename T, bool INV>
 void box_rows(Plan& plan, int R, cudaStream_t st) {
   const Box3& bx = plan.box3;
   BoxRowsArgs<T> a{};
-  a.tw = (const cpx<T>*)bx.tw;
+  a.tw = (const cv<VecOf<T>>*)bx.tw;
   a.m = bx.fft;
   a.YB = bx.rows;
-  a.PB = bx.pairs;
+  a.PB = bx.groups;
   const int B = a.YB * a.PB;
-  // an odd multiple of the pair group: the mode-by-mode reads of the split spread over the banks
+  // an odd multiple of the channel groups: the mode-by-mode reads of the split spread over the banks
   a.pitch = a.YB % 2 ? B : B + a.PB;
   a.lo = bx.lo[2];
   a.ext = bx.ext[2];
   a.M = (int)plan.geom.M;
-  a.C = plan.geom.C;
   a.Cp = bx.Cp;
-  a.Qp = bx.Qp;
+  a.Ce = (plan.geom.C + kLanes<T> - 1) / kLanes<T>;
+  a.Qe = bx.Qe;
   a.nrows = (long long)bx.ext[0] * bx.ext[1];
-  const size_t smem = sizeof(cpx<T>) * (size_t)a.m.N * a.pitch;
+  const size_t smem = 16 * (size_t)a.m.N * a.pitch;
   void (*k)(BoxRowsArgs<T>) = INV ? k_box_rows_inv<T> : k_box_rows_fwd<T>;
   GPN_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const dim3 grid((unsigned)((a.nrows + a.YB - 1) / a.YB), (unsigned)((bx.Cp / 2 + a.PB - 1) / a.PB));
+  const int ngroups = (bx.Cp + 2 * kLanes<T> - 1) / (2 * kLanes<T>);
+  const dim3 grid((unsigned)((a.nrows + a.YB - 1) / a.YB), (unsigned)((ngroups + a.PB - 1) / a.PB));
   for (int r = 0; r < R; ++r) {
     a.grid = (T*)(INV ? plan.grid_out : plan.grid) + (size_t)r * plan.view.rstride;
-    a.X = (cpx<T>*)bx.buf_a + (size_t)r * bx.size_a;
+    a.X = (cv<VecOf<T>>*)bx.buf_a + (size_t)r * bx.size_a;
     k<<<grid, a.m.J * B, smem, st>>>(a);
   }
   GPN_CUDA(cudaGetLastError());
@@ -553,23 +630,25 @@ void box3_setup(Plan& plan) {
   }
   const bool f32 = plan.precision == GP_FP32;
   bx.Cp = (C + 1) / 2 * 2;
-  bx.Qp = ((h.M + 1) * C + 15) / 16 * 16;
+  const int lanes = f32 ? 2 : 1;
+  bx.Qe = ((h.M + 1) * ((C + lanes - 1) / lanes) + 7) / 8 * 8;
   bx.fft = fft::mixed_plan((int)h.nf);
-  const int tmax = f32 ? kBoxThreads<float> : kBoxThreads<double>, J = bx.fft.J;
-  bx.cols = f32 ? 16 : 8;                     // 128-byte segments of adjacent columns
-  while (bx.cols > 1 && bx.cols * J > tmax) bx.cols /= 2;
-  bx.pairs = std::max(1, std::min(bx.Cp / 2, tmax / J));
-  bx.rows = std::max(1, std::min((f32 ? 16 : 8) / bx.pairs, tmax / (J * bx.pairs)));
+  const int J = bx.fft.J, groups = (bx.Cp + 2 * lanes - 1) / (2 * lanes);
+  bx.cols = 8;                                // 128-byte segments of adjacent columns
+  while (bx.cols > 1 && bx.cols * J > kBoxThreads) bx.cols /= 2;
+  bx.groups = std::max(1, std::min(groups, kBoxThreads / J));
+  bx.rows = std::max(1, std::min(8 / bx.groups, kBoxThreads / (J * bx.groups)));
   const long long W = 2 * h.M + 1;
-  bx.size_a = std::max((long long)bx.ext[0] * bx.ext[1], W * W) * bx.Qp;
-  bx.size_b = (long long)bx.ext[0] * W * bx.Qp;
-  const size_t cs = 2 * plan.real_size;
-  bx.buf_a = plan.alloc(cs * bx.size_a * plan.grid_rhs);
-  bx.buf_b = plan.alloc(cs * bx.size_b * plan.grid_rhs);
+  bx.size_a = std::max((long long)bx.ext[0] * bx.ext[1], W * W) * bx.Qe;
+  bx.size_b = (long long)bx.ext[0] * W * bx.Qe;
+  bx.buf_a = plan.alloc(16 * bx.size_a * plan.grid_rhs);
+  bx.buf_b = plan.alloc(16 * bx.size_b * plan.grid_rhs);
   const std::vector<double> t = fft::mixed_tables(bx.fft);
-  bx.tw = plan.alloc(t.size() * plan.real_size);
+  bx.tw = plan.alloc(std::max<size_t>(t.size() / 2, 1) * 16);
   if (f32) {
-    const std::vector<float> f(t.begin(), t.end());
+    // each twiddle part twice, once per lane
+    std::vector<float> f;
+    for (double v : t) f.insert(f.end(), 2, (float)v);
     GPN_CUDA(cudaMemcpy(bx.tw, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
   } else {
     GPN_CUDA(cudaMemcpy(bx.tw, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));

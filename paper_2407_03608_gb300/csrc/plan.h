@@ -59,13 +59,13 @@ struct Box3 {
   bool on = false;
   int lo[3] = {0, 0, 0}, ext[3] = {0, 0, 0};   // box cells per axis
   int Cp = 0;                                  // channel pitch of the grids (even)
-  long long Qp = 0;                            // row pitch of the spectra ((M + 1) C, padded)
-  long long size_a = 0, size_b = 0;            // complex values per right-hand side
+  long long Qe = 0;                            // row pitch of the spectra, in 16-byte elements
+  long long size_a = 0, size_b = 0;            // elements per right-hand side
   void* buf_a = nullptr;
   void* buf_b = nullptr;
   void* tw = nullptr;
   fft::MixedPlan fft;
-  int cols = 1, rows = 1, pairs = 1;           // columns / rows and channel pairs a block
+  int cols = 1, rows = 1, groups = 1;          // columns / rows and channel groups a block
 };
 
 // Per-phase event timing of matvecs (diagnostic, off by default).

@@ -28,7 +28,7 @@ def test_mixed_radix_transform(prog, n):
     inp = "%d\n" % n + "\n".join("%.17g" % v for v in np.column_stack([z.real, z.imag]).ravel())
     out = subprocess.run([prog], input=inp, capture_output=True, text=True, check=True).stdout.split()
     passes, lanes = int(out[0]), int(out[1])
-    assert 2 <= passes <= 4 and lanes * 20 >= n
+    assert 2 <= passes <= 4 and lanes * 10 >= n
     v = np.array([float(x) for x in out[2:]]).reshape(3, n, 2)
     got = v[..., 0] + 1j * v[..., 1]
     fwd, inv = np.fft.fft(z), np.fft.ifft(z) * n
