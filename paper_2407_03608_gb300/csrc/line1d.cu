@@ -66,62 +66,84 @@ struct Spread1Args {
   long long n;
   T* grid;               // [r][k][nf]
   long long nf;
-  int width, C;
+  int width, C, R;
   T beta, inv_halfw;
 };
 
 // One thread takes one (cell, channel) pair, one block a run of `cells` cells.  The points that
 // reach the run are one contiguous run of the cell-sorted points; the block stages their kernel
-// values and w_k alpha in shared memory, kChunk points at a time, and every thread walks the
-// points that reach its own cell (again contiguous), so that every multiply-add is a needed
+// values, weights and the alpha of RB right-hand sides in shared memory, kChunk points at a
+// time, and every thread walks the points that reach its own cell (again contiguous), so that every multiply-add is a needed
 // one.  The order of the sums is the points' order (results do not depend on scheduling), and
 // every cell the points reach is written, so the grid needs no clearing.
-template <typename T>
+template <typename T, int RB>
 __global__ void __launch_bounds__(kSpreadThreads) k_spread1d(Spread1Args<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int W = a.width, C = a.C, r = blockIdx.y, tid = threadIdx.x;
+  const int W = a.width, C = a.C, r0 = blockIdx.y * RB, tid = threadIdx.x;
   T* s_wk = reinterpret_cast<T*>(smem_raw);   // [kChunk][C]
   T* s_psi = s_wk + kChunk * C;               // [kChunk][W]
-  T* s_amp = s_psi + kChunk * W;              // [kChunk]: alpha, converted once a point
-  int* s_l0 = reinterpret_cast<int*>(s_amp + kChunk);
+  T* s_amp = s_psi + kChunk * W;              // [kChunk][RB]: alpha, converted once a point
+  int* s_l0 = reinterpret_cast<int*>(s_amp + kChunk * RB);
   const int c0 = a.cell0 + blockIdx.x * a.cells, c1 = min(c0 + a.cells, a.cell1);
   const int p0 = a.start[max(0, c0 - W + 1)], p1 = a.start[c1];
   const int ci = tid / C, k = tid - ci * C, cell = c0 + ci;
   const int pi = tid / W, j = tid - pi * W, pstep = kSpreadThreads / W;
   const bool on = ci < a.cells && cell < c1;
   const int q0 = on ? a.start[max(0, cell - W + 1)] : 0, q1 = on ? a.start[cell + 1] : 0;
-  const double* alpha = a.alpha + (size_t)r * a.n;
-  T acc = T(0);
+  const double* alpha = a.alpha + (size_t)r0 * a.n;
+  T acc[RB];
+#pragma unroll
+  for (int r = 0; r < RB; ++r) acc[r] = T(0);
   for (int base = p0; base < p1; base += kChunk) {
     const int m = min(kChunk, p1 - base);
     for (int i = tid; i < m; i += kSpreadThreads) {
       s_l0[i] = a.l0[base + i];
-      s_amp[i] = (T)alpha[a.perm ? a.perm[base + i] : base + i];
+      const int q = a.perm ? a.perm[base + i] : base + i;
+#pragma unroll
+      for (int r = 0; r < RB; ++r) s_amp[i * RB + r] = r0 + r < a.R ? (T)alpha[(size_t)r * a.n + q] : T(0);
     }
     if (pi < pstep)
       for (int q = pi; q < m; q += pstep)
         s_psi[q * W + j] = a.psi ? a.psi[(size_t)(base + q) * W + j]
                                  : psi_at<T>(j, a.xi[base + q], a.beta, a.inv_halfw);
-    __syncthreads();
-    if (ci < a.cells)
-      for (int q = ci; q < m; q += a.cells) s_wk[q * C + k] = a.wk[(size_t)(base + q) * C + k] * s_amp[q];
+    for (int i = tid; i < m * C; i += kSpreadThreads) s_wk[i] = a.wk[(size_t)base * C + i];
     __syncthreads();
     const int e = min(q1 - base, m);
-    T part = T(0);   // a chunk's sum on its own: dense cells add their points in two levels
+    T part[RB];   // a chunk's sum on its own: dense cells add their points in two levels
+#pragma unroll
+    for (int r = 0; r < RB; ++r) part[r] = T(0);
 #pragma unroll 4
-    for (int q = max(q0 - base, 0); q < e; ++q) part += s_psi[q * W + (cell - s_l0[q])] * s_wk[q * C + k];
-    acc += part;
+    for (int q = max(q0 - base, 0); q < e; ++q) {
+      const T v = s_psi[q * W + (cell - s_l0[q])] * s_wk[q * C + k];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) part[r] += v * s_amp[q * RB + r];
+    }
+#pragma unroll
+    for (int r = 0; r < RB; ++r) acc[r] += part[r];
     __syncthreads();
   }
   // the run's sums leave through shared memory, cells fastest
   T* s_out = reinterpret_cast<T*>(smem_raw);
-  if (on) s_out[k * a.cells + ci] = acc;
-  __syncthreads();
   const int nc = c1 - c0;
-  for (int i = tid; i < nc * C; i += kSpreadThreads) {
-    const int kk = i / nc, c = i - kk * nc;
-    a.grid[((size_t)r * C + kk) * a.nf + c0 + c] = s_out[kk * a.cells + c];
+#pragma unroll
+  for (int r = 0; r < RB; ++r) {
+    if (r0 + r >= a.R) break;
+    if (on) s_out[k * a.cells + ci] = acc[r];
+    __syncthreads();
+    for (int i = tid; i < nc * C; i += kSpreadThreads) {
+      const int kk = i / nc, c = i - kk * nc;
+      a.grid[((size_t)(r0 + r) * C + kk) * a.nf + c0 + c] = s_out[kk * a.cells + c];
+    }
+    __syncthreads();
   }
+}
+
+template <typename T, int RB>
+void spread_launch(const Spread1Args<T>& a, int R, cudaStream_t st) {
+  const size_t smem = kChunk * ((a.C + a.width + RB) * sizeof(T) + sizeof(int));
+  GPN_CUDA(cudaFuncSetAttribute(k_spread1d<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int blocks = (a.cell1 - a.cell0 + a.cells - 1) / a.cells;
+  k_spread1d<T, RB><<<dim3((unsigned)blocks, (unsigned)((R + RB - 1) / RB)), kSpreadThreads, smem, st>>>(a);
 }
 
 template <typename T>
@@ -146,10 +168,14 @@ void spread_impl(Plan& plan, const double* alpha, const int* perm, int R, cudaSt
   a.C = g.C;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);
-  const size_t smem = kChunk * ((g.C + g.width + 1) * sizeof(T) + sizeof(int));
-  GPN_CUDA(cudaFuncSetAttribute(k_spread1d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int blocks = (a.cell1 - a.cell0 + a.cells - 1) / a.cells;
-  k_spread1d<T><<<dim3((unsigned)blocks, (unsigned)R), kSpreadThreads, smem, st>>>(a);
+  a.R = R;
+  // several right-hand sides a block share the staged points
+  if (R == 1)
+    spread_launch<T, 1>(a, R, st);
+  else if (R == 2)
+    spread_launch<T, 2>(a, R, st);
+  else
+    spread_launch<T, 4>(a, R, st);
   GPN_CUDA(cudaGetLastError());
 }
 
@@ -237,37 +263,51 @@ __global__ void __launch_bounds__(128) k_interp1d_lanes(Interp1Args<T> a) {
 }
 
 // A thread a point, NC = C channels in registers (32 with the extra ones unused): neighbouring
-// points read neighbouring cells.
+// points read neighbouring cells; the points' weights (rows of C values) come through shared
+// memory, a row a lane would touch a line each.
+constexpr int kInterpThreads = 128;
 template <typename T, int NC>
-__global__ void __launch_bounds__(128) k_interp1d(Interp1Args<T> a) {
-  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kInterpThreads) k_interp1d(Interp1Args<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* s_wk = reinterpret_cast<T*>(smem_raw);   // [kInterpThreads][C | 1]
+  const long long p0 = blockIdx.x * (long long)kInterpThreads, p = p0 + threadIdx.x;
   const int r = blockIdx.y, W = a.width, C = NC <= 16 ? NC : a.C;
-  if (p >= a.n) return;
-  const T* g = a.grid + (size_t)r * C * a.nf + a.l0[p];
-  const T x = a.xi[p];
+  const int m = (int)min((long long)kInterpThreads, a.n - p0) * C;
+  for (int i = threadIdx.x; i < m; i += kInterpThreads) {
+    const int q = i / C;
+    s_wk[q * (C | 1) + (i - q * C)] = a.wk[p0 * C + i];
+  }
+  const bool on = p < a.n;
+  const T* g = a.grid + (size_t)r * C * a.nf + (on ? a.l0[p] : 0);
+  const T x = on ? a.xi[p] : T(0);
   T acc[NC];
 #pragma unroll
   for (int k = 0; k < NC; ++k) acc[k] = T(0);
-  for (int j = 0; j < W; ++j) {
-    const T ps = a.psi ? a.psi[p * W + j] : psi_at<T>(j, x, a.beta, a.inv_halfw);
+  if (on) {
+    for (int j = 0; j < W; ++j) {
+      const T ps = a.psi ? a.psi[p * W + j] : psi_at<T>(j, x, a.beta, a.inv_halfw);
 #pragma unroll
-    for (int k = 0; k < NC; ++k)
-      if (NC <= 16 || k < C) acc[k] += ps * __ldg(g + (size_t)k * a.nf + j);
+      for (int k = 0; k < NC; ++k)
+        if (NC <= 16 || k < C) acc[k] += ps * __ldg(g + (size_t)k * a.nf + j);
+    }
   }
+  __syncthreads();
+  if (!on) return;
+  const T* w = s_wk + threadIdx.x * (C | 1);
   SumOf<T> res(0.0);
 #pragma unroll
   for (int k = 0; k < NC; ++k)
-    if (NC <= 16 || k < C) add_product(res, a.wk[p * C + k], acc[k]);
+    if (NC <= 16 || k < C) add_product(res, w[k], acc[k]);
   finish_point(a, p, r, (double)res);
 }
 
 template <typename T, int NC>
 void interp_dispatch(const Interp1Args<T>& a, dim3 grid, cudaStream_t st) {
   if constexpr (NC > 16) {
-    k_interp1d<T, 32><<<grid, 128, 0, st>>>(a);
+    k_interp1d<T, 32><<<grid, kInterpThreads, sizeof(T) * kInterpThreads * (a.C | 1), st>>>(a);
   } else {
     if (a.C == NC)
-      k_interp1d<T, NC><<<grid, 128, 0, st>>>(a);
+      k_interp1d<T, NC><<<grid, kInterpThreads, sizeof(T) * kInterpThreads * (a.C | 1), st>>>(a);
     else
       interp_dispatch<T, NC + 1>(a, grid, st);
   }
@@ -295,7 +335,7 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha, double shi
                    out};
   // a thread a point once the points fill half of the chip's threads (152 SMs x 1024)
   if (ps.n * R >= 152ll * 1024)
-    interp_dispatch<T, 1>(a, dim3((unsigned)((ps.n + 127) / 128), (unsigned)R), st);
+    interp_dispatch<T, 1>(a, dim3((unsigned)((ps.n + kInterpThreads - 1) / kInterpThreads), (unsigned)R), st);
   else
     k_interp1d_lanes<T><<<dim3((unsigned)((ps.n + 7) / 8), (unsigned)R), 128, 0, st>>>(a);
   GPN_CUDA(cudaGetLastError());
@@ -334,15 +374,27 @@ __device__ __forceinline__ cpx<T> quarter_turns(cpx<T> a, int q) {
   return q & 2 ? cpx<T>{-a.x, -a.y} : a;
 }
 
+// padded shared-memory index: the first passes store at strides of 4 and 8 elements, which would
+// fall in a few banks
+template <typename T>
+__device__ __forceinline__ int spos(int n) { return n + (n >> (sizeof(T) == 4 ? 4 : 3)); }
+
 // one Stockham pass in place, NB butterflies a thread (J threads)
 template <int R, int NB, bool INV, typename T>
 __device__ __forceinline__ void line_pass(cpx<T>* s, int N, int J, int Ns, int t, const cpx<T>* tw) {
   const int nbf = N / R;
-  cpx<T> v[NB][R];
+  cpx<T> v[NB][R], w[NB][R];
+  // the twiddles (global memory) are on their way before the barrier
+  if (Ns > 1) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 1; r < R; ++r) w[b][r] = load_c(tw + (r - 1) * Ns + ((t + b * J) & (Ns - 1)));
+  }
 #pragma unroll
   for (int b = 0; b < NB; ++b)
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[b][r] = load_c(s + t + b * J + r * nbf);
+    for (int r = 0; r < R; ++r) v[b][r] = load_c(s + spos<T>(t + b * J + r * nbf));
   __syncthreads();
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
@@ -350,14 +402,13 @@ __device__ __forceinline__ void line_pass(cpx<T>* s, int N, int J, int Ns, int t
     if (Ns > 1) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        cpx<T> w = load_c(tw + (r - 1) * Ns + k);
-        if (INV) w.y = -w.y;
-        v[b][r] = fft::cmul(v[b][r], w);
+        if (INV) w[b][r].y = -w[b][r].y;
+        v[b][r] = fft::cmul(v[b][r], w[b][r]);
       }
     }
     fft::dft<INV, R>(v[b]);
 #pragma unroll
-    for (int r = 0; r < R; ++r) store_c(s + (j - k) * R + k + r * Ns, v[b][r]);
+    for (int r = 0; r < R; ++r) store_c(s + spos<T>((j - k) * R + k + r * Ns), v[b][r]);
   }
   __syncthreads();
 }
@@ -376,7 +427,7 @@ __global__ void __launch_bounds__(512) k_line(LineArgs<T> a) {
     return w;
   };
   const cpx<T> w8 = S == 8 ? twid(q * (a.h / 4)) : cpx<T>{T(1), T(0)};   // W_8^q
-#pragma unroll 2
+#pragma unroll 4
   for (int n = t; n < N; n += J) {
     cpx<T> z[S];
 #pragma unroll
@@ -396,7 +447,7 @@ __global__ void __launch_bounds__(512) k_line(LineArgs<T> a) {
       }
       z[0] = fft::cmul(z[0], w);
     }
-    store_c(s + n, z[0]);
+    store_c(s + spos<T>(n), z[0]);
   }
   __syncthreads();
   const cpx<T>* tw = a.ptw;
@@ -411,7 +462,7 @@ __global__ void __launch_bounds__(512) k_line(LineArgs<T> a) {
   }
   for (int n = t; n < N; n += J) {
     const int j = q + S * n;
-    if (!INV || (j >= a.lo && j < a.hi)) store_c(dst + j, load_c(s + n));
+    if (!INV || (j >= a.lo && j < a.hi)) store_c(dst + j, load_c(s + spos<T>(n)));
   }
 }
 
@@ -527,7 +578,7 @@ int line_split(const Plan& plan, int CR) {
 
 template <typename T, bool INV, int S>
 void line_launch(const LineArgs<T>& a, const LinePlan& m, int CR, cudaStream_t st) {
-  const size_t smem = sizeof(cpx<T>) * (size_t)a.N;
+  const size_t smem = sizeof(cpx<T>) * ((size_t)a.N + a.N / (sizeof(T) == 4 ? 16 : 8) + 1);
   void (*k)(LineArgs<T>) = nullptr;
   if constexpr (sizeof(T) == 4)
     k = m.R == 4 ? k_line<T, INV, S, 4, 1> : (m.NB == 1 ? k_line<T, INV, S, 8, 1> : k_line<T, INV, S, 8, 2>);
