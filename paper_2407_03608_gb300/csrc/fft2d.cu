@@ -30,13 +30,11 @@
 #include <vector>
 
 #include "fft_core.h"
-#include "kernels.h"
+#include "fft2d.h"
 
 namespace gpn {
 
 namespace {
-
-using fft::cpx;
 
 template <typename T>
 struct Vec2;
@@ -92,8 +90,6 @@ constexpr int kPassUnroll = 4;
 // shared-memory elements of one row buffer: the padded length-N2 FFT plus the slot N2,
 // rounded up to an even count (16-byte alignment of what follows)
 __host__ __device__ constexpr int row_buf(int n2) { return (n2 + n2 / 16 + 2) & ~1; }
-// entries of one high-part twiddle table (W^{64 q}, q <= N2 / 64)
-__host__ __device__ constexpr int tw_hi(int n2) { return n2 / 64 + 1; }
 // The FP32 forward kernel reads per-pass twiddle tables (fft::pass_tables) staged in
 // shared memory, one load a twiddle; the others form the FFT twiddles from the
 // two-level tables (measured: the inverse kernel runs faster with the smaller
@@ -112,23 +108,6 @@ template <typename T, bool INV>
 constexpr size_t row_smem(int L, int rb) {
   return ((size_t)rb * row_buf(1 << L) + tw_count<T, INV>(L)) * sizeof(cpx<T>);
 }
-
-// the twiddle functors over the tables staged in shared memory
-template <typename T>
-struct RowsArgs {
-  const T* gin;            // spreading grids (forward input), (R*C) x nf x nf
-  T* gout;                 // interp grids (inverse output)
-  cpx<T>* X;               // forward row output / inverse row input: [cr][M+1][nf]
-  const cpx<T>* tw;        // two-level tables: W_{N2} (hi, lo), then W_nf (hi, lo)
-  long long nf;
-  long long G;             // nf^2
-  int M;
-  int row0;                // first row of item 0 (a multiple of RB)
-  int row_hi;
-  long long npairs;        // RB-row groups per grid
-  long long nitems;        // npairs * C * R
-  int col_lo, col_hi;
-};
 
 // In-place complex FFT of length N = 2^L on the row buffer b by Stockham passes (one of
 // radix 2^(L mod 4) when L is not a multiple of 4, then radix 16), NT = N / 16 threads per
@@ -690,7 +669,10 @@ template <typename T, int L, int RB>
 void rows_launch(bool inv, const RowsArgs<T>& a, cudaStream_t st) {
   const size_t smem = inv ? row_smem<T, true>(L, RB) : row_smem<T, false>(L, RB);
   const int threads = RB * (1 << L) / 16;
-  void (*k)(RowsArgs<T>) = inv ? k_rows_inv<T, L, RB> : k_rows_fwd<T, L, RB>;
+  void (*k)(RowsArgs<T>) = k_rows_fwd<T, L, RB>;
+  if constexpr (sizeof(T) == 8) {   // (FP32 inverse rows: rows2d.cu)
+    if (inv) k = k_rows_inv<T, L, RB>;
+  }
   GPN_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // one item per block: adjacent row groups run together, so the two halves of a
   // 32-byte sector of the transposed output meet in L2 (a persistent grid, tried,
@@ -760,7 +742,15 @@ void rows_run(Plan& plan, bool inv, const void* X, int R, cudaStream_t st) {
   if (plan.row_hi <= a.row0) return;
   a.npairs = (plan.row_hi - a.row0 + plan.t3_rb - 1) / plan.t3_rb;
   a.nitems = a.npairs * plan.geom.C * R;
-  rows<T>(inv, log2_exact(plan.geom.nf / 2), plan.t3_rb, a, st);
+  const int L = log2_exact(plan.geom.nf / 2);
+  if constexpr (sizeof(T) == 4) {
+    if (inv) {
+      rows_pairs_inv(L, a, plan.row_lo, plan.geom.C * R, st);
+      GPN_CUDA(cudaGetLastError());
+      return;
+    }
+  }
+  rows<T>(inv, L, plan.t3_rb, a, st);
   GPN_CUDA(cudaGetLastError());
 }
 
