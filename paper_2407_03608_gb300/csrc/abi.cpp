@@ -177,6 +177,7 @@ Plan::~Plan() {
   if (cg_graph.exec) cudaGraphExecDestroy(cg_graph.exec);
   if (cap_stream) cudaStreamDestroy(cap_stream);
   for (void* p : owned) cudaFree(p);
+  if (query_ws) cudaFree(query_ws);
   if (host_scal) cudaFreeHost(host_scal);
   if (host_status) cudaFreeHost(host_status);
 }
@@ -626,6 +627,26 @@ struct DevOut {
   }
 };
 
+// The plan's workspace for posterior means, grown to `need` bytes, or null when it would pass
+// kQueryKeep or the plan's max_bytes (the caller then allocates for the call).
+void* query_workspace(Plan& p, size_t need) {
+  if (need <= p.query_ws_bytes) return p.query_ws;
+  const long long after = p.bytes + (long long)(need - p.query_ws_bytes);
+  if (need > kQueryKeep || (p.max_bytes > 0 && after > p.max_bytes)) return nullptr;
+  if (p.query_ws) GPN_CUDA(cudaFree(p.query_ws));
+  p.bytes -= (long long)p.query_ws_bytes;
+  p.query_ws = nullptr;
+  p.query_ws_bytes = 0;
+  if (cudaMalloc(&p.query_ws, need) != cudaSuccess) {
+    cudaGetLastError();
+    p.query_ws = nullptr;
+    return nullptr;
+  }
+  p.query_ws_bytes = need;
+  p.bytes += (long long)need;
+  return p.query_ws;
+}
+
 // Input through the plan staging buffer when on the host.
 const double* dev_input(const double* src, double* stage, size_t count, cudaStream_t st) {
   if (is_device_ptr(src)) return src;
@@ -820,10 +841,24 @@ int gp_posterior_mean(gp_plan_t plan, const double* alpha, const double* xq, lon
     GPN_CHECK(Nq >= 1, GP_EINVAL, "Nq must be >= 1");
     const int d = p->h.d;
     DevIn x(xq, (size_t)Nq * d, st), a(field_aq, Nq, st), b(field_bq, Nq, st);
-    DevTmp wbuf(sizeof(double) * Nq), sbuf(sizeof(double) * Nq), outs(sizeof(double) * Nq), outo(sizeof(double) * Nq);
-    fields_to_paper(a.ptr, b.ptr, (double*)wbuf.p, (double*)sbuf.p, Nq, d, p->param_mode, st);
+    // one allocation: the paper-native fields, two vectors of results, the statistics' partial
+    // sums and, for query sets that are not binned, their cells and weights
+    const bool direct = query_unbinned(*p, Nq);
+    const size_t vb = (sizeof(double) * (size_t)Nq + 255) / 256 * 256;
+    const size_t need = 4 * vb + kStatsBytes + (direct ? query_work_bytes(*p, Nq) : 0);
+    std::unique_ptr<DevTmp> work;
+    char* wp = (char*)query_workspace(*p, need);
+    if (!wp) {
+      work.reset(new DevTmp(need));
+      wp = (char*)work->p;
+    }
+    double* const wq = (double*)wp;
+    double* const sq = (double*)(wp + vb);
+    double* const outs = (double*)(wp + 2 * vb);
+    double* const outo = (double*)(wp + 3 * vb);
+    fields_to_paper(a.ptr, b.ptr, wq, sq, Nq, d, p->param_mode, st);
     double stats[9];
-    field_stats(x.ptr, (double*)wbuf.p, (double*)sbuf.p, Nq, d, stats, st);
+    field_stats(x.ptr, wq, sq, Nq, d, stats, st, wp + 4 * vb);
     GPN_CHECK(stats[8] == 0.0, GP_EINVAL, "invalid query entries");
     GPN_CHECK(stats[0] >= p->h.sig_lo * (1 - 1e-12) && stats[1] <= p->h.sig_hi * (1 + 1e-12), GP_EINVAL,
               "query sigma outside the plan's [sigma_lo, sigma_hi]");
@@ -832,16 +867,23 @@ int gp_posterior_mean(gp_plan_t plan, const double* alpha, const double* xq, lon
                 "query points outside the plan box");
     TmpList tl;
     PointSet qs;
-    build_pointset(*p, qs, x.ptr, (double*)wbuf.p, (double*)sbuf.p, Nq, st, tmp_alloc_cb, &tl);
+    if (direct)
+      build_query_points(*p, qs, x.ptr, wq, sq, Nq, wp + 4 * vb + kStatsBytes, st);
+    else
+      build_pointset(*p, qs, x.ptr, wq, sq, Nq, st, tmp_alloc_cb, &tl);
     const double* al = dev_input(alpha, p->stage_in, (size_t)p->N, st);
     gather_sorted(p->pts, al, p->vec_a, 1, st);
     launch_spread(*p, p->vec_a, 1, st);
     run_fft_forward(*p, 1, st);
     launch_diag(*p, 1, st);
     run_fft_inverse(*p, 1, st);
-    launch_interp(*p, qs, nullptr, 0.0, (double*)outs.p, 1, st);
-    DevOut o(mu, (double*)outo.p, (size_t)Nq);
-    scatter_sorted(qs, (double*)outs.p, o.dev, 1, st);
+    DevOut o(mu, outo, (size_t)Nq);
+    if (direct) {
+      launch_query_mean(*p, qs, o.dev, st);
+    } else {
+      launch_interp(*p, qs, nullptr, 0.0, outs, 1, st);
+      scatter_sorted(qs, outs, o.dev, 1, st);
+    }
     GPN_CUDA(cudaGetLastError());
     o.finish(*p, st);
     check_device_status(*p, st);  // temporaries are freed on return

@@ -143,7 +143,11 @@ __device__ __forceinline__ double to_f64(T v) {
 
 // Chebyshev weights of Eq. (Wk) from the paper-native fields of one point:
 // w_k(x) = w (2 pi sigma^2)^(-d/2) P_k(sigma), P_k by the barycentric formula on the
-// Chebyshev-Lobatto nodes (weights (-1)^k, halved at both ends); exact at a node.
+// Chebyshev-Lobatto nodes (weights (-1)^k, halved at both ends) with numerator and denominator
+// multiplied by prod_j (sigma - sigma_j): P_k = b_k prod_{j != k} (sigma - sigma_j) / sum of the
+// same, 4 C products and one division instead of 2 C divisions (float64 divisions made the
+// weights the largest kernel of a posterior mean), and exact at a node.  The differences are
+// scaled by the interval, so that the products of up to 31 of them stay in range.
 struct ChebArgs {
   double nodes[kMaxChannels];
   double bary[kMaxChannels];
@@ -151,17 +155,27 @@ struct ChebArgs {
   int d;
 };
 __device__ __forceinline__ void cheb_weights(double w, double s, const ChebArgs& cb, double* out) {
-  const double pre = w * pow(6.283185307179586476925286766559 * s * s, -0.5 * cb.d);
-  int hit = -1;
-  for (int k = 0; k < cb.C; ++k)
-    if (s == cb.nodes[k]) hit = k;
-  if (hit >= 0 || cb.C == 1) {
-    for (int k = 0; k < cb.C; ++k) out[k] = (k == hit || cb.C == 1) ? pre : 0.0;
+  // x^(-d/2) by a square root and a division (pow costs several times the rest of the weights)
+  const double x = 6.283185307179586476925286766559 * s * s;
+  const double pre = w / (cb.d == 1 ? sqrt(x) : cb.d == 2 ? x : x * sqrt(x));
+  if (cb.C == 1) {
+    out[0] = pre;
     return;
   }
-  double den = 0.0;
-  for (int k = 0; k < cb.C; ++k) den += cb.bary[k] / (s - cb.nodes[k]);
-  for (int k = 0; k < cb.C; ++k) out[k] = pre * (cb.bary[k] / (s - cb.nodes[k])) / den;
+  const double inv = 1.0 / fabs(cb.nodes[cb.C - 1] - cb.nodes[0]);
+  double run = 1.0, den = 0.0;
+  for (int k = 0; k < cb.C; ++k) {   // products of the differences before k ...
+    out[k] = cb.bary[k] * run;
+    run *= (s - cb.nodes[k]) * inv;
+  }
+  run = 1.0;
+  for (int k = cb.C - 1; k >= 0; --k) {   // ... times those after k
+    out[k] *= run;
+    den += out[k];
+    run *= (s - cb.nodes[k]) * inv;
+  }
+  const double scale = pre / den;
+  for (int k = 0; k < cb.C; ++k) out[k] *= scale;
 }
 
 // Channel-count buckets: kernels keep per-channel values in registers sized by a

@@ -183,6 +183,9 @@ struct Plan {
   bool tr3 = false;
   Box3 box3;                            // d = 3 over the occupied box
   GridView view;                        // layout of grid and grid_out
+  // workspace of posterior means, kept between calls up to kQueryKeep bytes (and max_bytes)
+  void* query_ws = nullptr;
+  size_t query_ws_bytes = 0;
   // d = 1 (line1d.cu): where each cell's points start, and the split transforms
   int* line_start = nullptr;            // first sorted point with l0 >= c, c = 0..nf
   int line_cell0 = 0, line_cell1 = 0;   // cells the points reach
@@ -241,8 +244,10 @@ void fields_to_paper(const double* a, const double* b, double* w_out, double* si
                      cudaStream_t st);
 
 // min / max of sigma and of each coordinate, and the count of invalid entries.
+// work: kStatsBytes of device memory (null: allocated for the call)
+constexpr size_t kStatsBytes = sizeof(double) * 9 * 1024;
 void field_stats(const double* x, const double* w, const double* sig, long long n, int d, double* host_out,
-                 cudaStream_t st);
+                 cudaStream_t st, void* work = nullptr);
 
 // Build the packed A' tensor on the device from the E' tables.
 void build_a_tensor(Plan& plan, cudaStream_t st);
@@ -251,6 +256,7 @@ void build_a_tensor(Plan& plan, cudaStream_t st);
 constexpr size_t kInterpSmemBudget = size_t(96) << 10;   // target when sizing channel chunks
 constexpr size_t kInterpSmemMax = size_t(200) << 10;      // one staged channel must fit
 constexpr size_t kSpreadSmemMax = size_t(160) << 10;      // shared tile of one spreading channel chunk
+constexpr size_t kQueryKeep = size_t(64) << 20;
 constexpr double kHostTableMax = 32e9;                     // bytes of plan-time host tables
 int spread_pitch(int d, int tile);
 size_t spread_smem_bytes(int d, int tile, int C, size_t rs, int width);
@@ -295,6 +301,14 @@ void launch_interp(Plan& plan, const PointSet& ps, const double* alpha_sorted, d
 // ... on the 3-D box grids (interp3d.cu)
 void launch_interp3d(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shift, double* out_sorted,
                      int R, cudaStream_t st);
+
+// Query points without binning (query.cu): work holds query_work_bytes(n); the mean is written
+// in the order of the queries.
+bool query_unbinned(const Plan& plan, long long n);
+size_t query_work_bytes(const Plan& plan, long long n);
+void build_query_points(const Plan& plan, PointSet& qs, const double* x, const double* w, const double* sig,
+                        long long n, void* work, cudaStream_t st);
+void launch_query_mean(Plan& plan, const PointSet& qs, double* mu, cudaStream_t st);
 
 // Static scratch of gp_posterior_mean_noalloc (one array per device): a rejected-
 // query counter in the first kNoAllocHeaderBytes, then float64 staging for host
