@@ -167,6 +167,57 @@ void read_scalars(Plan& plan, int R, cudaStream_t st) {
 // iterations per host check (and per captured graph)
 constexpr int kCgBlock = 16;
 
+// The vector part of an iteration for short columns in one launch: p.Ap, x += a p, r -= a Ap,
+// r.r, p = r + b p, the scalars and the convergence test, one block a column (fixed-order
+// sums).  The separate kernels cost seven launches of 3 to 4 us each; one SM's float64 pipe does
+// a column of kCgSmall points in about 8 us.
+constexpr long long kCgSmall = 4096;
+constexpr int kCgSmallThreads = 512;
+
+__device__ __forceinline__ double block_total(double v, double* sh) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  __syncthreads();   // sh is free again
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < kCgSmallThreads / 32; ++w) s += sh[w];
+  return s;
+}
+
+__global__ void __launch_bounds__(kCgSmallThreads) k_cg_small(double* __restrict__ x, double* __restrict__ res,
+                                                              double* __restrict__ p, const double* __restrict__ ap,
+                                                              int n, double* scal, int R, double rtol2, int* cnt) {
+  __shared__ double sh[kCgSmallThreads / 32];
+  const int r = blockIdx.x;
+  if (scal[4 * R + r] == 0.0) return;
+  x += (size_t)r * n, res += (size_t)r * n, p += (size_t)r * n, ap += (size_t)r * n;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += kCgSmallThreads) s += p[i] * ap[i];
+  const double pap = block_total(s, sh), rr = scal[0 * R + r], a = rr / pap;
+  s = 0.0;
+  for (int i = threadIdx.x; i < n; i += kCgSmallThreads) {
+    x[i] += a * p[i];
+    const double ri = res[i] - a * ap[i];
+    res[i] = ri;
+    s += ri * ri;
+  }
+  const double rrn = block_total(s, sh), b = rrn / rr;
+  for (int i = threadIdx.x; i < n; i += kCgSmallThreads) p[i] = res[i] + b * p[i];
+  if (threadIdx.x == 0) {
+    scal[0 * R + r] = rrn;
+    scal[1 * R + r] = pap;
+    scal[2 * R + r] = rrn;
+    cnt[r] += 1;
+    if (!(pap > 0.0) || !isfinite(pap) || !isfinite(rrn)) {
+      scal[4 * R + r] = 0.0;
+      cnt[R] = 1;
+    } else if (rrn <= rtol2 * scal[3 * R + r]) {
+      scal[4 * R + r] = 0.0;
+    }
+  }
+}
+
 void cg_iteration(Plan& plan, double* xr, int R, double eta2, double rtol, cudaStream_t st) {
   const long long n = plan.N;
   const int nb = red_blocks(n);
@@ -174,6 +225,10 @@ void cg_iteration(Plan& plan, double* xr, int R, double eta2, double rtol, cudaS
   double* p = plan.cg_p;
   double* ap = plan.cg_ap;
   matvec_sorted(plan, p, ap, R, eta2, st);
+  if (n <= kCgSmall) {
+    k_cg_small<<<R, kCgSmallThreads, 0, st>>>(xr, r, p, ap, (int)n, plan.scal, R, rtol * rtol, plan.cg_cnt);
+    return;
+  }
   dot(p, ap, n, R, plan.partials, plan.scal, 1, st);
   k_update_xr<<<dim3(nb, R), kRedThreads, 0, st>>>(xr, r, p, ap, n, plan.scal, R, plan.partials);
   k_dot_final<<<R, kRedThreads, 0, st>>>(plan.partials, nb, plan.scal, 2, R);
