@@ -14,11 +14,14 @@
 // The order, and so the summation order, is fixed (results are reproducible bit for bit).
 // Every grid value is written once; tiles no point can reach are never launched and stay zero.
 //
+// FP32 sums are kept as pairs of channels, one packed multiply-add each (the same roundings).
+//
 // Bound: FP32 issue.  A point meets 54 (warp, group) cells sets at width 9 (RPW = 4), 42 % of
 // whose multiply-adds fall inside its support.
 #include <algorithm>
 #include <type_traits>
 
+#include "fft_mixed.h"
 #include "kernels.h"
 
 namespace gpn {
@@ -34,6 +37,8 @@ constexpr int kWarps = kTZ * kBands;
 constexpr int kThreads = 32 * kWarps;
 constexpr int kLists = kWarps * kGroups;
 constexpr int kSlots = kThreads;           // points a batch (one a thread fills its tables)
+constexpr int kScan = 4;                   // candidates a thread tests at a time
+constexpr int kQueue = (kScan + 1) * kSlots;   // a scan adds up to kScan kSlots to less than kSlots
 constexpr int kMaxRanges = 64;             // bin rows a tile's candidates can come from
 
 // per-slot shared tables (odd strides against bank conflicts); the row table has RPW - 1 zeros
@@ -69,6 +74,9 @@ struct Spread3Args {
 template <typename T, int NC, int RPW>
 __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2)) k_spread3d(Spread3Args<T> a) {
   constexpr int TY = kBands * RPW, WP = wk_pitch<T>(NC), VW = (int)(16 / sizeof(T));
+  // a sum: two channels (FP32) or one
+  using Acc = typename std::conditional<sizeof(T) == 4, fft::f2, double>::type;
+  constexpr int AL = fft::Elem<Acc>::lanes, NA = (NC + AL - 1) / AL;
   using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
   const int W = a.width, PS = axis_stride(W), SY = row_stride(W, RPW), C = a.C, r = blockIdx.y;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -77,9 +85,9 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
   T* s_psx = reinterpret_cast<T*>(s_l0 + kSlots);                // [kSlots][PS]
   T* s_psz = s_psx + kSlots * PS;                                // [kSlots][PS]
   T* s_psy = s_psz + kSlots * PS;                                // [kSlots][SY]
-  int* s_idx = reinterpret_cast<int*>(s_psy + kSlots * SY);      // [2 kSlots]: queue of points
-  unsigned char* s_list = reinterpret_cast<unsigned char*>(s_idx + 2 * kSlots);  // [kLists][kSlots]
-  __shared__ int s_rs[kMaxRanges], s_rl[kMaxRanges], s_wcnt[kWarps];
+  int* s_idx = reinterpret_cast<int*>(s_psy + kSlots * SY);      // [kQueue]: queue of points
+  unsigned char* s_list = reinterpret_cast<unsigned char*>(s_idx + kQueue);      // [kLists][kSlots]
+  __shared__ int s_rs[kMaxRanges], s_rl[kMaxRanges], s_wcnt[kScan][kWarps];
   __shared__ int s_cnt[kLists][kWarps], s_len[kLists];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -104,11 +112,11 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
   int total = 0;
   for (int q = 0; q < nr; ++q) total += s_rl[q];
 
-  T acc[RPW][NC];
+  Acc acc[RPW][NA];
 #pragma unroll
   for (int rr = 0; rr < RPW; ++rr)
 #pragma unroll
-    for (int k = 0; k < NC; ++k) acc[rr][k] = T(0);
+    for (int k = 0; k < NA; ++k) acc[rr][k] = fft::vset<Acc>(T(0));
   const int grp = lane >> 3;
   const int xg = x0 + grp * kStrip + (lane & 7);                     // this lane's column
   const int zw = z0 + warp / kBands, rw0 = y0 + warp % kBands * RPW;  // the warp's plane, first row
@@ -117,36 +125,59 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
   const double* alpha_r = a.alpha + (size_t)r * a.n;
 
   int queued = 0;
-  for (int c0 = 0; c0 < total || queued > 0; c0 += kThreads) {
-    if (c0 < total) {
-      // scan: one candidate per thread; the ones meeting the tile join the queue in order
-      int c = c0 + tid, p = 0;
-      bool meets = c < total;
-      if (meets) {
-        for (int q = 0; q < nr; ++q) {
-          if (c < s_rl[q]) {
-            p = s_rs[q] + c;
-            break;
-          }
-          c -= s_rl[q];
-        }
-        const int lz = a.l0[0][p], ly = a.l0[1][p], lx = a.l0[2][p];
-        meets = lz + W > z0 && lz < z0 + kTZ && ly + W > y0 && ly < y0 + TY && lx + W > x0 && lx < x0 + kTX;
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, meets);
-      if (lane == 0) s_wcnt[warp] = __popc(bal);
-      __syncthreads();
-      int off = queued, nrel = 0;
+  for (int c0 = 0; c0 < total || queued > 0; ) {
+    if (c0 < total && queued < kSlots) {
+      // scan: kScan candidates per thread (their cells are loaded before the first test); the
+      // ones meeting the tile join the queue in order
+      int p[kScan];
+      unsigned bal[kScan];
+      bool meets[kScan];
 #pragma unroll
-      for (int q = 0; q < kWarps; ++q) {
-        const int v = s_wcnt[q];
-        off += q < warp ? v : 0;
-        nrel += v;
+      for (int i = 0; i < kScan; ++i) {
+        int c = c0 + i * kThreads + tid;
+        meets[i] = c < total;
+        p[i] = 0;
+        if (meets[i]) {
+          for (int q = 0; q < nr; ++q) {
+            if (c < s_rl[q]) {
+              p[i] = s_rs[q] + c;
+              break;
+            }
+            c -= s_rl[q];
+          }
+        }
       }
-      if (meets) s_idx[off + __popc(bal & lt)] = p;
-      queued += nrel;
+      int lz[kScan], ly[kScan], lx[kScan];
+#pragma unroll
+      for (int i = 0; i < kScan; ++i) {
+        lz[i] = a.l0[0][p[i]];
+        ly[i] = a.l0[1][p[i]];
+        lx[i] = a.l0[2][p[i]];
+      }
+#pragma unroll
+      for (int i = 0; i < kScan; ++i) {
+        meets[i] = meets[i] && lz[i] + W > z0 && lz[i] < z0 + kTZ && ly[i] + W > y0 && ly[i] < y0 + TY &&
+                   lx[i] + W > x0 && lx[i] < x0 + kTX;
+        bal[i] = __ballot_sync(0xffffffffu, meets[i]);
+        if (lane == 0) s_wcnt[i][warp] = __popc(bal[i]);
+      }
       __syncthreads();
-      if (queued < kSlots && c0 + kThreads < total) continue;
+      int end = queued;
+#pragma unroll
+      for (int i = 0; i < kScan; ++i) {
+        int off = end;
+#pragma unroll
+        for (int q = 0; q < kWarps; ++q) {
+          const int v = s_wcnt[i][q];
+          off += q < warp ? v : 0;
+          end += v;
+        }
+        if (meets[i]) s_idx[off + __popc(bal[i] & lt)] = p[i];
+      }
+      queued = end;
+      c0 += kScan * kThreads;
+      __syncthreads();
+      if (queued < kSlots && c0 < total) continue;
     }
     // a batch: tables of its points, one per thread
     const int nb = min(queued, kSlots);
@@ -200,9 +231,14 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
       if (q == 7) s_len[L] = inc;
     }
     // the queue's rest moves to its front
-    const int rest = queued - nb, moved = tid < rest ? s_idx[kSlots + tid] : 0;
+    const int rest = queued - nb;
+    int moved[kScan];
+#pragma unroll
+    for (int i = 0; i < kScan; ++i) moved[i] = i * kThreads + tid < rest ? s_idx[kSlots + i * kThreads + tid] : 0;
     __syncthreads();
-    if (tid < rest) s_idx[tid] = moved;
+#pragma unroll
+    for (int i = 0; i < kScan; ++i)
+      if (i * kThreads + tid < rest) s_idx[i * kThreads + tid] = moved[i];
     queued = rest;
 #pragma unroll
     for (int L = 0; L < kLists; ++L) {
@@ -224,24 +260,25 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
       const int dx = xg - l0.z;
       const bool in = ok && (unsigned)dx < (unsigned)W;
       const T pxz = in ? s_psx[is * PS + dx] * s_psz[is * PS + (zw - l0.x)] : T(0);
-      T wk[WP];
+      Acc wk[WP / AL];
 #pragma unroll
       for (int v = 0; v < WP / VW; ++v) {
         const V u = reinterpret_cast<const V*>(s_wk + is * WP)[v];
-        wk[VW * v] = u.x;
-        wk[VW * v + 1] = u.y;
         if constexpr (VW == 4) {
-          wk[VW * v + 2] = u.z;
-          wk[VW * v + 3] = u.w;
+          wk[2 * v] = {u.x, u.y};
+          wk[2 * v + 1] = {u.z, u.w};
+        } else {
+          wk[2 * v] = u.x;
+          wk[2 * v + 1] = u.y;
         }
       }
       // rows of the band relative to the support: in [1 - RPW, W - 1] for list members
       const T* pyr = s_psy + is * SY + (RPW - 1) + (ok ? rw0 - l0.y : 0);
 #pragma unroll
       for (int rr = 0; rr < RPW; ++rr) {
-        const T v = pxz * pyr[rr];
+        const Acc v = fft::vset<Acc>(pxz * pyr[rr]);
 #pragma unroll
-        for (int k = 0; k < NC; ++k) acc[rr][k] += v * wk[k];
+        for (int k = 0; k < NA; ++k) acc[rr][k] = fft::vfma(v, wk[k], acc[rr][k]);
       }
     }
     __syncthreads();  // slots, lists and counters are refilled by the next batch
@@ -256,15 +293,10 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
     const int gy = rw0 + rr - a.v.lo[1];
     if (gy < a.v.ext[1]) {
       T* o = gr + gy * a.v.stride[1];
-      if constexpr (NC <= 16 && NC % 4 == 0 && sizeof(T) == 4) {
+      // whole sums: the pitch holds them (in FP32 it is even, a padding channel's weights are zero)
 #pragma unroll
-        for (int k = 0; k < NC; k += 4)
-          *reinterpret_cast<float4*>(o + k) = make_float4(acc[rr][k], acc[rr][k + 1], acc[rr][k + 2], acc[rr][k + 3]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < NC; ++k)
-          if (k < C) o[k] = acc[rr][k];
-      }
+      for (int k = 0; k < NA; ++k)
+        if (k * AL < C) *reinterpret_cast<Acc*>(o + k * AL) = acc[rr][k];
     }
   }
 }
@@ -275,7 +307,8 @@ constexpr int rows_per_warp(int nc) { return (sizeof(T) == 8 || nc > 16) ? 2 : 4
 
 size_t smem_bytes(size_t rs, int nc, int rpw, int w) {
   const int wp = rs == 4 ? wk_pitch<float>(nc) : wk_pitch<double>(nc);
-  return (size_t)kSlots * ((2 * axis_stride(w) + row_stride(w, rpw) + wp) * rs + sizeof(int4) + 2 * sizeof(int) + kLists);
+  return (size_t)kSlots * ((2 * axis_stride(w) + row_stride(w, rpw) + wp) * rs + sizeof(int4) + kLists) +
+         sizeof(int) * kQueue;
 }
 
 template <typename T, int NC>
