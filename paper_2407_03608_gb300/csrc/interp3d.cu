@@ -10,7 +10,10 @@
 // then the planes weighted by psi(z); the 32 partial sums are added in float-float (FP32
 // plans) or float64.
 //
-// Bound: L1 load throughput and issue (about 9 instructions a row).
+// Bound: latency of the L1/L2 loads and issue (about 9 instructions a row).  On 2e6 points, ms:
+// the staged kernel of interp.cu 15.1 (8 channels, width 9, nf 512) and 26.7 (10, 9, nf 864); here
+// with 48 warps an SM 4.35 and 6.00, with 64 4.17 and 5.35.  Loads of two channels with packed
+// sums need 48 registers: 4.95; sorting the points finer than by bins changes nothing.
 #include <algorithm>
 
 #include "kernels.h"
@@ -19,7 +22,10 @@ namespace gpn {
 
 namespace {
 
-constexpr int kWarps = 8;
+// the rows are short chains of loads, so what counts is warps in flight: up to three loads a row
+// 64 an SM (32 registers, a few spilled outside the loop), above that what the registers allow
+template <int S>
+constexpr int kWarps = S <= 3 ? 16 : 8;
 constexpr int kPointsPerBlock = 64;
 
 template <typename T>
@@ -52,7 +58,7 @@ __device__ __forceinline__ double warp_total(double v) {
 
 // S: loads a row, ceil(width Cp / 32)
 template <typename T, int S>
-__global__ void __launch_bounds__(32 * kWarps) k_interp3d(Interp3Args<T> a) {
+__global__ void __launch_bounds__(32 * kWarps<S>, S <= 3 ? 4 : 1) k_interp3d(Interp3Args<T> a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = a.width, r = blockIdx.y;
   const long long s0 = a.v.stride[0], s1 = a.v.stride[1];
   const T* grid = a.grid + r * a.v.rstride + lane;
@@ -65,7 +71,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_interp3d(Interp3Args<T> a) {
     ks[s] = (s * 32 + lane) - xs[s] * a.Cp;
   }
   const long long p1 = min(a.n, (long long)(blockIdx.x + 1) * kPointsPerBlock);
-  for (long long p = (long long)blockIdx.x * kPointsPerBlock + warp; p < p1; p += kWarps) {
+  for (long long p = (long long)blockIdx.x * kPointsPerBlock + warp; p < p1; p += kWarps<S>) {
     const int lz = a.l0[0][p] - a.v.lo[0], ly = a.l0[1][p] - a.v.lo[1], lx = a.l0[2][p] - a.v.lo[2];
     T pz = T(0), py = T(0), px = T(0);
     if (lane < W) {
@@ -109,7 +115,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_interp3d(Interp3Args<T> a) {
 template <typename T, int S>
 void dispatch(const Interp3Args<T>& a, dim3 grid, cudaStream_t st) {
   if (a.width * a.Cp <= 32 * S)
-    k_interp3d<T, S><<<grid, 32 * kWarps, 0, st>>>(a);
+    k_interp3d<T, S><<<grid, 32 * kWarps<S>, 0, st>>>(a);
   else if constexpr (S < kMaxWidth * kMaxChannels / 32)
     dispatch<T, S + 1>(a, grid, st);
 }
