@@ -162,13 +162,21 @@ void interp_impl(const Plan& plan, const PointSet& qs, double* mu, cudaStream_t 
 
 }  // namespace
 
-// Query sets evaluated without binning: the 1-D and 2-D plans' and the 3-D box plans', up to
-// the sizes where the unsorted reads cost more than the sort (the 2-D and 3-D supports then come
-// from DRAM again and again).
+// Query sets evaluated without binning: the 1-D, 2-D and 3-D box plans', up to the sizes where
+// the unsorted reads of the supports cost more than the sort.  A posterior mean without / with
+// binning, ms (1e5 training points, 2e4 in 3-D float64):
+//   1-D FP32         1e5 queries .25 / .68   1e6 1.21 / 1.71
+//   2-D FP32         1e5 1.36 / 1.79         2.5e5 1.82 / 2.18     1e6 4.25 / 2.73
+//   2-D float-float  1e5 4.28 / 4.66         2.5e5 5.16 / 5.14     1e6 9.73 / 6.19
+//   2-D float64      1e5 4.70 / 4.74         2.5e5 5.89 / 5.41     1e6 11.9 / 7.28
+//   3-D FP32         2e3 1.54 / 1.71         2e5 2.08 / 2.75
+//   3-D float64      2e3 11.4 / 11.6         2e5 16.8 / 17.8
+// (2-D float64: the kernel values of an unbinned query are not tabulated, and their float64
+// arithmetic sets the line.)
 bool query_unbinned(const Plan& plan, long long n) {
   if (plan.geom.d == 1) return true;
-  if (plan.geom.d == 2) return n <= (1 << 18);
-  return plan.box3.on && n <= (1 << 16);
+  if (plan.geom.d == 3) return plan.box3.on && n <= (1 << 18);
+  return n <= (plan.precision == GP_FP64 ? 1 << 17 : 1 << 18);
 }
 
 size_t query_work_bytes(const Plan& plan, long long n) {
