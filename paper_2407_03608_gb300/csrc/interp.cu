@@ -3,17 +3,17 @@
 //   out_i = sum_k w_k(x_i) beta_k(x_i)  (+ shift * alpha_i).
 //
 // One CTA per non-empty tile bin and right-hand side.  The bin's points need the
-// cells [b*tile, b*tile + tile + width - 1) in every dimension.  For d >= 2 the
-// CTA brings that block of `cc` channels into shared memory with one TMA tile
-// copy (cp.async.bulk.tensor, completion on an mbarrier; out-of-range cells read
-// as zero); for d = 1 with a plain coalesced loop.  Then a group of lanes handles
-// each point:
-//   d = 1: one lane per point;  d = 2: one lane per support row (width lanes);
+// cells [b*tile, b*tile + tile + width - 1) in every dimension.  The CTA brings that
+// block of `cc` channels into shared memory with one TMA tile copy
+// (cp.async.bulk.tensor, completion on an mbarrier; out-of-range cells read as zero).
+// Then a group of lanes handles each point:
+//   d = 2: one lane per support row (width lanes);
 //   d = 3: one warp per point, lanes over the width^2 pencils.
+// 1-D plans read their grids in line1d.cu, 3-D plans with the box transforms in interp3d.cu.
 // Each lane accumulates its channels in registers.  d = 2: the lanes of a point write
 // their per-row sums to shared memory and lane k of the point adds up channel k's rows
 // (a transpose instead of one shuffle tree per channel), forms w_k(x_i) beta_k in FP32 and
-// the group sums the products in float64.  d = 1, 3: the group is reduced with shuffles
+// the group sums the products in float64.  d = 3: the group is reduced with shuffles
 // and the group leader applies w_k(x_i) in float64.
 // The mbarrier wait is bounded: when it runs out the CTA records a timeout in the
 // plan's device status word and returns.
@@ -38,9 +38,6 @@ struct InterpArgs {
   const int* bins;       // non-empty bins
   int nbins[kMaxDim];
   long long n;
-  const T* grid;
-  long long nf;
-  long long G;
   int width;
   T beta;
   T inv_halfw;
@@ -65,7 +62,7 @@ __host__ __device__ constexpr size_t transpose_bytes() { return use_transpose<T,
 
 // EXACT: every channel chunk holds exactly CMAX channels (C = cc = CMAX), so the
 // channel loops run without guards.
-template <typename T, int D, int CMAX, bool TMA, bool EXACT>
+template <typename T, int D, int CMAX, bool EXACT>
 __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw);
@@ -90,7 +87,7 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
   for (int q = 0; q < D - 1; ++q) lead_e *= E;
   const int SV = lead_e * EP;  // staged volume per channel
 
-  constexpr int kGroup = D == 1 ? 1 : (D == 2 ? 0 : 32);  // 0: width lanes
+  constexpr int kGroup = D == 2 ? 0 : 32;  // 0: width lanes
   const int Gs = kGroup == 0 ? W : kGroup;
   const int ppw = 32 / Gs;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -98,11 +95,10 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
   int P = 1;
 #pragma unroll
   for (int q = 0; q < D - 1; ++q) P *= W;
-  const T* grid_r = a.grid + (size_t)r * C * a.G;
   double* out_r = a.out + (size_t)r * a.n;
   const double* alpha_r = a.alpha ? a.alpha + (size_t)r * a.n : nullptr;
 
-  if (TMA && threadIdx.x == 0) mbar_init(bar, 1);
+  if (threadIdx.x == 0) mbar_init(bar, 1);
   unsigned phase = 0;
 
   // a batch's per-point data (first support cell relative to the block, offset xi);
@@ -123,51 +119,22 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
     int nl0[kMaxDim];
     T nx[kMaxDim];
     load_pt(warp * ppw, nl0, nx);
-    if (TMA) {
-      if (threadIdx.x == 0) {
-        mbar_expect_tx(bar, a.box_bytes);
-        if (D == 2)
-          tma_load_3d(st, &tmap, base[1], base[0], r * C + c0, bar);
-        else
-          tma_load_4d(st, &tmap, base[2], base[1], base[0], r * C + c0, bar);
-      }
-      const bool ok = mbar_wait_bounded(bar, phase, kMaxPolls);
-      if (__syncthreads_or(!ok)) {
-        if (threadIdx.x == 0) {
-          atomicExch(a.status, kStatusTimeout);
-          mbar_wait_bounded(bar, phase, kMaxPolls);  // let an in-flight copy land before exiting
-        }
-        return;
-      }
-      phase ^= 1u;
-    } else {
-      const int total = ncur * lead_e * E;
-      for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        int rem = idx;
-        const int last = rem % E;
-        rem /= E;
-        int soff = 0;
-        long long goff = 0;
-        bool in = (long long)base[D - 1] + last < a.nf;
-        int lcoord[kMaxDim];
-#pragma unroll
-        for (int q = D - 2; q >= 0; --q) {
-          lcoord[q] = rem % E;
-          rem /= E;
-        }
-        const int k = rem;
-#pragma unroll
-        for (int q = 0; q < D - 1; ++q) {
-          const long long gq = (long long)base[q] + lcoord[q];
-          in = in && gq < a.nf;
-          soff = soff * E + lcoord[q];
-          goff = goff * a.nf + gq;
-        }
-        goff = goff * a.nf + base[D - 1] + last;
-        st[(size_t)k * SV + soff * EP + last] = in ? grid_r[(size_t)(c0 + k) * a.G + goff] : T(0);
-      }
-      __syncthreads();
+    if (threadIdx.x == 0) {
+      mbar_expect_tx(bar, a.box_bytes);
+      if (D == 2)
+        tma_load_3d(st, &tmap, base[1], base[0], r * C + c0, bar);
+      else
+        tma_load_4d(st, &tmap, base[2], base[1], base[0], r * C + c0, bar);
     }
+    const bool ok = mbar_wait_bounded(bar, phase, kMaxPolls);
+    if (__syncthreads_or(!ok)) {
+      if (threadIdx.x == 0) {
+        atomicExch(a.status, kStatusTimeout);
+        mbar_wait_bounded(bar, phase, kMaxPolls);  // let an in-flight copy land before exiting
+      }
+      return;
+    }
+    phase ^= 1u;
 
     for (int pb = warp * ppw; pb < npts; pb += nwarps * ppw) {
       const int pi = pb + grp;
@@ -192,50 +159,38 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
         if (active && gl == 0 && c0 == 0 && alpha_r)
           shift_al = (a.dcorr ? a.shift + a.dcorr[p] : a.shift) * alpha_r[p];
       }
-      if (D == 1) {
-        if (active) {
-          const T* rowp = st + l0[0];
-          for (int i = 0; i < W; ++i) {
-            const T wgt = psi_at<T>(i, x[0], a.beta, a.inv_halfw);
+      // lane j of the group holds psi_q(j - xi_q) for every axis q; the others
+      // fetch them by shuffles (every lane executes every shuffle)
+      const int src = kGroup == 0 ? grp * Gs : 0;
+      T pq[kMaxDim];
+#pragma unroll
+      for (int q = 0; q < D; ++q)
+        pq[q] = gl < W ? (a.psi[q] ? a.psi[q][(size_t)p * W + gl] : psi_at<T>(gl, x[q], a.beta, a.inv_halfw))
+                       : T(0);
+      for (int pen0 = 0; pen0 < P; pen0 += Gs) {
+        const int pen = pen0 + gl;
+        const bool valid = active && pen < P;
+        int rem = valid ? pen : 0, off = 0;
+        T plead = T(1);
+        int iq[kMaxDim];
+#pragma unroll
+        for (int q = D - 2; q >= 0; --q) {
+          iq[q] = rem % W;
+          rem /= W;
+        }
+#pragma unroll
+        for (int q = 0; q < D - 1; ++q) {
+          plead *= shfl_val(pq[q], src + iq[q]);
+          off = off * E + l0[q] + iq[q];
+        }
+        const T* rowp = st + (size_t)off * EP + l0[D - 1];
+#pragma unroll 3
+        for (int i = 0; i < W; ++i) {
+          const T wgt = plead * shfl_val(pq[D - 1], src + i);
+          if (valid) {
 #pragma unroll
             for (int k = 0; k < CMAX; ++k)
               if (EXACT || k < ncur) madd_lazy(acc[k], wgt, rowp[(size_t)k * SV + i]);
-          }
-        }
-      } else {
-        // lane j of the group holds psi_q(j - xi_q) for every axis q; the others
-        // fetch them by shuffles (every lane executes every shuffle)
-        const int src = kGroup == 0 ? grp * Gs : 0;
-        T pq[kMaxDim];
-#pragma unroll
-        for (int q = 0; q < D; ++q)
-          pq[q] = gl < W ? (a.psi[q] ? a.psi[q][(size_t)p * W + gl] : psi_at<T>(gl, x[q], a.beta, a.inv_halfw))
-                         : T(0);
-        for (int pen0 = 0; pen0 < P; pen0 += Gs) {
-          const int pen = pen0 + gl;
-          const bool valid = active && pen < P;
-          int rem = valid ? pen : 0, off = 0;
-          T plead = T(1);
-          int iq[kMaxDim];
-#pragma unroll
-          for (int q = D - 2; q >= 0; --q) {
-            iq[q] = rem % W;
-            rem /= W;
-          }
-#pragma unroll
-          for (int q = 0; q < D - 1; ++q) {
-            plead *= shfl_val(pq[q], src + iq[q]);
-            off = off * E + l0[q] + iq[q];
-          }
-          const T* rowp = st + (size_t)off * EP + l0[D - 1];
-#pragma unroll 3
-          for (int i = 0; i < W; ++i) {
-            const T wgt = plead * shfl_val(pq[D - 1], src + i);
-            if (valid) {
-#pragma unroll
-              for (int k = 0; k < CMAX; ++k)
-                if (EXACT || k < ncur) madd_lazy(acc[k], wgt, rowp[(size_t)k * SV + i]);
-            }
           }
         }
       }
@@ -312,31 +267,31 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs<T> a, const __grid_co
   }
 }
 
-template <typename T, int D, int CMAX, bool TMA, bool EXACT = false>
+template <typename T, int D, int CMAX, bool EXACT = false>
 void launch(const InterpArgs<T>& a, const CUtensorMap& tm, dim3 grid, size_t smem0, cudaStream_t st) {
   const size_t smem = smem0 + transpose_bytes<T, D, CMAX>();
-  GPN_CUDA(cudaFuncSetAttribute(k_interp<T, D, CMAX, TMA, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  GPN_CUDA(cudaFuncSetAttribute(k_interp<T, D, CMAX, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem));
-  k_interp<T, D, CMAX, TMA, EXACT><<<grid, 256, smem, st>>>(a, tm);
+  k_interp<T, D, CMAX, EXACT><<<grid, 256, smem, st>>>(a, tm);
 }
 
 // d = 2 with all channels in one chunk and C <= 16: the exact channel count
 template <typename T, int NC>
 void launch_exact2(const InterpArgs<T>& a, const CUtensorMap& tm, dim3 grid, size_t smem, cudaStream_t st) {
   if constexpr (NC <= 16) {
-    if (a.C == NC) return launch<T, 2, NC, true, true>(a, tm, grid, smem, st);
+    if (a.C == NC) return launch<T, 2, NC, true>(a, tm, grid, smem, st);
     launch_exact2<T, NC + 1>(a, tm, grid, smem, st);
   }
 }
 
-template <typename T, int D, bool TMA>
+template <typename T, int D>
 void launch_c(const InterpArgs<T>& a, const CUtensorMap& tm, dim3 grid, size_t smem, cudaStream_t st) {
   if (D == 2 && a.cc == a.C && a.C <= 16) return launch_exact2<T, 1>(a, tm, grid, smem, st);
   switch (cmax_bucket(a.cc)) {
-    case 8: launch<T, D, 8, TMA>(a, tm, grid, smem, st); break;
-    case 12: launch<T, D, 12, TMA>(a, tm, grid, smem, st); break;
-    case 16: launch<T, D, 16, TMA>(a, tm, grid, smem, st); break;
-    default: launch<T, D, 32, TMA>(a, tm, grid, smem, st);
+    case 8: launch<T, D, 8>(a, tm, grid, smem, st); break;
+    case 12: launch<T, D, 12>(a, tm, grid, smem, st); break;
+    case 16: launch<T, D, 16>(a, tm, grid, smem, st); break;
+    default: launch<T, D, 32>(a, tm, grid, smem, st);
   }
 }
 
@@ -356,9 +311,6 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
   a.bin_start = ps.bin_start;
   a.bins = ps.active_bins;
   a.n = ps.n;
-  a.grid = (const T*)plan.grid_out;
-  a.nf = g.nf;
-  a.G = plan.grid_elems;
   a.width = g.width;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);
@@ -374,15 +326,14 @@ void interp_impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, dou
   a.out = out_sorted;
   a.status = plan.dev_status;
   // a TMA tile copy must start on a 16-byte boundary along x (x = bin * tile)
-  GPN_CHECK(g.d == 1 || (g.tile * sizeof(T)) % 16 == 0, GP_EUNSUPPORTED,
+  GPN_CHECK((g.tile * sizeof(T)) % 16 == 0, GP_EUNSUPPORTED,
             "interp tile must be a multiple of 16 bytes of grid values for the TMA copies");
   const size_t smem = 128 + (size_t)a.box_bytes;
   dim3 grid((unsigned)ps.n_active_bins, (unsigned)R);
-  switch (g.d) {
-    case 1: launch_c<T, 1, false>(a, plan.tmap_out, grid, smem, st); break;
-    case 2: launch_c<T, 2, true>(a, plan.tmap_out, grid, smem, st); break;
-    default: launch_c<T, 3, true>(a, plan.tmap_out, grid, smem, st);
-  }
+  if (g.d == 2)
+    launch_c<T, 2>(a, plan.tmap_out, grid, smem, st);
+  else
+    launch_c<T, 3>(a, plan.tmap_out, grid, smem, st);
   GPN_CUDA(cudaGetLastError());
 }
 
