@@ -416,7 +416,7 @@ PlanShape plan_shape(int d, long long N, double nu, double eps, const gp_plan_op
   const long long inv_work = (full && !pow2) ? CR * S * 2 * (long long)rs : 0;
   ps.est_rest = 2 * CR * grid_pitch * (long long)rs + spectra + N * (long long)(d * (4 + rs) + 8 + C * rs) +
                 (long long)N * max_rhs * 8 * 9 +
-                (psi_tabulated(d, o.precision) ? N * (long long)d * h.width * (long long)rs : 0);
+                (psi_tabulated(d, o.precision, false) ? N * (long long)d * h.width * (long long)rs : 0);
   // step 3: the stored tensor A' (1) or the memory-lean form from per-dimension
   // factors (2); auto takes the tensor unless it alone breaks max_bytes or the free
   // device memory
@@ -440,8 +440,8 @@ PlanShape plan_shape(int d, long long N, double nu, double eps, const gp_plan_op
 
 namespace {
 
-Plan* make_plan(const double* points, long long N, int d, const double* fa, const double* fb, double nu, double eps,
-                const gp_plan_opts& o, cudaStream_t st) {
+Plan* build_plan(const double* points, long long N, int d, const double* fa, const double* fb, double nu, double eps,
+                 const gp_plan_opts& o, cudaStream_t st, bool spare) {
   GPN_CHECK(d >= 1 && d <= 3, GP_EINVAL, "d must be 1, 2 or 3");
   GPN_CHECK(N >= 1, GP_EINVAL, "N must be >= 1");
   GPN_CHECK(points && fa && fb, GP_EINVAL, "null points or fields");
@@ -463,6 +463,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   plan->grid_rhs = (o.rhs_block > 0 && o.rhs_block < max_rhs) ? o.rhs_block : max_rhs;
   const int grid_rhs = plan->grid_rhs;
   plan->max_bytes = o.max_bytes;
+  plan->spare = spare;
   plan->real_size = o.precision == GP_FP32 ? 4 : 8;
 
   DevIn x(points, (size_t)N * d, st), a(fa, N, st), b(fb, N, st);
@@ -496,7 +497,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   plan->grid_elems = ps.G;
   plan->spec_elems = ps.S;
   plan->n_freq = ps.nfreq;
-  const bool box3 = !ps.tr3 && !ps.rowfft && box3_supported(d, h.nf);
+  const bool box3 = spare && !ps.tr3 && !ps.rowfft && box3_supported(d, h.nf);
   // box transforms keep A' on the octant |n_a| = 0..M only
   plan->box3.on = box3;
   if (box3) plan->n_freq = (h.M + 1) * (h.M + 1) * (h.M + 1);
@@ -513,7 +514,7 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   if (o.diag_correct) build_diag_correction(*plan, w, sig, st);
   GPN_CHECK(o.near_radius >= 0.0 && std::isfinite(o.near_radius), GP_EINVAL, "near_radius must be >= 0");
   if (o.near_radius > 0.0) build_near_field(*plan, o.near_radius, x.ptr, w, sig, st);
-  if (d == 1) line_points_setup(*plan, st);
+  if (d == 1 && spare) line_points_setup(*plan, st);
   build_active_tiles(*plan, bstart);
   if (spread2d_supported(*plan)) build_spread2d_tiles(*plan, bstart);
   GPN_CHECK(o.precision != GP_DF64 || plan->sp2_tiles, GP_EUNSUPPORTED,
@@ -563,13 +564,13 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
     GPN_CUDA(cudaMemsetAsync(plan->fz, 0, fbytes, st));
     if (plan->tr3)
       tr3_setup(*plan);
-    else if (line_supported(d, h.nf, o.precision, 3 * (h.M + 1)))
+    else if (spare && line_supported(d, h.nf, o.precision, 3 * (h.M + 1)))
       line_setup(*plan, plan->fx);
     else
       build_twiddles(*plan);
   } else if (!box3) {
     plan->spec = plan->alloc((size_t)C * grid_rhs * S * 2 * rs);
-    if (!plan->lean && line_supported(d, h.nf, o.precision, S)) line_setup(*plan, plan->spec);
+    if (spare && !plan->lean && line_supported(d, h.nf, o.precision, S)) line_setup(*plan, plan->spec);
   }
   plan->interp_cc = (int)std::max<size_t>(
       1, std::min<size_t>((size_t)C, kInterpSmemBudget / interp_stage_bytes(d, h.tile, h.width, rs)));
@@ -605,6 +606,18 @@ Plan* make_plan(const double* points, long long N, int d, const double* fa, cons
   GPN_CUDA(cudaStreamSynchronize(st));
   GPN_CHECK(plan->max_bytes <= 0 || plan->bytes <= plan->max_bytes, GP_ENOMEM, "plan exceeds max_bytes");
   return plan.release();
+}
+
+// A plan, with its spare tables wherever they fit.  (2-D plans have none.)
+Plan* make_plan(const double* points, long long N, int d, const double* fa, const double* fb, double nu, double eps,
+                const gp_plan_opts& o, cudaStream_t st) {
+  try {
+    return build_plan(points, N, d, fa, fb, nu, eps, o, st, true);
+  } catch (const Error& e) {
+    if (e.status != GP_ENOMEM || d == 2) throw;
+    cudaGetLastError();   // clear a failed allocation's error state
+  }
+  return build_plan(points, N, d, fa, fb, nu, eps, o, st, false);
 }
 
 // Resolve an output pointer: device pointers are written in place; host pointers go

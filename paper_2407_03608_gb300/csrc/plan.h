@@ -189,6 +189,10 @@ struct Plan {
   // d = 1 (line1d.cu): where each cell's points start, and the split transforms
   int* line_start = nullptr;            // first sorted point with l0 >= c, c = 0..nf
   int line_cell0 = 0, line_cell1 = 0;   // cells the points reach
+  // tables that only speed a plan up and are left out where it fits max_bytes (or the device)
+  // without them alone: the 1-D kernels' (then the tiled spread and the row or cuFFT transforms
+  // run) and the 3-D box's buffers
+  bool spare = true;
   bool line = false;
   void* line_spec = nullptr;            // [r][C][nf/2] complex
   void* line_tw = nullptr;              // exp(-2 pi i k / nf)
@@ -208,9 +212,12 @@ struct Plan {
   cufftHandle inv_plan(int R);
 };
 
-// Kernel values tabulated per point (PointSet::psi): the 1-D and 2-D float64 and float-float plans
-inline bool psi_tabulated(int d, int precision) { return d <= 2 && precision != GP_FP32; }
-inline bool psi_tabulated(const Plan& p) { return psi_tabulated(p.geom.d, p.precision); }
+// Kernel values tabulated per point (PointSet::psi): the 2-D float64 and float-float plans, and
+// the 1-D float64 ones that hold their spare tables (Plan::spare)
+inline bool psi_tabulated(int d, int precision, bool spare) {
+  return precision != GP_FP32 && (d == 2 || (d == 1 && spare));
+}
+inline bool psi_tabulated(const Plan& p) { return psi_tabulated(p.geom.d, p.precision, p.spare); }
 
 // Hyperparameters, layout and device footprint of a plan (host only; abi.cpp).
 struct PlanShape {

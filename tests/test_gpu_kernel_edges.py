@@ -1,0 +1,134 @@
+"""The 1-D line kernels, the 3-D box kernels, posterior means without binning and the short CG
+iteration at the sizes where they can go wrong: the smallest and largest transforms, odd radices,
+remainders of the tiles, channel counts on both sides of the kernels' groups.
+
+Bars: those stated for the same quantities elsewhere in the tests, relative l2 and max: the exact
+NUDFT 1e-9 (FP64 plans with a tight NUFFT tolerance) and 1e-4 (FP32); two routes through the same
+K~ 1e-12 and 2e-6.
+"""
+import numpy as np
+import pytest
+import torch
+
+import gpinputs
+from oracle import kernel as okern
+from oracle import ktilde
+
+from test_gpu_matvec import explicit_params, plan_kwargs, rel, small_case
+
+pytestmark = pytest.mark.gpu
+
+BAR = {"fp64": 1e-9, "fp32": 1e-4}
+SAME = {"fp64": 1e-12, "fp32": 2e-6}
+NU = {1: 1.5, 2: 1.5, 3: 2.5}
+
+
+def build(gpn, d, n, precision, n_t=12, n_sigma=4, M=20, **kw):
+    w = small_case(d, n, 0)
+    wp, sig = okern.paper_fields(w.s, w.l, d)
+    p = explicit_params(d, NU[d], sig, w.points, n_t=n_t, n_sigma=n_sigma, M=M)
+    plan = gpn.Plan(w.points, w.s, w.l, nu=NU[d], eps=1e-6, nufft_tol=1e-11 if precision == "fp64" else 1e-6,
+                    precision=gpn.GP_FP64 if precision == "fp64" else gpn.GP_FP32, **plan_kwargs(p), **kw)
+    return w, wp, sig, p, plan
+
+
+def check_matvec(gpn, d, n, precision, R, **kw):
+    w, wp, sig, p, plan = build(gpn, d, n, precision, max_rhs=R, **kw)
+    assert "nf" not in kw or plan.info["nf"] == kw["nf"]
+    for seed in (71, 72):     # the second call finds the buffers used
+        a = gpinputs.random_alpha(n, R, seed=seed)
+        ref = ktilde.matvec(w.points, wp, sig, a, p)
+        got = plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy()
+        e = rel(got, ref)
+        assert e <= BAR[precision], e
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf,M,n_sigma,R,n", [
+    (64, 12, 4, 1, 3000),        # the smallest transform, 70 points a cell
+    (128, 28, 1, 3, 700),        # two channels
+    (512, 100, 16, 5, 33),       # more channels than a group of 16, most cells empty
+    (8192, 1500, 14, 2, 2000),   # FP64: the split transform
+    (65536, 400, 9, 4, 1000),    # few modes of a long transform (FP64: the general row kernels)
+    (65536, 11000, 3, 1, 300),
+    (1 << 20, 300, 3, 1, 257),   # FP32: the longest transform
+])
+def test_line_kernels(gpn, precision, nf, M, n_sigma, R, n):
+    check_matvec(gpn, 1, n, precision, R, nf=nf, M=M, n_sigma=n_sigma)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf,M,n_sigma,step3,R,n", [
+    (54, 8, 3, 1, 2, 200),       # 2 3 3 3, the box is all but a cell of the grid
+    (56, 10, 1, 2, 1, 100),      # 2 2 2 7, two channels, memory-lean
+    (100, 10, 5, 1, 1, 1300),    # 2 2 5 5
+    (84, 10, 12, 2, 2, 150),     # 13 channels, memory-lean
+    (128, 8, 15, 1, 1, 100),     # 16 channels
+    (432, 5, 2, 1, 1, 70),       # passes held and not held in registers
+    (864, 4, 1, 2, 1, 65),       # the most passes
+])
+def test_box_kernels(gpn, precision, nf, M, n_sigma, step3, R, n):
+    if precision == "fp32" and nf % 4:
+        pytest.skip("FP32 plans take grids of a multiple of 4 cells")
+    check_matvec(gpn, 3, n, precision, R, nf=nf, M=M, n_sigma=n_sigma, step3=step3)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("d", [1, 2, 3])
+def test_posterior_mean_with_and_without_binning(gpn, precision, d):
+    """``many`` queries (2-D, 3-D: the first count that is binned), and the same ones in
+    calls that are not: one, a warp and one, all but one.  The first 40 against the oracle."""
+    many = 70000 if d == 1 else (1 << (17 if d == 2 and precision == "fp64" else 18)) + 1
+    w, wp, sig, p, plan = build(gpn, d, 400, precision, M={1: 60, 2: 24, 3: 8}[d])
+    g = np.random.default_rng(81)
+    i = g.integers(0, 400, (2, many))
+    t = g.random((many, 1))
+    t[:2] = [[0.0], [1.0]]
+    i[:, 0] = np.argmin(w.points[:, 0]), np.argmax(w.points[:, 0])   # the ends of the box
+    i[:, 1] = i[:, 0]
+    q = w.points[i[0]] * (1.0 - t) + w.points[i[1]] * t
+    s, l = (np.asarray(f)[i[0]] for f in (w.s, w.l))
+    alpha = torch.from_numpy(gpinputs.random_alpha(400, 1, seed=82)).cuda()
+    dev = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (q, s, l)]
+    full = plan.posterior_mean(alpha, *dev).cpu().numpy()
+    for m in (1, 33, many - 1):
+        part = plan.posterior_mean(alpha, *(v[:m] for v in dev)).cpu().numpy()
+        assert float(np.max(np.abs(part - full[:m]))) <= SAME[precision] * float(np.max(np.abs(full))), m
+    wq, sq = okern.paper_fields(s[:40], l[:40], d)
+    ref = ktilde.apply_cross(q[:40], wq, sq, w.points, wp, sig, alpha.cpu().numpy(), p)
+    assert rel(full[:40], ref) <= BAR[precision]
+
+
+@pytest.mark.parametrize("n", [33, 255, 4096, 4097])
+def test_cg_iterations_of_short_columns(gpn, n):
+    """Six iterations against the same recurrence on the host with the plan's own products;
+    columns up to 4096 points take the one-launch form.  The system is well conditioned
+    (eigenvalues within a factor 4), so rounding grows by less than 10 in six iterations."""
+    w, _, _, _, plan = build(gpn, 1, n, "fp64", M=60, max_rhs=2)
+    eta2 = 0.2 * n
+    y = gpinputs.random_alpha(n, 2, seed=91)
+    got, _ = plan.solve(torch.from_numpy(y).cuda(), eta2=eta2, rtol=1e-100, maxit=6)
+    x, r = np.zeros((n, 2)), y.copy()
+    s, rr = r.copy(), np.sum(r * r, axis=0)
+    for _ in range(6):
+        ap = plan.matvec(torch.from_numpy(s).cuda(), shift=eta2).cpu().numpy()
+        a = rr / np.sum(s * ap, axis=0)
+        x, r = x + a * s, r - a * ap
+        new = np.sum(r * r, axis=0)
+        s, rr = r + (new / rr) * s, new
+    assert rel(got.cpu().numpy(), x) <= 1e-12
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_1d_plan_without_spare_tables(gpn, precision):
+    """A limit that the 1-D kernels' tables do not fit: the plan is built without them, holds
+    less, and computes the same K~ (a limit below that is refused, as ever)."""
+    w, wp, sig, p, full = build(gpn, 1, 700, precision, M=300, max_rhs=2)
+    need = full.info["bytes_resident"]
+    *_, lean = build(gpn, 1, 700, precision, M=300, max_rhs=2, max_bytes=need - 1)
+    assert lean.info["bytes_resident"] < need
+    with pytest.raises(gpn.GPError):
+        build(gpn, 1, 700, precision, M=300, max_rhs=2, max_bytes=need // 2)
+    a = gpinputs.random_alpha(700, 2, seed=95)
+    for plan in (full, lean):
+        assert rel(plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy(), ktilde.matvec(w.points, wp, sig, a, p)) <= BAR[precision]
