@@ -593,7 +593,7 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   plan->partials = (double*)plan->alloc(sizeof(double) * 512 * max_rhs);
   GPN_CUDA(cudaMallocHost(&plan->host_scal, sizeof(double) * 8 * max_rhs));
   if (plan->tr3) {
-    if (o.precision != GP_DF64) plan->t3_plan(1);   // float-float columns are the library's own kernel
+    if (!own_cols(*plan)) plan->t3_plan(1);
   } else if (plan->rowfft) {
     if (d == 2) plan->col_plan(1);
   } else if (!box3 && !plan->line) {
@@ -608,13 +608,13 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   return plan.release();
 }
 
-// A plan, with its spare tables wherever they fit.  (2-D plans have none.)
+// A plan, with its spare tables wherever they fit.
 Plan* make_plan(const double* points, long long N, int d, const double* fa, const double* fb, double nu, double eps,
                 const gp_plan_opts& o, cudaStream_t st) {
   try {
     return build_plan(points, N, d, fa, fb, nu, eps, o, st, true);
   } catch (const Error& e) {
-    if (e.status != GP_ENOMEM || d == 2) throw;
+    if (e.status != GP_ENOMEM) throw;
     cudaGetLastError();   // clear a failed allocation's error state
   }
   return build_plan(points, N, d, fa, fb, nu, eps, o, st, false);

@@ -12,8 +12,8 @@
 //      X[cr][m][y] (cr = rhs * C + channel), the RB rows side by side.  Rows outside
 //      [row_lo, row_hi) are never written and stay zero.
 //   2. columns, forward: batched 1-D C2C of length nf over the C R (M+1) contiguous
-//      columns, from X into Y: cuFFT for float and double plans, the library's own
-//      k_cols for float-float plans (cuFFT has no float-float type).
+//      columns, from X into Y: the library's own k_cols, which skips the rows that hold
+//      nothing or that nothing reads, or cuFFT (own_cols() says which).
 //   3. step 3 (k_diag_t): a_k = sum_l A'_kl b_l for |n_1| <= M, from Y into Z.  A'
 //      depends on |n_1| and m only; one thread serves n_1 and -n_1 from the same A'
 //      entries.  Rows |n_1| > M of Z stay zero from plan creation on.
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(RB*(1 << L) / 16, (rows_min_blocks<T, L, RB>()
   if (first) cp_async_wait_all();
 }
 
-// ---- column transforms (float-float plans) -------------------------------------------
+// ---- column transforms ---------------------------------------------------------------
 //
 // The first-axis transforms of the transposed layout: every (rhs, channel, mode m)
 // column of nf complex values is contiguous, so one CTA takes one column, loads it
@@ -359,11 +359,23 @@ __global__ void __launch_bounds__(RB*(1 << L) / 16, (rows_min_blocks<T, L, RB>()
 //     [out_lo, out_hi) (the row groups the inverse row kernel reads).
 // Twiddles come from the pass tables of the length-nf FFT in global memory (L1/L2
 // resident; too large for shared memory next to a 16-byte-per-value column).
+// Bound: the FP32 issue rate (float-float), the FP64 pipe (float64), the latency of the
+// loads and exchanges at about 4 TB/s (FP32).
 
 // one complex value through the read-only path
 template <typename T>
 __device__ __forceinline__ cpx<T> ldg_c(const cpx<T>* p) {
   return *p;
+}
+template <>
+__device__ __forceinline__ cpx<float> ldg_c<float>(const cpx<float>* p) {
+  const float2 u = __ldg(reinterpret_cast<const float2*>(p));
+  return {u.x, u.y};
+}
+template <>
+__device__ __forceinline__ cpx<double> ldg_c<double>(const cpx<double>* p) {
+  const double2 u = __ldg(reinterpret_cast<const double2*>(p));
+  return {u.x, u.y};
 }
 template <>
 __device__ __forceinline__ cpx<dd> ldg_c<dd>(const cpx<dd>* p) {
@@ -429,8 +441,14 @@ __device__ __forceinline__ bool in_ranges(int y, int a0, int a1, int b0, int b1)
   return (y >= a0 && y < a1) || (y >= b0 && y < b1);
 }
 
+// resident CTAs asked for: 1024 threads an SM in FP32 (64 registers), 512 in float64
+template <typename T, int L>
+constexpr int cols_min_blocks() {
+  return is_dd<T>::value ? 1 : std::max(1, std::min(16, (sizeof(T) == 4 ? 1024 : 512) / ((1 << L) / 16)));
+}
+
 template <typename T, int L, bool INV>
-__global__ void __launch_bounds__((1 << L) / 16, 1) k_cols(ColsArgs<T> a) {
+__global__ void __launch_bounds__((1 << L) / 16, (cols_min_blocks<T, L>())) k_cols(ColsArgs<T> a) {
   constexpr int N = 1 << L, NT = N / 16;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* b = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -774,6 +792,20 @@ bool tr3_supported(int d, long long nf, int precision) {
   return (precision == GP_FP32 ? row_smem<float, false>(L, 1) : row_smem<double, false>(L, 1)) <= kRowSmemMax;
 }
 
+// Column transforms by k_cols, whose tables are among the spare ones (float-float has no other
+// transform).  cuFFT / k_cols, ms a direction, 8 channels (R = 1 unless stated), about nf/3 modes:
+//   FP32     nf 256 .006 / .006    512 .008 / .008   1024 .014 / .012   2048 .033 / .027
+//            4096 .115 / .102   (R = 4: .426 / .386)   8192 .497 / .578
+//   float64  nf 64 .010 / .015   256 .033 / .025   1024 .205 / .168   2048 .763 / .627
+//            4096 3.72 / 2.95   8192 16.9 / 14.3
+// The pruned rows (about a third of what cuFFT reads and writes) pay in FP32 until a column needs
+// four passes and 512 threads (8192; with radix 32 and three passes .508); float64 is bound by
+// its pipe.  Below 256 a column leaves most of its warp idle.
+bool own_cols(const Plan& plan) {
+  if (plan.precision == GP_DF64) return true;
+  return plan.spare && plan.geom.nf >= 256 && plan.geom.nf <= (plan.precision == GP_FP32 ? 4096 : 8192);
+}
+
 void tr3_setup(Plan& plan) {
   const long long nf = plan.geom.nf, N2 = nf / 2;
   const int L = log2_exact(N2);
@@ -812,27 +844,35 @@ void tr3_setup(Plan& plan) {
     GPN_CUDA(cudaMemcpy(plan.tw_half, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
   } else if (ddp) {
     upload_dd(plan.tw_half, w);
-    // the column transforms' pass tables (length nf), read from global memory
-    const std::vector<double> ct = fft::pass_tables(L + 1);
-    plan.col_tw = plan.alloc(std::max<size_t>(ct.size(), 2) * sizeof(dd));
-    if (!ct.empty()) upload_dd(plan.col_tw, ct);
   } else {
     GPN_CUDA(cudaMemcpy(plan.tw_half, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice));
+  }
+  if (!own_cols(plan)) return;
+  // the column transforms' pass tables (length nf), read from global memory
+  const std::vector<double> ct = fft::pass_tables(L + 1);
+  plan.col_tw = plan.alloc(std::max<size_t>(ct.size(), 2) * plan.real_size);
+  if (ct.empty()) return;
+  if (ddp) {
+    upload_dd(plan.col_tw, ct);
+  } else if (f32) {
+    const std::vector<float> f(ct.begin(), ct.end());
+    GPN_CUDA(cudaMemcpy(plan.col_tw, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
+  } else {
+    GPN_CUDA(cudaMemcpy(plan.col_tw, ct.data(), ct.size() * sizeof(double), cudaMemcpyHostToDevice));
   }
 }
 
 namespace {
-// the column transforms of the float-float plans (cuFFT has no float-float type)
-void cols_run_dd(Plan& plan, bool inv, const void* in, void* out, int R, cudaStream_t st) {
-  ColsArgs<dd> a{};
-  a.in = (const cpx<dd>*)in;
-  a.out = (cpx<dd>*)out;
-  a.ptab = (const cpx<dd>*)plan.col_tw;
+template <typename T>
+void cols_run(Plan& plan, bool inv, const void* in, void* out, int R, cudaStream_t st) {
+  ColsArgs<T> a{};
+  a.in = (const cpx<T>*)in;
+  a.out = (cpx<T>*)out;
+  a.ptab = (const cpx<T>*)plan.col_tw;
   a.ncols = (long long)plan.geom.C * R * (plan.geom.M + 1);
   const int nf = (int)plan.geom.nf, M = (int)plan.geom.M;
-  // the row groups of the inverse row kernel: [row0, row0 + npairs RB)
-  const int row0 = plan.row_lo / plan.t3_rb * plan.t3_rb;
-  const int rows_end = std::min(nf, row0 + (plan.row_hi - row0 + plan.t3_rb - 1) / plan.t3_rb * plan.t3_rb);
+  // the inverse row kernels read whole groups of 1, 2 or 4 rows
+  const int row0 = plan.row_lo / 4 * 4, rows_end = std::min(nf, (plan.row_hi + 3) / 4 * 4);
   if (!inv) {
     a.in_lo0 = plan.row_lo, a.in_hi0 = plan.row_hi, a.in_lo1 = 0, a.in_hi1 = 0;
     a.out_lo0 = 0, a.out_hi0 = M + 1, a.out_lo1 = nf - M, a.out_hi1 = nf;
@@ -841,8 +881,37 @@ void cols_run_dd(Plan& plan, bool inv, const void* in, void* out, int R, cudaStr
     a.out_lo0 = row0, a.out_hi0 = rows_end, a.out_lo1 = 0, a.out_hi1 = 0;
   }
   if (a.ncols == 0) return;
-  cols<dd>(inv, log2_exact(nf), a, st);
+  cols<T>(inv, log2_exact(nf), a, st);
   GPN_CUDA(cudaGetLastError());
+}
+
+// one direction of the column transforms (sign: CUFFT_FORWARD or CUFFT_INVERSE)
+void columns(Plan& plan, int sign, void* in, void* out, int R, cudaStream_t st) {
+  const bool inv = sign == CUFFT_INVERSE;
+  if (own_cols(plan)) {
+    if (plan.precision == GP_DF64)
+      cols_run<dd>(plan, inv, in, out, R, st);
+    else if (plan.precision == GP_FP32)
+      cols_run<float>(plan, inv, in, out, R, st);
+    else
+      cols_run<double>(plan, inv, in, out, R, st);
+    return;
+  }
+  cufftHandle h = plan.t3_plan(R);
+  GPN_CUFFT3(cufftSetStream(h, st));
+  if (plan.precision == GP_FP32)
+    GPN_CUFFT3(cufftExecC2C(h, (cufftComplex*)in, (cufftComplex*)out, sign));
+  else
+    GPN_CUFFT3(cufftExecZ2Z(h, (cufftDoubleComplex*)in, (cufftDoubleComplex*)out, sign));
+}
+
+void rows_any(Plan& plan, bool inv, void* cols, int R, cudaStream_t st) {
+  if (plan.precision == GP_DF64)
+    rows_run<dd>(plan, inv, cols, R, st);
+  else if (plan.precision == GP_FP32)
+    rows_run<float>(plan, inv, cols, R, st);
+  else
+    rows_run<double>(plan, inv, cols, R, st);
 }
 }  // namespace
 
@@ -858,24 +927,9 @@ cufftHandle Plan::t3_plan(int R) {
 }
 
 void tr3_forward(Plan& plan, int R, cudaStream_t st) {
-  if (plan.precision == GP_DF64) {
-    rows_run<dd>(plan, false, plan.fx, R, st);
-    prof_mark(plan, 0, st);
-    cols_run_dd(plan, false, plan.fx, plan.fy, R, st);
-    return;
-  }
-  cufftHandle h = plan.t3_plan(R);
-  if (plan.precision == GP_FP32) {
-    rows_run<float>(plan, false, plan.fx, R, st);
-    prof_mark(plan, 0, st);
-    GPN_CUFFT3(cufftSetStream(h, st));
-    GPN_CUFFT3(cufftExecC2C(h, (cufftComplex*)plan.fx, (cufftComplex*)plan.fy, CUFFT_FORWARD));
-  } else {
-    rows_run<double>(plan, false, plan.fx, R, st);
-    prof_mark(plan, 0, st);
-    GPN_CUFFT3(cufftSetStream(h, st));
-    GPN_CUFFT3(cufftExecZ2Z(h, (cufftDoubleComplex*)plan.fx, (cufftDoubleComplex*)plan.fy, CUFFT_FORWARD));
-  }
+  rows_any(plan, false, plan.fx, R, st);
+  prof_mark(plan, 0, st);
+  columns(plan, CUFFT_FORWARD, plan.fx, plan.fy, R, st);
 }
 
 void tr3_diag(Plan& plan, int R, cudaStream_t st) {
@@ -896,23 +950,9 @@ void tr3_diag(Plan& plan, int R, cudaStream_t st) {
 }
 
 void tr3_inverse(Plan& plan, int R, cudaStream_t st) {
-  if (plan.precision == GP_DF64) {
-    cols_run_dd(plan, true, plan.fz, plan.fy, R, st);
-    prof_mark(plan, 1, st);
-    rows_run<dd>(plan, true, plan.fy, R, st);
-    return;
-  }
-  cufftHandle h = plan.t3_plan(R);
-  GPN_CUFFT3(cufftSetStream(h, st));
-  if (plan.precision == GP_FP32) {
-    GPN_CUFFT3(cufftExecC2C(h, (cufftComplex*)plan.fz, (cufftComplex*)plan.fy, CUFFT_INVERSE));
-    prof_mark(plan, 1, st);
-    rows_run<float>(plan, true, plan.fy, R, st);
-  } else {
-    GPN_CUFFT3(cufftExecZ2Z(h, (cufftDoubleComplex*)plan.fz, (cufftDoubleComplex*)plan.fy, CUFFT_INVERSE));
-    prof_mark(plan, 1, st);
-    rows_run<double>(plan, true, plan.fy, R, st);
-  }
+  columns(plan, CUFFT_INVERSE, plan.fz, plan.fy, R, st);
+  prof_mark(plan, 1, st);
+  rows_any(plan, true, plan.fy, R, st);
 }
 
 }  // namespace gpn

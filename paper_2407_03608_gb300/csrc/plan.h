@@ -191,7 +191,7 @@ struct Plan {
   int line_cell0 = 0, line_cell1 = 0;   // cells the points reach
   // tables that only speed a plan up and are left out where it fits max_bytes (or the device)
   // without them alone: the 1-D kernels' (then the tiled spread and the row or cuFFT transforms
-  // run) and the 3-D box's buffers
+  // run), the 2-D column transforms' (then cuFFT's run) and the 3-D box's buffers
   bool spare = true;
   bool line = false;
   void* line_spec = nullptr;            // [r][C][nf/2] complex
@@ -351,6 +351,7 @@ void rowfft_diag(Plan& plan, int R, cudaStream_t st);
 void rowfft_inverse(Plan& plan, int R, cudaStream_t st);
 // transposed pruned transforms (d = 2, nf = 2^a)
 bool tr3_supported(int d, long long nf, int precision);
+bool own_cols(const Plan& plan);   // the plan's column transforms are the library's own
 void tr3_setup(Plan& plan);
 void tr3_forward(Plan& plan, int R, cudaStream_t st);
 void tr3_diag(Plan& plan, int R, cudaStream_t st);

@@ -1,6 +1,7 @@
-"""The 1-D line kernels, the 3-D box kernels, posterior means without binning and the short CG
-iteration at the sizes where they can go wrong: the smallest and largest transforms, odd radices,
-remainders of the tiles, channel counts on both sides of the kernels' groups.
+"""The 1-D line kernels, the 3-D box kernels, the 2-D column transforms, posterior means
+without binning and the short CG iteration at the sizes where they can go wrong: the smallest
+and largest transforms, odd radices, remainders of the tiles, channel counts on both sides of
+the kernels' groups.
 
 Bars: those stated for the same quantities elsewhere in the tests, relative l2 and max: the exact
 NUDFT 1e-9 (FP64 plans with a tight NUFFT tolerance) and 1e-4 (FP32); two routes through the same
@@ -71,6 +72,14 @@ def test_box_kernels(gpn, precision, nf, M, n_sigma, step3, R, n):
     if precision == "fp32" and nf % 4:
         pytest.skip("FP32 plans take grids of a multiple of 4 cells")
     check_matvec(gpn, 3, n, precision, R, nf=nf, M=M, n_sigma=n_sigma, step3=step3)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf,M,R", [(128, 20, 1), (256, 40, 2), (512, 30, 1), (1024, 30, 3), (2048, 20, 1), (4096, 20, 1),
+                                    (8192, 12, 1)])
+def test_column_kernels(gpn, precision, nf, M, R):
+    """Column transforms of every first-pass radix (and the lengths that stay with cuFFT)."""
+    check_matvec(gpn, 2, 301, precision, R, nf=nf, M=M, n_sigma=2, transform=3)
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
