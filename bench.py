@@ -157,6 +157,14 @@ def workload(args):
     return w
 
 
+def own_columns(info):
+    """Whether a 2-D plan's column transforms are the library's own (csrc/fft2d.cu, own_cols;
+    0 float64, 1 FP32, 2 float-float)."""
+    if info["precision"] == 2:
+        return True
+    return 256 <= info["nf"] <= (4096 if info["precision"] == 1 else 8192)
+
+
 def algorithmic_bytes(info, N, R, rs):
     """Algorithmic HBM bytes per launch of each matvec phase (reads + writes once).
 
@@ -175,9 +183,9 @@ def algorithmic_bytes(info, N, R, rs):
     out = {"spread": C * R * Gocc * rs + pts + N * R * 8, "interp": C * R * Gocc * rs + pts + 2 * N * R * 8}
     if info["transform"] == 3:
         rows = C * R * (Gocc * rs + (M + 1) * ext * cp)
-        if info["precision"] == 2:
-            # the float-float column kernels read the rows that can be nonzero and write
-            # the rows the next stage reads: the data extent and the 2M + 1 kept modes
+        if own_columns(info):
+            # the column kernels read the rows that can be nonzero and write the rows the
+            # next stage reads: the data extent and the 2M + 1 kept modes
             cols = C * R * (M + 1) * (ext + 2 * M + 1) * cp
         else:
             cols = 2 * C * R * (M + 1) * nf * cp
@@ -217,7 +225,7 @@ PHASES = ["spread", "fft_fwd", "diag", "fft_inv", "interp"]
 def launches_per_step(own_columns: bool) -> int:
     """Our kernels in one CG iteration on the 2-D path: spread, forward rows, step 3, inverse
     rows, interp, and the CG kernels (dot partial + final, update_xr + dot final, update_p,
-    roll, check); the two column transforms are cuFFT's, or ours on float-float plans."""
+    roll, check); the two column transforms are ours or cuFFT's (own_columns)."""
     return 5 + 7 + (2 if own_columns else 0)
 
 
@@ -251,9 +259,9 @@ def alu_ops(info, R):
       the real split (two complex sums, a complex product, two normalised sums and two
       halvings: 102) and the split twiddle (a complex product, shared by the RB rows of a
       block);
-    rows_inv: the merge of each mode pair (two merges of 88 and one twiddle of 34 per pair
-      of the nf/2 + 1 modes: the second twiddle is minus the conjugate of the first), then
-      the nf/2-point FFT;
+    rows_inv: the merge of each mode pair (per pair of the nf/2 + 1 modes two complex sums,
+      one complex product, two normalised complex sums: 110, and one twiddle of 34), then the
+      nf/2-point FFT;
     cols_*: one nf-point complex FFT per kept mode column."""
     nf, M, W = info["nf"], info["M"], info["kernel_width"]
     C = info["n_sigma"] + 1
@@ -262,7 +270,7 @@ def alu_ops(info, R):
     l2 = int(round(math.log2(nf // 2)))
     rows = C * R * ext
     fwd = rows * (ff_fft_ops(l2) + (M + 1) * 102) + C * R * (ext // 2) * (M + 1) * 34
-    inv = rows * (ff_fft_ops(l2) + (nf // 4 + 1) * (2 * 88 + 34))
+    inv = rows * (ff_fft_ops(l2) + (nf // 4 + 1) * (110 + 34))
     cols = C * R * (M + 1) * ff_fft_ops(int(round(math.log2(nf))))
     return {"rows_fwd": fwd, "rows_inv": inv, "cols_fwd": cols, "cols_inv": cols}
 
@@ -340,7 +348,7 @@ def _phases(abi, pl, y, x, eta2, k):
 
 def _kernel_ms(phase_ms, rows_ms, own_columns):
     """Our own kernels: spread, step 3, interp, the row kernels inside the transform phases,
-    and (float-float plans) the column kernels, the rest of those phases."""
+    and (own_columns) the column kernels, the rest of those phases."""
     km = {"spread": phase_ms[0], "diag": phase_ms[2], "interp": phase_ms[4]}
     for name, ms in zip(("rows_fwd", "rows_inv"), rows_ms):
         if ms > 0:
@@ -418,14 +426,14 @@ def run_ours(args, ws, rank, local):
         return {"rel_l2": float(torch.linalg.norm(u - v) / torch.linalg.norm(v)),
                 "rel_max": float((u - v).abs().max() / v.abs().max())}
 
-    def leg(pl, pn, own_cols):
+    def leg(pl, pn):
         """Another precision on the same K~: the same K steps, its kernels' rooflines."""
         xx = torch.empty_like(y)
         _cg(abi, pl, 2, y, xx, eta2)
         ms_k, it_k = _timed_steps(abi, torch, pl, args.steps, y, xx, eta2, stream)
         ph, rw, _ = _phases(abi, pl, y, xx, eta2, min(args.steps, 5))
         ab_k = algorithmic_bytes(pl.info, N, 1, PRECISIONS[pn][2])
-        km = _kernel_ms(ph, rw, own_cols)
+        km = _kernel_ms(ph, rw, own_columns(pl.info))
         return {"value": round(N / (ms_k / it_k * 1e-3) / 1e6, 3), "ms_per_step": round(ms_k / it_k, 4),
                 "steps": it_k, "arith": PRECISIONS[pn][3],
                 "phase_ms": {PHASES[q]: round(ph[q], 4) for q in range(5)},
@@ -436,13 +444,13 @@ def run_ours(args, ws, rank, local):
         p64 = gpn.Plan(pts, s, l, nu=w.nu, eps=w.eps, precision=gpn.GP_FP64, **plan.matched_opts())
         o64 = p64.matvec(a)
         extra["matvec_err_vs_fp64_gpu"] = err_pair(out_main, o64)
-        extra["fp64_path"] = leg(p64, "fp64", False)
+        extra["fp64_path"] = leg(p64, "fp64")
     else:
         o64 = out_main
     # the mixed-precision FP32 path on the same K~
     if prec != gpn.GP_FP32:
         p32 = gpn.Plan(pts, s, l, nu=w.nu, eps=w.eps, precision=gpn.GP_FP32, **plan.matched_opts())
-        m32 = leg(p32, "fp32", False)
+        m32 = leg(p32, "fp32")
         m32["matvec_err_vs_fp64_gpu"] = err_pair(p32.matvec(a), o64)
         extra["mixed_fp32"] = m32
         p32.close()
@@ -451,7 +459,7 @@ def run_ours(args, ws, rank, local):
     out_sample = out_main.cpu().numpy()
 
     ab = algorithmic_bytes(info, N, 1, rs)
-    kern_ms = _kernel_ms(phase_ms, rows_ms, prec == gpn.GP_DF64)
+    kern_ms = _kernel_ms(phase_ms, rows_ms, own_columns(plan.info))
     dom = max(range(5), key=lambda q: phase_ms[q])
     dom_ours = max(kern_ms, key=kern_ms.get)
     traffic = MEASURED_TRAFFIC.get((w.name, dtype, w.eps), {})
@@ -483,7 +491,7 @@ def run_ours(args, ws, rank, local):
         "timing": dist_stats,
         "clocks": clocks,
         "e2e": e2e,
-        "gpu_launches": launches_per_step(prec == gpn.GP_DF64) * iters,
+        "gpu_launches": launches_per_step(own_columns(plan.info)) * iters,
     }
     result.update(extra)
     return result, w, out_sample, plan

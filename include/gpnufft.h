@@ -103,14 +103,20 @@ typedef struct gp_plan_opts {
                                library's own transforms over the box of cells the
                                plan's points and queries can reach, and from them to
                                the modes |n_a| <= M (then info.bytes_resident is well
-                               below gp_plan_params' estimate);
-                             2 pruned: custom shared-memory row FFTs keeping modes 0..M,
-                               cuFFT along the first axis (d <= 2, nf = 2^a);
+                               below gp_plan_params' estimate); d = 1 with nf = 2^a:
+                               the library's own split transforms;
+                             2 pruned (d <= 2, nf = 2^a): d = 2 custom shared-memory row
+                               FFTs keeping modes 0..M, cuFFT along the first axis;
+                               d = 1 the split transforms, or the row FFTs where the
+                               modes are few;
                              3 pruned, transposed (d = 2, nf = 2^a): custom row FFTs
-                               write columns of modes 0..M, cuFFT transforms each
-                               contiguous column, step 3 on the mode box only    */
+                               write columns of modes 0..M, each contiguous column is
+                               transformed (custom column FFTs, or cuFFT for very short
+                               ones and FP32 ones above 4096), step 3 on the mode box
+                               only                                              */
   int max_rhs;            /* largest R the plan will be called with (default 1)         */
-  long long max_bytes;    /* refuse plans whose resident device bytes exceed this (0 = no limit) */
+  long long max_bytes;    /* refuse plans whose resident device bytes exceed this (0 = no limit);
+                             tables that only make a plan faster are left out first      */
   int step3;              /* step (3) of Sec. 4.2:
                              0 auto: 1 unless the tensor alone would break max_bytes or
                                the free device memory, then 2;
@@ -270,7 +276,9 @@ int gp_cg_solve_refined(gp_plan_t plan_lo, gp_plan_t plan_hi, const double* y, d
  *   xq : Nq x d row-major; field_aq, field_bq : the two scale fields at the queries, in
  *        the plan's param_mode.  Queries must lie in the plan box and their sigma in
  *        [sigma_lo, sigma_hi] (gp_plan_info), else GP_EINVAL.
- *   mu : Nq float64. */
+ *   mu : Nq float64.
+ * The plan keeps the call's workspace for the next one (at most 64 MiB, and within max_bytes;
+ * it counts in info.bytes_resident), larger ones are allocated for the call. */
 int gp_posterior_mean(gp_plan_t plan, const double* alpha, const double* xq, long long Nq, const double* field_aq,
                       const double* field_bq, double* mu, void* cuda_stream);
 
@@ -331,8 +339,8 @@ int gp_profile_read(gp_plan_t plan, double* ms_avg, long long* count);
 /* The library's own row kernels inside the two transform phases of the same
  * recording (App. D: the row half of each 2-D FFT), as average milliseconds per
  * matvec: ms_avg[0] of phase [1] (forward) and ms_avg[1] of phase [3] (inverse).
- * The rest of each phase is cuFFT (the column transforms in d = 2).  Plans whose
- * transforms are cuFFT alone give 0; the 1-D row transforms, which use no cuFFT,
+ * The rest of each phase is the column transforms (d = 2).  Plans whose transforms
+ * are cuFFT alone or the 3-D box's give 0; the 1-D transforms, which use no cuFFT,
  * give the whole phase.  It waits for the last recorded matvec.
  * Errors: GP_EINVAL, GP_ECUDA. */
 int gp_profile_read_rows(gp_plan_t plan, double* ms_avg);

@@ -181,7 +181,7 @@ cufftHandle Plan::inv_plan(int R) {
 }
 
 void run_fft_forward(Plan& plan, int R, cudaStream_t st) {
-  // the row-kernel paths mark between their rows and cuFFT's columns themselves
+  // the row-kernel paths mark between their rows and columns themselves
   if (plan.tr3) return tr3_forward(plan, R, st);
   if (plan.line) {
     line_forward(plan, R, st);

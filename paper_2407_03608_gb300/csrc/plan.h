@@ -75,8 +75,8 @@ struct PhaseProfile {
   bool pending = false;
   bool in_matvec = false;   // between the first and last event of a recorded matvec
   cudaEvent_t ev[6];
-  // mid[0]: the forward phase's own row kernels end and its cuFFT part begins;
-  // mid[1]: the inverse phase's cuFFT part ends and its own row kernels begin
+  // mid[0]: the forward phase's row kernels end and its columns begin;
+  // mid[1]: the inverse phase's columns end and its row kernels begin
   cudaEvent_t mid[2];
   double acc[5] = {0, 0, 0, 0, 0};
   double acc_rows[2] = {0, 0};   // ms in the transform phases' own row kernels

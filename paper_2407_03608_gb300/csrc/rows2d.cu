@@ -8,6 +8,12 @@
 // is one whole 32-byte sector (with one pair, half of every sector is fetched for nothing:
 // measured 1.58 ms against 1.19 ms at nf = 8192), and loads several pairs of modes before it
 // uses the first, merging them into the half-length input on their way to shared memory.
+//
+// Bound: latency of the sector-sized column reads and the shared-memory exchanges (neither fewer
+// instructions nor more warps helped further: radix 8 at 64 registers and 32 warps 1.31 ms).
+// Against one row at a time: nf 2048 with 30 grids .288 -> .169 ms, nf 4096 1.94 -> 1.80 (64
+// grids), nf 8192 1.22 -> 1.21 (9 grids).  The forward rows in this form: 1.06 -> 1.17 ms at
+// nf = 8192, so they stay as they were.
 #include "fft2d.h"
 #include "fft_mixed.h"
 

@@ -17,7 +17,10 @@
 // FP32 sums are kept as pairs of channels, one packed multiply-add each (the same roundings).
 //
 // Bound: FP32 issue.  A point meets 54 (warp, group) cells sets at width 9 (RPW = 4), 42 % of
-// whose multiply-adds fall inside its support.
+// whose multiply-adds fall inside its support.  2e6 points in FP32, ms, the general kernel
+// (integer shared-memory atomics) -> here: 8 channels 20.1 -> 4.80, 10 channels 28.4 -> 6.05;
+// without the packed pairs and with one candidate a thread and scan 5.21 and 7.24.  Float64, 2e4
+// points, 7 channels: 2.31 -> 1.71.
 #include <algorithm>
 #include <type_traits>
 
