@@ -176,7 +176,7 @@ void interp_impl(const Plan& plan, const PointSet& qs, double* mu, cudaStream_t 
 // (2-D float64: the kernel values of an unbinned query are not tabulated, and their float64
 // arithmetic sets the line.)
 bool query_unbinned(const Plan& plan, long long n) {
-  if (plan.geom.d == 1) return true;
+  if (plan.geom.d == 1) return n < (1ll << 31);   // (more are refused by the binning, as ever)
   if (plan.geom.d == 3) return plan.box3.on && n <= (1 << 18);
   return n <= (plan.precision == GP_FP64 ? 1 << 17 : 1 << 18);
 }

@@ -53,6 +53,7 @@ def check_matvec(gpn, d, n, precision, R, **kw):
     (65536, 400, 9, 4, 1000),    # few modes of a long transform (FP64: the general row kernels)
     (65536, 11000, 3, 1, 300),
     (1 << 20, 300, 3, 1, 257),   # FP32: the longest transform
+    (512, 60, 31, 2, 200),       # the most channels
 ])
 def test_line_kernels(gpn, precision, nf, M, n_sigma, R, n):
     check_matvec(gpn, 1, n, precision, R, nf=nf, M=M, n_sigma=n_sigma)
@@ -67,6 +68,8 @@ def test_line_kernels(gpn, precision, nf, M, n_sigma, R, n):
     (128, 8, 15, 1, 1, 100),     # 16 channels
     (432, 5, 2, 1, 1, 70),       # passes held and not held in registers
     (864, 4, 1, 2, 1, 65),       # the most passes
+    (64, 8, 31, 1, 1, 60),       # the most channels
+    (64, 6, 31, 2, 1, 60),
 ])
 def test_box_kernels(gpn, precision, nf, M, n_sigma, step3, R, n):
     if precision == "fp32" and nf % 4:
@@ -160,3 +163,22 @@ def test_1d_plan_without_spare_tables(gpn, precision):
     a = gpinputs.random_alpha(700, 2, seed=95)
     for plan in (full, lean):
         assert rel(plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy(), ktilde.matvec(w.points, wp, sig, a, p)) <= BAR[precision]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("d,step3", [(1, 1), (2, 1), (3, 1), (3, 2)])
+def test_one_channel(gpn, precision, d, step3):
+    """A constant length scale needs one channel: product and posterior mean against the dense
+    kernel.  The plan is asked for 1e-4, FP32 rounding is below that; the bar is ten times it."""
+    n = 300
+    w = small_case(d, n, 0)
+    s, l = np.ones(n), np.full(n, 0.15)
+    plan = gpn.Plan(w.points, s, l, nu=2.5, eps=1e-4, max_rhs=2, step3=step3,
+                    precision=gpn.GP_FP64 if precision == "fp64" else gpn.GP_FP32)
+    assert plan.info["n_sigma"] == 0
+    wp, sig = okern.paper_fields(s, l, d)
+    K = okern.kernel_dense(w.points, wp, sig, 2.5)
+    a = gpinputs.random_alpha(n, 2, seed=99)
+    assert rel(plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy(), K @ a) <= 1e-3
+    mu = plan.posterior_mean(torch.from_numpy(a[:, 0].copy()).cuda(), *(torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (w.points, s, l)))
+    assert rel(mu.cpu().numpy(), K @ a[:, 0]) <= 1e-3
