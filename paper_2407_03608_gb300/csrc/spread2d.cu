@@ -72,7 +72,7 @@ struct Spread2Args {
 
 // NC: channels held in registers (C itself up to 16, else 32 with the extra ones zero).
 template <typename T, int NC, int RPW>
-__device__ __forceinline__ void spread2d_tile(const Spread2Args<T>& a) {
+__global__ void __launch_bounds__(256) k_spread2d(Spread2Args<T> a) {
   constexpr int TY = kWarps * RPW;
   constexpr int WP = wk_pitch<T>(NC);
   constexpr int VW = (int)(16 / sizeof(T));
@@ -281,32 +281,17 @@ __device__ __forceinline__ void spread2d_tile(const Spread2Args<T>& a) {
   }
 }
 
-template <typename T, int NC, int RPW>
-__global__ void __launch_bounds__(256) k_spread2d(Spread2Args<T> a) {
-  spread2d_tile<T, NC, RPW>(a);
-}
-// held to 128 registers, for two CTAs an SM (the bound changes the registers of every type, so
-// it has its own entry)
-template <int NC>
-__global__ void __launch_bounds__(256, 2) k_spread2d_dd4(Spread2Args<dd> a) {
-  spread2d_tile<dd, NC, 4>(a);
-}
-
 // channels held in registers: C itself up to 16, else 32
 constexpr int reg_channels(int C) { return C <= 16 ? C : 32; }
 
 template <typename T>
 constexpr int rows_per_warp(int nc) {
-  // float64 and float-float sums take two registers each: two rows a warp; FP32 keeps four
+  // float64 and float-float sums take two registers each: two rows a warp (four rows of
+  // float-float sums held 156 registers at 9 channels, one CTA an SM, and the spread ran
+  // 4.29 ms at the 2-D benchmark size against 3.14 ms with two rows and 80 registers);
+  // FP32 keeps four
   return (sizeof(T) == 8 || nc > 16) ? 2 : 4;
 }
-
-// Float-float with up to 9 channels: four rows a warp as well, where two CTAs' tables fit an SM.
-// The 1e6-point plan (9 channels, width 11): 3.19 ms with two rows (80 registers, three CTAs),
-// 2.97 with four held to 128 registers (24 bytes spilled), 4.29 with four and 156 registers (one
-// CTA).
-constexpr int kDD4Channels = 9;
-constexpr size_t kDD4Smem = 112 * 1024;
 
 size_t smem_bytes(size_t rs, int nc, int rpw, int w) {
   const int wp = rs == 4 ? wk_pitch<float>(nc) : wk_pitch<double>(nc);
@@ -314,15 +299,7 @@ size_t smem_bytes(size_t rs, int nc, int rpw, int w) {
 }
 
 template <typename T, int NC>
-void launch(const Spread2Args<T>& a, dim3 grid, int rows, cudaStream_t st) {
-  if constexpr (is_dd<T>::value && NC <= kDD4Channels) {
-    if (rows == 4 * kWarps) {
-      const size_t smem = smem_bytes(sizeof(T), NC, 4, a.width);
-      GPN_CUDA(cudaFuncSetAttribute(k_spread2d_dd4<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k_spread2d_dd4<NC><<<grid, kWarps * 32, smem, st>>>(a);
-      return;
-    }
-  }
+void launch(const Spread2Args<T>& a, dim3 grid, cudaStream_t st) {
   constexpr int RPW = rows_per_warp<T>(NC);
   const size_t smem = smem_bytes(sizeof(T), NC, RPW, a.width);
   GPN_CUDA(cudaFuncSetAttribute(k_spread2d<T, NC, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -330,14 +307,14 @@ void launch(const Spread2Args<T>& a, dim3 grid, int rows, cudaStream_t st) {
 }
 
 template <typename T, int NC>
-void dispatch(const Spread2Args<T>& a, dim3 grid, int rows, cudaStream_t st) {
+void dispatch(const Spread2Args<T>& a, dim3 grid, cudaStream_t st) {
   if constexpr (NC > 16) {
-    launch<T, 32>(a, grid, rows, st);
+    launch<T, 32>(a, grid, st);
   } else {
     if (a.C == NC)
-      launch<T, NC>(a, grid, rows, st);
+      launch<T, NC>(a, grid, st);
     else
-      dispatch<T, NC + 1>(a, grid, rows, st);
+      dispatch<T, NC + 1>(a, grid, st);
   }
 }
 
@@ -370,31 +347,27 @@ void impl(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st) {
   a.inv_halfw = (T)(2.0 / g.width);
   a.C = g.C;
   dim3 grid((unsigned)plan.n_sp2_tiles, (unsigned)R);
-  dispatch<T, 1>(a, grid, spread2d_rows(plan), st);
+  dispatch<T, 1>(a, grid, st);
   GPN_CUDA(cudaGetLastError());
 }
 
 }  // namespace
 
-// the bin rows a tile's candidates come from
-static int bin_rows(const Plan& plan, int rows) { return (rows + plan.geom.width - 2) / plan.geom.tile + 2; }
-
 int spread2d_rows(const Plan& plan) {
   const int nc = reg_channels(plan.geom.C);
-  if (plan.precision == GP_DF64) {
-    const bool four = nc <= kDD4Channels && bin_rows(plan, 4 * kWarps) <= kMaxRanges &&
-                      smem_bytes(sizeof(dd), nc, 4, plan.geom.width) <= kDD4Smem;
-    return kWarps * (four ? 4 : rows_per_warp<dd>(nc));
-  }
-  return kWarps * (plan.precision == GP_FP32 ? rows_per_warp<float>(nc) : rows_per_warp<double>(nc));
+  const int rpw = plan.precision == GP_FP32   ? rows_per_warp<float>(nc)
+                  : plan.precision == GP_DF64 ? rows_per_warp<dd>(nc)
+                                              : rows_per_warp<double>(nc);
+  return kWarps * rpw;
 }
 
 bool spread2d_supported(const Plan& plan) {
   const GridGeom& g = plan.geom;
   if (g.d != 2 || g.width > kMaxW || g.C > kMaxChannels) return false;
   const int TY = spread2d_rows(plan);
+  const int bin_rows = (TY + g.width - 2) / g.tile + 2;
   const int nc = reg_channels(g.C);
-  return bin_rows(plan, TY) <= kMaxRanges && smem_bytes(plan.real_size, nc, TY / kWarps, g.width) <= 200 * 1024;
+  return bin_rows <= kMaxRanges && smem_bytes(plan.real_size, nc, TY / kWarps, g.width) <= 200 * 1024;
 }
 
 // Tiles whose candidate bins hold at least one point; the others stay zero.

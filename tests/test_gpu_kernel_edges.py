@@ -85,25 +85,6 @@ def test_column_kernels(gpn, precision, nf, M, R):
     check_matvec(gpn, 2, 301, precision, R, nf=nf, M=M, n_sigma=2, transform=3)
 
 
-@pytest.mark.parametrize("tol,n_sigma,tile", [(1e-11, 8, None), (1e-11, 9, None), (1e-3, 1, 4), (1e-11, 2, 16)])
-def test_float_float_spread_rows(gpn, tol, n_sigma, tile):
-    """Float-float spreads of four rows a warp (up to 9 channels), of two (10 channels; tiles so
-    small that four rows would meet too many bin rows).  At the loose NUFFT tolerance against
-    the float64 plan of the same K~, at the tight one against the oracle."""
-    w = gpinputs.config_2d(700, 1.5)
-    wp, sig = okern.paper_fields(w.s, w.l, 2)
-    p = explicit_params(2, 1.5, sig, w.points, n_t=12, n_sigma=n_sigma, M=30)
-    kw = dict(nu=1.5, eps=1e-6, nufft_tol=tol, max_rhs=2, nf=256, **({"tile": tile} if tile else {}), **plan_kwargs(p))
-    plan = gpn.Plan(w.points, w.s, w.l, precision=gpn.GP_DF64, **kw)
-    a = gpinputs.random_alpha(700, 2, seed=97)
-    got = plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy()
-    if tol > 1e-9:
-        ref = gpn.Plan(w.points, w.s, w.l, precision=gpn.GP_FP64, transform=3, **kw).matvec(torch.from_numpy(a).cuda()).cpu().numpy()
-    else:
-        ref = ktilde.matvec(w.points, wp, sig, a, p)
-    assert rel(got, ref) <= 1e-9
-
-
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("d", [1, 2, 3])
 def test_posterior_mean_with_and_without_binning(gpn, precision, d):
