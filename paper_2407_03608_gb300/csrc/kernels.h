@@ -146,8 +146,11 @@ __device__ __forceinline__ double to_f64(T v) {
 // Chebyshev-Lobatto nodes (weights (-1)^k, halved at both ends) with numerator and denominator
 // multiplied by prod_j (sigma - sigma_j): P_k = b_k prod_{j != k} (sigma - sigma_j) / sum of the
 // same, 4 C products and one division instead of 2 C divisions (float64 divisions made the
-// weights the largest kernel of a posterior mean), and exact at a node.  The differences are
-// scaled by the interval, so that the products of up to 31 of them stay in range.
+// weights the largest kernel of a posterior mean).  The differences are scaled by the interval,
+// so that the products of up to 31 of them stay in range.  A sigma that is a node has weight one
+// there: nodes may round to the same value (an interval of a few ulps, or of no width at all when
+// n_sigma >= 1 is asked for on a constant scale), and every product above then holds a zero.  On
+// an interval of no width any one node carries the weight, whatever the rounding of sigma.
 struct ChebArgs {
   double nodes[kMaxChannels];
   double bary[kMaxChannels];
@@ -158,11 +161,15 @@ __device__ __forceinline__ void cheb_weights(double w, double s, const ChebArgs&
   // x^(-d/2) by a square root and a division (pow costs several times the rest of the weights)
   const double x = 6.283185307179586476925286766559 * s * s;
   const double pre = w / (cb.d == 1 ? sqrt(x) : cb.d == 2 ? x : x * sqrt(x));
-  if (cb.C == 1) {
-    out[0] = pre;
+  const double span = fabs(cb.nodes[cb.C - 1] - cb.nodes[0]);
+  int hit = span > 0.0 ? -1 : 0;
+  for (int k = 0; k < cb.C; ++k)
+    if (s == cb.nodes[k]) hit = k;
+  if (hit >= 0) {
+    for (int k = 0; k < cb.C; ++k) out[k] = k == hit ? pre : 0.0;
     return;
   }
-  const double inv = 1.0 / fabs(cb.nodes[cb.C - 1] - cb.nodes[0]);
+  const double inv = 1.0 / span;
   double run = 1.0, den = 0.0;
   for (int k = 0; k < cb.C; ++k) {   // products of the differences before k ...
     out[k] = cb.bary[k] * run;

@@ -69,8 +69,7 @@ struct QueryArgs {
   double half_w;
   double sig_lo;
   double sig_hi;
-  double nodes[kMaxChannels];
-  double bary[kMaxChannels];
+  ChebArgs cb;         // channels and their nodes
   int C;
   const T* grid;       // inverse-transformed fine grids, channel k at k * G
   GridView v;            // layout of the grid
@@ -165,26 +164,12 @@ __global__ void __launch_bounds__(256) k_query_interp(QueryArgs<T> a) {
       }
     }
     if (lane == 0) {
-      // w_k = w (2 pi sigma^2)^(-d/2) P_k(sigma), P_k barycentric on the Chebyshev-Lobatto nodes
-      const double pre = w * pow(kTwoPi * s * s, -0.5 * D);
-      int hit = -1;
-      for (int k = 0; k < a.C; ++k)
-        if (s == a.nodes[k]) hit = k;
-      double den = 0.0;
-      if (hit < 0 && a.C > 1)
-        for (int k = 0; k < a.C; ++k) den += a.bary[k] / (s - a.nodes[k]);
+      double wk[kMaxChannels];
+      cheb_weights(w, s, a.cb, wk);
       double res = 0.0;
 #pragma unroll
-      for (int k = 0; k < CMAX; ++k) {
-        if (k < a.C) {
-          double wk;
-          if (hit >= 0 || a.C == 1)
-            wk = (k == hit || a.C == 1) ? pre : 0.0;
-          else
-            wk = pre * (a.bary[k] / (s - a.nodes[k])) / den;
-          res += (double)(T)wk * (double)acc[k];
-        }
-      }
+      for (int k = 0; k < CMAX; ++k)
+        if (k < a.C) res += (double)(T)wk[k] * (double)acc[k];
       a.mu[qi] = res;
     }
   }
@@ -223,10 +208,11 @@ void query_impl(Plan& plan, const double* x, const double* fa, const double* fb,
   a.half_w = 0.5 * h.width;
   a.sig_lo = h.sig_lo;
   a.sig_hi = h.sig_hi;
-  a.C = g.C;
+  a.C = a.cb.C = g.C;
+  a.cb.d = h.d;
   for (int k = 0; k < g.C; ++k) {
-    a.nodes[k] = plan.tb.nodes[k];
-    a.bary[k] = plan.tb.bary[k];
+    a.cb.nodes[k] = plan.tb.nodes[k];
+    a.cb.bary[k] = plan.tb.bary[k];
   }
   a.grid = (const T*)plan.grid_out;
   a.v = plan.view;

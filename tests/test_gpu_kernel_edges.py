@@ -163,3 +163,31 @@ def test_one_channel(gpn, precision, d, step3):
     assert rel(plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy(), K @ a) <= 1e-3
     mu = plan.posterior_mean(torch.from_numpy(a[:, 0].copy()).cuda(), *(torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (w.points, s, l)))
     assert rel(mu.cpu().numpy(), K @ a[:, 0]) <= 1e-3
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("d,step3", [(1, 1), (2, 1), (3, 1), (3, 2)])
+@pytest.mark.parametrize("n_sigma,width", [(1, 0.0), (4, 0.0), (31, 0.0), (31, 2.3e-14)])
+def test_coincident_nodes(gpn, precision, d, step3, n_sigma, width):
+    """More channels than a constant length scale needs: all Chebyshev nodes fall on one value
+    (or, with an interval of that relative width, some of them do), and one of them carries the
+    weight, so product and both posterior means are the one-channel plan's (that plan against
+    the dense kernel: test_one_channel)."""
+    n = 300
+    w = small_case(d, n, 0)
+    s, l = np.ones(n), np.full(n, 0.15)
+    kw = dict(nu=2.5, eps=1e-4, max_rhs=2, step3=step3, precision=gpn.GP_FP64 if precision == "fp64" else gpn.GP_FP32)
+    one = gpn.Plan(w.points, s, l, **kw)
+    sigma = 0.15 * 0.70710678118654752440
+    plan = gpn.Plan(w.points, s, l, **kw, **{**one.matched_opts(), "n_sigma": n_sigma, "sigma_lo": sigma,
+                                             "sigma_hi": sigma * (1.0 + width)})
+    assert plan.info["n_sigma"] == n_sigma and one.info["n_sigma"] == 0
+    a = torch.from_numpy(gpinputs.random_alpha(n, 2, seed=97)).cuda()
+    assert rel(plan.matvec(a).cpu().numpy(), one.matvec(a).cpu().numpy()) <= SAME[precision]
+    al = a[:, 0].contiguous()
+    dev = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (w.points, s, l)]
+    ref = one.posterior_mean(al, *dev).cpu().numpy()
+    assert rel(plan.posterior_mean(al, *dev).cpu().numpy(), ref) <= SAME[precision]
+    mu = torch.empty(n, dtype=torch.float64, device="cuda")
+    gpn.abi.gp_posterior_mean_noalloc(plan.handle, al, *dev, mu)
+    assert rel(mu.cpu().numpy(), ref) <= SAME[precision]
