@@ -14,13 +14,19 @@
 // The order, and so the summation order, is fixed (results are reproducible bit for bit).
 // Every grid value is written once; tiles no point can reach are never launched and stay zero.
 //
-// FP32 sums are kept as pairs of channels, one packed multiply-add each (the same roundings).
+// FP32 sums are kept as pairs of channels, one packed multiply-add each (the same roundings), and
+// in two words: every kFold list steps the running sum joins the total by TwoSum (ff64.h), and its
+// rounding error starts the next running sum.  So a cell's error is that of kFold additions
+// however many points reach it.  Relative l2 error of an FP32 product to the float64 plan on the
+// same grid, 2e5 points of one sign in a tenth of the box (8600 contributions a cell): 1.05e-6 with
+// the general kernel's fixed-point sums, 7.7e-7 here, 7.9e-6 with one word a sum; 2e6 uniform points
+// at nf 540 6.0e-7, 5.1e-7 and 5.2e-7.
 //
-// Bound: FP32 issue.  A point meets 54 (warp, group) cells sets at width 9 (RPW = 4), 42 % of
-// whose multiply-adds fall inside its support.  2e6 points in FP32, ms, the general kernel
-// (integer shared-memory atomics) -> here: 8 channels 20.1 -> 4.80, 10 channels 28.4 -> 6.05;
-// without the packed pairs and with one candidate a thread and scan 5.21 and 7.24.  Float64, 2e4
-// points, 7 channels: 2.31 -> 1.71.
+// Bound: FP32 issue, with the totals at two blocks an SM.  A point meets 54 (warp, group) sets of
+// cells at width 9 (RPW = 4), 42 % of whose multiply-adds fall inside its support.  2e6 points in
+// FP32, ms, the general kernel (integer shared-memory atomics) -> here: 8 channels 20.1 -> 6.32, 10
+// channels 28.4 -> 7.61 (one word a sum and three blocks an SM: 4.80 and 6.05, at the price above).
+// Folds every 16, 32, 64 steps: 6.56, 6.32, 6.20.  Float64, 2e4 points, 7 channels: 2.31 -> 1.71.
 #include <algorithm>
 #include <type_traits>
 
@@ -42,6 +48,7 @@ constexpr int kLists = kWarps * kGroups;
 constexpr int kSlots = kThreads;           // points a batch (one a thread fills its tables)
 constexpr int kScan = 4;                   // candidates a thread tests at a time
 constexpr int kQueue = (kScan + 1) * kSlots;   // a scan adds up to kScan kSlots to less than kSlots
+constexpr int kFold = 32;                  // list steps between folds into the totals (FP32)
 constexpr int kMaxRanges = 64;             // bin rows a tile's candidates can come from
 
 // per-slot shared tables (odd strides against bank conflicts); the row table has RPW - 1 zeros
@@ -73,13 +80,26 @@ struct Spread3Args {
   int C;
 };
 
+// tot + acc <- tot + acc exactly: the rounded sum, and what it left out
+__device__ __forceinline__ void fold(fft::f2& tot, fft::f2& acc) {
+  const fft::f2 s = fft::vadd(tot, acc), b = fft::vsub(s, tot);
+  acc = fft::vadd(fft::vsub(tot, fft::vsub(s, b)), fft::vsub(acc, b));
+  tot = s;
+}
+
+// Blocks an SM.  A lane's sums take 8 RPW NC bytes (one float64 or two FP32 words each); of the
+// registers left, 80 a thread do up to 160 bytes, 128 up to 320.
+template <typename T, int NC, int RPW>
+constexpr int kMinBlocks = 8 * RPW * NC <= 160 ? 3 : (8 * RPW * NC <= 320 || sizeof(T) == 8) ? 2 : 1;
+
 // NC: channels held in registers (C itself up to 16, else 32 with the extra ones zero)
 template <typename T, int NC, int RPW>
-__global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2)) k_spread3d(Spread3Args<T> a) {
+__global__ void __launch_bounds__(kThreads, (kMinBlocks<T, NC, RPW>)) k_spread3d(Spread3Args<T> a) {
   constexpr int TY = kBands * RPW, WP = wk_pitch<T>(NC), VW = (int)(16 / sizeof(T));
   // a sum: two channels (FP32) or one
   using Acc = typename std::conditional<sizeof(T) == 4, fft::f2, double>::type;
   constexpr int AL = fft::Elem<Acc>::lanes, NA = (NC + AL - 1) / AL;
+  constexpr bool kTwo = AL == 2;   // totals apart from the running sums
   using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
   const int W = a.width, PS = axis_stride(W), SY = row_stride(W, RPW), C = a.C, r = blockIdx.y;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -115,11 +135,14 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
   int total = 0;
   for (int q = 0; q < nr; ++q) total += s_rl[q];
 
-  Acc acc[RPW][NA];
+  Acc acc[RPW][NA], tot[kTwo ? RPW : 1][kTwo ? NA : 1];
 #pragma unroll
   for (int rr = 0; rr < RPW; ++rr)
 #pragma unroll
-    for (int k = 0; k < NA; ++k) acc[rr][k] = fft::vset<Acc>(T(0));
+    for (int k = 0; k < NA; ++k) {
+      acc[rr][k] = fft::vset<Acc>(T(0));
+      if constexpr (kTwo) tot[rr][k] = fft::vset<Acc>(T(0));
+    }
   const int grp = lane >> 3;
   const int xg = x0 + grp * kStrip + (lane & 7);                     // this lane's column
   const int zw = z0 + warp / kBands, rw0 = y0 + warp % kBands * RPW;  // the warp's plane, first row
@@ -256,32 +279,41 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
 #pragma unroll
     for (int q = 0; q < kGroups; ++q) steps = max(steps, s_len[warp * kGroups + q]);
     const unsigned char* lst = s_list + my_list * kSlots;
-    for (int j = 0; j < steps; ++j) {
-      const bool ok = j < len;
-      const int is = ok ? lst[j] : 0;
-      const int4 l0 = s_l0[is];
-      const int dx = xg - l0.z;
-      const bool in = ok && (unsigned)dx < (unsigned)W;
-      const T pxz = in ? s_psx[is * PS + dx] * s_psz[is * PS + (zw - l0.x)] : T(0);
-      Acc wk[WP / AL];
+    for (int j0 = 0; j0 < steps; j0 += kFold) {
+      const int j1 = min(j0 + kFold, steps);
+      for (int j = j0; j < j1; ++j) {
+        const bool ok = j < len;
+        const int is = ok ? lst[j] : 0;
+        const int4 l0 = s_l0[is];
+        const int dx = xg - l0.z;
+        const bool in = ok && (unsigned)dx < (unsigned)W;
+        const T pxz = in ? s_psx[is * PS + dx] * s_psz[is * PS + (zw - l0.x)] : T(0);
+        Acc wk[WP / AL];
 #pragma unroll
-      for (int v = 0; v < WP / VW; ++v) {
-        const V u = reinterpret_cast<const V*>(s_wk + is * WP)[v];
-        if constexpr (VW == 4) {
-          wk[2 * v] = {u.x, u.y};
-          wk[2 * v + 1] = {u.z, u.w};
-        } else {
-          wk[2 * v] = u.x;
-          wk[2 * v + 1] = u.y;
+        for (int v = 0; v < WP / VW; ++v) {
+          const V u = reinterpret_cast<const V*>(s_wk + is * WP)[v];
+          if constexpr (VW == 4) {
+            wk[2 * v] = {u.x, u.y};
+            wk[2 * v + 1] = {u.z, u.w};
+          } else {
+            wk[2 * v] = u.x;
+            wk[2 * v + 1] = u.y;
+          }
+        }
+        // rows of the band relative to the support: in [1 - RPW, W - 1] for list members
+        const T* pyr = s_psy + is * SY + (RPW - 1) + (ok ? rw0 - l0.y : 0);
+#pragma unroll
+        for (int rr = 0; rr < RPW; ++rr) {
+          const Acc v = fft::vset<Acc>(pxz * pyr[rr]);
+#pragma unroll
+          for (int k = 0; k < NA; ++k) acc[rr][k] = fft::vfma(v, wk[k], acc[rr][k]);
         }
       }
-      // rows of the band relative to the support: in [1 - RPW, W - 1] for list members
-      const T* pyr = s_psy + is * SY + (RPW - 1) + (ok ? rw0 - l0.y : 0);
+      if constexpr (kTwo) {
 #pragma unroll
-      for (int rr = 0; rr < RPW; ++rr) {
-        const Acc v = fft::vset<Acc>(pxz * pyr[rr]);
+        for (int rr = 0; rr < RPW; ++rr)
 #pragma unroll
-        for (int k = 0; k < NA; ++k) acc[rr][k] = fft::vfma(v, wk[k], acc[rr][k]);
+          for (int k = 0; k < NA; ++k) fold(tot[rr][k], acc[rr][k]);
       }
     }
     __syncthreads();  // slots, lists and counters are refilled by the next batch
@@ -299,14 +331,20 @@ __global__ void __launch_bounds__(kThreads, (RPW * NC * sizeof(T) <= 160 ? 3 : 2
       // whole sums: the pitch holds them (in FP32 it is even, a padding channel's weights are zero)
 #pragma unroll
       for (int k = 0; k < NA; ++k)
-        if (k * AL < C) *reinterpret_cast<Acc*>(o + k * AL) = acc[rr][k];
+        if (k * AL < C) {
+          if constexpr (kTwo) acc[rr][k] = fft::vadd(tot[rr][k], acc[rr][k]);
+          *reinterpret_cast<Acc*>(o + k * AL) = acc[rr][k];
+        }
     }
   }
 }
 
 constexpr int reg_channels(int C) { return C <= 16 ? C : 32; }
+// four rows a warp up to the channels whose sums leave two blocks an SM (12 channels, 5e5 points at
+// width 8: 1.66 ms with two rows, 2.09 with four and one block; 8 and 10 channels above: 6.58 and
+// 9.00 ms with two)
 template <typename T>
-constexpr int rows_per_warp(int nc) { return (sizeof(T) == 8 || nc > 16) ? 2 : 4; }
+constexpr int rows_per_warp(int nc) { return (sizeof(T) == 8 || nc > 10) ? 2 : 4; }
 
 size_t smem_bytes(size_t rs, int nc, int rpw, int w) {
   const int wp = rs == 4 ? wk_pitch<float>(nc) : wk_pitch<double>(nc);

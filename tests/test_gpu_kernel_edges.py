@@ -191,3 +191,28 @@ def test_coincident_nodes(gpn, precision, d, step3, n_sigma, width):
     mu = torch.empty(n, dtype=torch.float64, device="cuda")
     gpn.abi.gp_posterior_mean_noalloc(plan.handle, al, *dev, mu)
     assert rel(mu.cpu().numpy(), ref) <= SAME[precision]
+
+
+def fp32_against_fp64(gpn, x, s, l, alpha, nu, eps, call=lambda plan, a: plan.matvec(a), **kw):
+    """rel() of an FP32 plan to the float64 plan of the same K~ on the same fine grid with the same
+    spreading kernel: what FP32 rounds."""
+    lo = gpn.Plan(x, s, l, nu=nu, eps=eps, precision=gpn.GP_FP32, **kw)
+    hi = gpn.Plan(x, s, l, nu=nu, eps=eps, precision=gpn.GP_FP64, nf=lo.info["nf"], nufft_tol=lo.info["nufft_tol"],
+                  **{**lo.matched_opts(), **kw})
+    assert hi.info["kernel_width"] == lo.info["kernel_width"] and hi.info["nf"] == lo.info["nf"]
+    return lo, rel(call(lo, alpha).cpu().numpy(), call(hi, alpha).cpu().numpy())
+
+
+def test_fp32_spread_of_a_dense_cloud_3d(gpn):
+    """All points in a tenth of the box and of one sign: tens of thousands of contributions a grid
+    cell, whose FP32 sums must not lose what the plan's other roundings keep.  Bar: the six kernel
+    values a pair of points meets are each within beta 2^-24 of their value (their exponent, up to
+    beta, is an FP32 number), 5e-6 in all if these errors never cancelled."""
+    n = 600000
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = 0.45 + 0.1 * torch.rand((n, 3), generator=g, device="cuda", dtype=torch.float64)
+    s = 1.0 + 0.3 * x[:, 0]
+    l = 0.05 + 0.03 * x[:, 2]
+    alpha = 0.1 + torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
+    plan, e = fp32_against_fp64(gpn, x, s, l, alpha, 2.5, 1e-4, box_lo=[0.0] * 3, box_hi=[1.0] * 3)
+    assert e <= 6 * plan.info["kernel_beta"] * 2.0 ** -24, e
