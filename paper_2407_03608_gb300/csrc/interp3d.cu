@@ -3,17 +3,18 @@
 //
 // One warp a point, straight from the grid through L1: the channels are innermost, so one row
 // (z, y) of the support is width * Cp adjacent values, which the lanes read in S coalesced
-// loads.  A lane's position in that row fixes its cell x and channel k for the whole point, so
-// psi(x) w_k is formed once per lane and slot, and a row costs S loads and S + 1 multiply-adds.
-// Points come in bin order and a block takes consecutive ones, so the rows of neighbouring
-// points are served by L1.  Sums: a row's slots, then the rows of a plane weighted by psi(y),
-// then the planes weighted by psi(z); the 32 partial sums are added in float-float (FP32
-// plans) or float64.
+// loads; a row costs S loads and S multiply-adds.  A lane's position in the row fixes its cell x
+// and channel k for the whole point.  Points come in bin order and a block takes consecutive ones,
+// so the rows of neighbouring points are served by L1.  Sums: a slot's rows weighted by psi(y), the
+// planes weighted by psi(z); then the slots pass through shared memory, lane k sums channel k over
+// x, and the products w_k beta_k, whose signs alternate, are formed and added in float64.
 //
 // Bound: latency of the L1/L2 loads and issue (about 9 instructions a row).  On 2e6 points, ms:
 // the staged kernel of interp.cu 15.1 (8 channels, width 9, nf 512) and 26.7 (10, 9, nf 864); here
-// with 48 warps an SM 4.35 and 6.00, with 64 4.17 and 5.35.  Loads of two channels with packed
-// sums need 48 registers: 4.95; sorting the points finer than by bins changes nothing.
+// 4.27 and 5.61, 7 channels in float64 (2e5 points) 2.83.  What the loop's registers allow decides:
+// indexed rows instead of running pointers 4.98 and 6.25, unrolled by 3 as well 5.19 and 7.63, 48
+// warps an SM instead of 64 in that form 5.27 and 6.97.  Mixing the channels of a lane in one FP32 sum 4.17 and
+// 5.44.  Sorting the points finer than by bins changes nothing.
 #include <algorithm>
 
 #include "kernels.h"
@@ -37,24 +38,13 @@ struct Interp3Args {
   const T* grid;
   GridView v;
   int width, C, Cp;
+  int fold;              // half the power of two that holds C lanes
   T beta, inv_halfw;
   const double* alpha;   // sorted order (may be null)
   double shift;
   const double* dcorr;   // per-point addition to the shift (may be null)
   double* out;           // sorted order, n x R
 };
-
-__device__ __forceinline__ double warp_total(float v) {
-  dd s{v, 0.0f};
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += shfl_xor_val(s, o);
-  return (double)s;
-}
-__device__ __forceinline__ double warp_total(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // S: loads a row, ceil(width Cp / 32)
 template <typename T, int S>
@@ -64,12 +54,8 @@ __global__ void __launch_bounds__(32 * kWarps<S>, S <= 3 ? 4 : 1) k_interp3d(Int
   const T* grid = a.grid + r * a.v.rstride + lane;
   const double* alpha = a.alpha ? a.alpha + (size_t)r * a.n : nullptr;
   const int last = W * a.Cp - 32 * (S - 1);   // lanes of the last slot inside the row
-  int xs[S], ks[S];
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    xs[s] = (s * 32 + lane) / a.Cp;
-    ks[s] = (s * 32 + lane) - xs[s] * a.Cp;
-  }
+  __shared__ T s_sum[kWarps<S>][32 * S];   // a point's sums over z and y, in the order of a row
+  T* sums = s_sum[warp];
   const long long p1 = min(a.n, (long long)(blockIdx.x + 1) * kPointsPerBlock);
   for (long long p = (long long)blockIdx.x * kPointsPerBlock + warp; p < p1; p += kWarps<S>) {
     const int lz = a.l0[0][p] - a.v.lo[0], ly = a.l0[1][p] - a.v.lo[1], lx = a.l0[2][p] - a.v.lo[2];
@@ -79,32 +65,35 @@ __global__ void __launch_bounds__(32 * kWarps<S>, S <= 3 ? 4 : 1) k_interp3d(Int
       py = psi_at<T>(lane, a.xi[1][p], a.beta, a.inv_halfw);
       px = psi_at<T>(lane, a.xi[2][p], a.beta, a.inv_halfw);
     }
-    T v[S];
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const T q = shfl_val(px, xs[s] & 31);
-      const bool in = (s + 1 < S || lane < last) && ks[s] < a.C;
-      v[s] = in ? q * a.wk[p * a.C + ks[s]] : T(0);
-    }
     const T* g = grid + lz * s0 + ly * s1 + lx * a.v.stride[2];
-    T acc = T(0);
-    for (int z = 0; z < W; ++z) {
-      const T* gz = g + z * s0;
-      T plane = T(0);
-#pragma unroll 3
-      for (int y = 0; y < W; ++y) {
-        const T* gy = gz + y * s1;
-        T row = T(0);
+    T acc[S];
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const T u = (s + 1 < S || lane < last) ? __ldg(gy + 32 * s) : T(0);
-          row += v[s] * u;
-        }
-        plane += shfl_val(py, y) * row;
+    for (int s = 0; s < S; ++s) acc[s] = T(0);
+    for (int z = 0; z < W; ++z, g += s0) {
+      const T* gy = g;
+      T plane[S];
+#pragma unroll
+      for (int s = 0; s < S; ++s) plane[s] = T(0);
+#pragma unroll 4
+      for (int y = 0; y < W; ++y, gy += s1) {
+        const T wy = shfl_val(py, y);
+#pragma unroll
+        for (int s = 0; s < S; ++s) plane[s] += wy * ((s + 1 < S || lane < last) ? __ldg(gy + 32 * s) : T(0));
       }
-      acc += shfl_val(pz, z) * plane;
+      const T wz = shfl_val(pz, z);
+#pragma unroll
+      for (int s = 0; s < S; ++s) acc[s] += wz * plane[s];
     }
-    double res = warp_total(acc);
+    // lane k: the sum of channel k over x, times w_k in float64
+#pragma unroll
+    for (int s = 0; s < S; ++s) sums[32 * s + lane] = acc[s];
+    __syncwarp();
+    T beta = T(0);
+    const T* sk = sums + min(lane, a.C - 1);
+    for (int x = 0; x < W; ++x) beta += shfl_val(px, x) * sk[x * a.Cp];
+    double res = lane < a.C ? (double)a.wk[p * a.C + lane] * (double)beta : 0.0;
+    for (int o = a.fold; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+    __syncwarp();   // the next point's sums take the place of these
     if (lane == 0) {
       if (alpha) res += (a.dcorr ? a.shift + a.dcorr[p] : a.shift) * alpha[p];
       a.out[(size_t)r * a.n + p] = res;
@@ -136,6 +125,7 @@ void impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shi
   a.width = g.width;
   a.C = g.C;
   a.Cp = plan.box3.Cp;
+  for (int w = 1; w < g.C; w *= 2) a.fold = w;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);
   a.alpha = alpha_sorted;
