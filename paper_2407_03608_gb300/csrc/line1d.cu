@@ -226,15 +226,35 @@ __device__ __forceinline__ void finish_point(const Interp1Args<T>& a, long long 
   a.out[i] = res;
 }
 
-// sum + w b, the product exact: in float64, or for FP32 plans in float-float (conversions to
-// float64 run on its pipe, at a sixteenth of the FP32 rate)
+// The sum of exact products of FP32 values, in three words (about 72 bits): float64's precision on
+// the FP32 pipe (float64 sums run at a sixtieth of its rate, conversions at a sixteenth).
+struct Sum3 {
+  float a = 0.0f, b = 0.0f, c = 0.0f;
+
+  // + x + y, |y| below |x|'s last place or so
+  __device__ __forceinline__ void add(float x, float y) {
+    const dd s = two_sum(a, x), t = two_sum(b, s.lo), u = two_sum(t.hi, y);
+    a = s.hi;
+    b = u.hi;
+    c = ffops::add(c, ffops::add(t.lo, u.lo));
+  }
+  __device__ __forceinline__ explicit operator double() const { return (double)a + ((double)b + (double)c); }
+};
 __device__ __forceinline__ void add_product(double& sum, double w, double b) { sum += w * b; }
-__device__ __forceinline__ void add_product(dd& sum, float w, float b) {
+__device__ __forceinline__ void add_product(Sum3& sum, float w, float b) {
   const float p = ffops::mul(w, b);
-  sum += dd(p, ffops::fma(w, b, -p));
+  sum.add(p, ffops::fma(w, b, -p));
 }
 template <typename T>
-using SumOf = typename std::conditional<sizeof(T) == 4, dd, double>::type;
+using SumOf = typename std::conditional<sizeof(T) == 4, Sum3, double>::type;
+
+// + the same of lane ^ o
+__device__ __forceinline__ void add_lane(double& sum, int o) { sum += shfl_xor_val(sum, o); }
+__device__ __forceinline__ void add_lane(Sum3& sum, int o) {
+  const float x = shfl_xor_val(sum.a, o), y = shfl_xor_val(sum.b, o), z = shfl_xor_val(sum.c, o);
+  sum.add(x, y);
+  sum.c = ffops::add(sum.c, z);
+}
 
 // Sixteen lanes a point: lane j holds psi(j), lane k sums channel k (k + 16, ...) over the W
 // cells; the products w_k beta_k are added exactly (see add_product).  For point sets too small to fill the
@@ -248,7 +268,7 @@ __global__ void __launch_bounds__(128) k_interp1d_lanes(Interp1Args<T> a) {
   const T* g = a.grid + (size_t)r * a.C * a.nf + a.l0[q];
   T pj = T(0);
   if (gl < W) pj = a.psi ? a.psi[q * W + gl] : psi_at<T>(gl, a.xi[q], a.beta, a.inv_halfw);
-  SumOf<T> part(0.0);
+  SumOf<T> part{};
   for (int k0 = 0; k0 < a.C; k0 += 16) {
     const bool in = k0 + gl < a.C;
     const int k = in ? k0 + gl : a.C - 1;
@@ -263,7 +283,7 @@ __global__ void __launch_bounds__(128) k_interp1d_lanes(Interp1Args<T> a) {
     add_product(part, w, s);
   }
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) part += shfl_xor_val(part, o);
+  for (int o = 8; o > 0; o >>= 1) add_lane(part, o);
   if (on && gl == 0) finish_point(a, p, r, (double)part);
 }
 
@@ -299,7 +319,7 @@ __global__ void __launch_bounds__(kInterpThreads) k_interp1d(Interp1Args<T> a) {
   __syncthreads();
   if (!on) return;
   const T* w = s_wk + threadIdx.x * (C | 1);
-  SumOf<T> res(0.0);
+  SumOf<T> res{};
 #pragma unroll
   for (int k = 0; k < NC; ++k)
     if (NC <= 16 || k < C) add_product(res, w[k], acc[k]);
