@@ -414,7 +414,8 @@ PlanShape plan_shape(int d, long long N, double nu, double eps, const gp_plan_op
   const long long grid_pitch = full ? std::max(G, 2 * S) : G;
   const bool pow2 = (h.nf & (h.nf - 1)) == 0;
   const long long inv_work = (full && !pow2) ? CR * S * 2 * (long long)rs : 0;
-  ps.est_rest = 2 * CR * grid_pitch * (long long)rs + spectra + N * (long long)(d * (4 + rs) + 8 + C * rs) +
+  const long long arrays = 2 * CR * grid_pitch * (long long)rs + spectra;
+  ps.est_rest = arrays + N * (long long)(d * (4 + rs) + 8 + C * rs) +
                 (long long)N * max_rhs * 8 * 9 +
                 (psi_tabulated(d, o.precision, false) ? N * (long long)d * h.width * (long long)rs : 0);
   // step 3: the stored tensor A' (1) or the memory-lean form from per-dimension
@@ -435,13 +436,22 @@ PlanShape plan_shape(int d, long long N, double nu, double eps, const gp_plan_op
     ps.lean = over_budget || over_free;
   }
   ps.est = ps.est_rest + (ps.lean ? ps.lean_bytes : ps.a_bytes + inv_work);
+  ps.est_arrays = arrays + (ps.lean ? 0 : ps.a_bytes + inv_work);
   return ps;
 }
 
 namespace {
 
+// Device bytes of the large arrays of a 3-D plan over the box, and over the full grid.
+long long box3_bytes(const Plan& p, long long a_bytes) {
+  const long long grids = 2 * p.view.rstride * p.grid_rhs * (long long)p.real_size;
+  return grids + 16 * (p.box3.size_a + p.box3.size_b) * p.grid_rhs + (p.lean ? 0 : a_bytes);
+}
+
+// spare: with the tables that a plan can do without (Plan::spare).  lighter, when given, is set
+// before the first of the plan's own allocations: whether a plan without them would need less.
 Plan* build_plan(const double* points, long long N, int d, const double* fa, const double* fb, double nu, double eps,
-                 const gp_plan_opts& o, cudaStream_t st, bool spare) {
+                 const gp_plan_opts& o, cudaStream_t st, bool spare, bool* lighter) {
   GPN_CHECK(d >= 1 && d <= 3, GP_EINVAL, "d must be 1, 2 or 3");
   GPN_CHECK(N >= 1, GP_EINVAL, "N must be >= 1");
   GPN_CHECK(points && fa && fb, GP_EINVAL, "null points or fields");
@@ -508,6 +518,10 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   GPN_CHECK(o.max_bytes <= 0 || ps.est <= o.max_bytes, GP_ENOMEM,
             "plan needs about " + std::to_string(ps.est) + " device bytes, above max_bytes");
 
+  if (box3) box3_layout(*plan);
+  if (lighter)
+    *lighter = d == 1 || (ps.tr3 && spare_cols(*plan)) || (box3 && ps.est_arrays < box3_bytes(*plan, a_bytes));
+
   std::vector<int> bstart;
   build_pointset(*plan, plan->pts, x.ptr, w, sig, N, st, plan_alloc_cb, plan.get(), &bstart);
   GPN_CHECK(o.diag_correct == 0 || o.diag_correct == 1, GP_EINVAL, "diag_correct must be 0 or 1");
@@ -531,16 +545,17 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   const long long grid_pitch = (!plan->tr3 && !plan->rowfft) ? std::max(G, 2 * S) : G;
   plan->grid_bytes = (size_t)C * grid_rhs * grid_pitch * rs;
   GridView& v = plan->view;
-  v.cstride = G;
-  v.rstride = (long long)C * G;
-  for (long long q = d - 1, s = 1; q >= 0; --q, s *= h.nf) {
-    v.stride[q] = s;
-    v.ext[q] = (int)h.nf;
-  }
   if (box3) {
     box3_setup(*plan);
     plan->grid_bytes = (size_t)v.rstride * grid_rhs * rs;
     if (spread3d_supported(*plan)) build_spread3d_tiles(*plan, bstart);
+  } else {
+    v.cstride = G;
+    v.rstride = (long long)C * G;
+    for (long long q = d - 1, s = 1; q >= 0; --q, s *= h.nf) {
+      v.stride[q] = s;
+      v.ext[q] = (int)h.nf;
+    }
   }
   plan->grid = plan->alloc(plan->grid_bytes);
   GPN_CUDA(cudaMemsetAsync(plan->grid, 0, plan->grid_bytes, st));
@@ -608,16 +623,20 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   return plan.release();
 }
 
-// A plan, with its spare tables wherever they fit.
+// A plan, with its spare tables wherever they fit.  A plan that does not fit with them is built
+// again without them only where that needs less: not when the estimate or the host tables refuse it,
+// and of the 3-D ones only those whose box arrays are the larger ones (few channels in a box that
+// nearly fills the grid: the channels are padded to pairs).
 Plan* make_plan(const double* points, long long N, int d, const double* fa, const double* fb, double nu, double eps,
                 const gp_plan_opts& o, cudaStream_t st) {
+  bool lighter = false;
   try {
-    return build_plan(points, N, d, fa, fb, nu, eps, o, st, true);
+    return build_plan(points, N, d, fa, fb, nu, eps, o, st, true, &lighter);
   } catch (const Error& e) {
-    if (e.status != GP_ENOMEM) throw;
+    if (e.status != GP_ENOMEM || !lighter) throw;
     cudaGetLastError();   // clear a failed allocation's error state
   }
-  return build_plan(points, N, d, fa, fb, nu, eps, o, st, false);
+  return build_plan(points, N, d, fa, fb, nu, eps, o, st, false, nullptr);
 }
 
 // Resolve an output pointer: device pointers are written in place; host pointers go

@@ -801,9 +801,10 @@ bool tr3_supported(int d, long long nf, int precision) {
 // The pruned rows (about a third of what cuFFT reads and writes) pay in FP32 until a column needs
 // four passes and 512 threads (8192; with radix 32 and three passes .508); float64 is bound by
 // its pipe.  Below 256 a column leaves most of its warp idle.
-bool own_cols(const Plan& plan) {
-  if (plan.precision == GP_DF64) return true;
-  return plan.spare && plan.geom.nf >= 256 && plan.geom.nf <= (plan.precision == GP_FP32 ? 4096 : 8192);
+bool own_cols(const Plan& plan) { return plan.precision == GP_DF64 || spare_cols(plan); }
+bool spare_cols(const Plan& plan) {
+  const long long nf = plan.geom.nf;
+  return plan.precision != GP_DF64 && plan.spare && nf >= 256 && nf <= (plan.precision == GP_FP32 ? 4096 : 8192);
 }
 
 void tr3_setup(Plan& plan) {

@@ -624,8 +624,8 @@ void inverse_impl(Plan& plan, int R, cudaStream_t st) {
 bool box3_supported(int d, long long nf) { return d == 3 && nf <= 2048 && fft::mixed_plan((int)nf).np > 0; }
 
 // The box (the cells the support of any point or query of the plan's box can cover, and one
-// more on either side), the transform schedule and its tables, and the buffers.
-void box3_setup(Plan& plan) {
+// more on either side), the transform schedule, and the layout of the arrays.
+void box3_layout(Plan& plan) {
   const Hyper& h = plan.h;
   Box3& bx = plan.box3;
   const int C = plan.geom.C;
@@ -637,9 +637,8 @@ void box3_setup(Plan& plan) {
     bx.lo[q] = (int)std::max(0ll, lo);
     bx.ext[q] = (int)(std::min(h.nf, hi) - bx.lo[q]);
   }
-  const bool f32 = plan.precision == GP_FP32;
   bx.Cp = (C + 1) / 2 * 2;
-  const int lanes = f32 ? 2 : 1;
+  const int lanes = plan.precision == GP_FP32 ? 2 : 1;
   bx.Qe = ((h.M + 1) * ((C + lanes - 1) / lanes) + 7) / 8 * 8;
   bx.fft = fft::mixed_plan((int)h.nf);
   const int J = bx.fft.J, groups = (bx.Cp + 2 * lanes - 1) / (2 * lanes);
@@ -650,6 +649,22 @@ void box3_setup(Plan& plan) {
   const long long W = 2 * h.M + 1;
   bx.size_a = std::max((long long)bx.ext[0] * bx.ext[1], W * W) * bx.Qe;
   bx.size_b = (long long)bx.ext[0] * W * bx.Qe;
+  GridView& v = plan.view;
+  v.cstride = 1;
+  for (int q = 0; q < 3; ++q) {
+    v.lo[q] = bx.lo[q];
+    v.ext[q] = bx.ext[q];
+  }
+  v.stride[2] = bx.Cp;
+  v.stride[1] = v.stride[2] * bx.ext[2];
+  v.stride[0] = v.stride[1] * bx.ext[1];
+  v.rstride = v.stride[0] * bx.ext[0];
+}
+
+// the buffers of the spectra and the twiddle tables
+void box3_setup(Plan& plan) {
+  Box3& bx = plan.box3;
+  const bool f32 = plan.precision == GP_FP32;
   bx.buf_a = plan.alloc(16 * bx.size_a * plan.grid_rhs);
   bx.buf_b = plan.alloc(16 * bx.size_b * plan.grid_rhs);
   const std::vector<double> t = fft::mixed_tables(bx.fft);
@@ -662,17 +677,6 @@ void box3_setup(Plan& plan) {
   } else {
     GPN_CUDA(cudaMemcpy(bx.tw, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
   }
-  // the grids' layout
-  GridView& v = plan.view;
-  v.cstride = 1;
-  for (int q = 0; q < 3; ++q) {
-    v.lo[q] = bx.lo[q];
-    v.ext[q] = bx.ext[q];
-  }
-  v.stride[2] = bx.Cp;
-  v.stride[1] = v.stride[2] * bx.ext[2];
-  v.stride[0] = v.stride[1] * bx.ext[1];
-  v.rstride = v.stride[0] * bx.ext[0];
 }
 
 void box3_forward(Plan& plan, int R, cudaStream_t st) {

@@ -226,6 +226,7 @@ struct PlanShape {
   bool tr3 = false, rowfft = false, lean = false;
   long long G = 0, S = 0, nfreq = 0;
   long long a_bytes = 0, lean_bytes = 0, est_rest = 0, est = 0;
+  long long est_arrays = 0;              // of est: grids, spectra, their work area and the tensor
 };
 PlanShape plan_shape(int d, long long N, double nu, double eps, const gp_plan_opts& o, double smin, double smax,
                      const double* lo, const double* hi, long long free_b, Tables* tb);
@@ -352,6 +353,7 @@ void rowfft_inverse(Plan& plan, int R, cudaStream_t st);
 // transposed pruned transforms (d = 2, nf = 2^a)
 bool tr3_supported(int d, long long nf, int precision);
 bool own_cols(const Plan& plan);   // the plan's column transforms are the library's own
+bool spare_cols(const Plan& plan); // ... with tables that it can do without
 void tr3_setup(Plan& plan);
 void tr3_forward(Plan& plan, int R, cudaStream_t st);
 void tr3_diag(Plan& plan, int R, cudaStream_t st);
@@ -359,6 +361,7 @@ void tr3_inverse(Plan& plan, int R, cudaStream_t st);
 
 // 3-D transforms and step 3 over the occupied box (fft3d.cu)
 bool box3_supported(int d, long long nf);
+void box3_layout(Plan& plan);
 void box3_setup(Plan& plan);
 void box3_forward(Plan& plan, int R, cudaStream_t st);
 void box3_diag(Plan& plan, int R, cudaStream_t st);

@@ -216,3 +216,57 @@ def test_fp32_spread_of_a_dense_cloud_3d(gpn):
     alpha = 0.1 + torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
     plan, e = fp32_against_fp64(gpn, x, s, l, alpha, 2.5, 1e-4, box_lo=[0.0] * 3, box_hi=[1.0] * 3)
     assert e <= 6 * plan.info["kernel_beta"] * 2.0 ** -24, e
+
+
+def check_means(gpn, plan, w, wp, sig, p, precision):
+    """Both posterior means at the plan's own points against the oracle."""
+    alpha = gpinputs.random_alpha(plan.N, 1, seed=83)
+    ref = ktilde.apply_cross(w.points, wp, sig, w.points, wp, sig, alpha, p)
+    dev = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (alpha, w.points, w.s, w.l)]
+    assert rel(plan.posterior_mean(*dev).cpu().numpy(), ref) <= BAR[precision]
+    mu = torch.empty(plan.N, dtype=torch.float64, device="cuda")
+    gpn.abi.gp_posterior_mean_noalloc(plan.handle, *dev, mu)
+    assert rel(mu.cpu().numpy(), ref) <= BAR[precision]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("step3", [1, 2])
+def test_3d_plan_that_fits_without_the_box_alone(gpn, precision, step3):
+    """One channel in a box that nearly fills the grid: padded to a pair of channels the box needs
+    more than the full grid (FP32, and float64 with the memory-lean step 3).  Under a limit between
+    the two the plan is built on the full grid and computes the same K~; where the full grid needs
+    more, a limit below the box's bytes is refused."""
+    n = 300
+    w = small_case(3, n, 0)
+    s, l = np.ones(n), np.full(n, 0.05)
+    kw = dict(nu=2.5, eps=1e-3, max_rhs=2, step3=step3, precision=gpn.GP_FP64 if precision == "fp64" else gpn.GP_FP32)
+    box = gpn.Plan(w.points, s, l, **kw)
+    need = box.info["bytes_resident"]
+    assert box.info["n_sigma"] == 0
+    if precision == "fp64" and step3 == 1:
+        with pytest.raises(gpn.GPError):
+            gpn.Plan(w.points, s, l, max_bytes=need - 1, **kw)
+        return
+    full = gpn.Plan(w.points, s, l, max_bytes=need - 1, **kw)
+    assert full.info["bytes_resident"] < need and full.info["nf"] == box.info["nf"]
+    for seed in (101, 102):     # the second call finds the buffers used
+        a = torch.from_numpy(gpinputs.random_alpha(n, 2, seed=seed)).cuda()
+        assert rel(full.matvec(a).cpu().numpy(), box.matvec(a).cpu().numpy()) <= SAME[precision]
+    with pytest.raises(gpn.GPError):
+        gpn.Plan(w.points, s, l, max_bytes=need // 4, **kw)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf", [256, 2048])
+def test_2d_plan_without_spare_tables(gpn, precision, nf):
+    """A limit that the column transforms' tables do not fit: the plan takes cuFFT's columns."""
+    kw = dict(nf=nf, M=40, n_sigma=2, transform=3, max_rhs=2)
+    w, wp, sig, p, full = build(gpn, 2, 301, precision, **kw)
+    need = full.info["bytes_resident"]
+    *_, lean = build(gpn, 2, 301, precision, max_bytes=need - 1, **kw)
+    assert lean.info["bytes_resident"] < need
+    a = gpinputs.random_alpha(301, 2, seed=95)
+    ref = ktilde.matvec(w.points, wp, sig, a, p)
+    for plan in (full, lean):
+        assert rel(plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy(), ref) <= BAR[precision]
+    check_means(gpn, lean, w, wp, sig, p, precision)
