@@ -548,7 +548,7 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   if (box3) {
     box3_setup(*plan);
     plan->grid_bytes = (size_t)v.rstride * grid_rhs * rs;
-    if (spread3d_supported(*plan)) build_spread3d_tiles(*plan, bstart);
+    build_spread3d_tiles(*plan, bstart);
   } else {
     v.cstride = G;
     v.rstride = (long long)C * G;

@@ -280,7 +280,6 @@ int spread2d_rows(const Plan& plan);
 void build_spread2d_tiles(Plan& plan, const std::vector<int>& bstart);
 void launch_spread2d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st);
 // 3-D spreading with register accumulators on the box grids
-bool spread3d_supported(const Plan& plan);
 void build_spread3d_tiles(Plan& plan, const std::vector<int>& bstart);
 void launch_spread3d(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st);
 // Steps (2b)+(3)+(4a): deconvolve, apply A', zero outside the mode box (in spec).

@@ -42,8 +42,9 @@ struct SpreadArgs {
   int nbins[kMaxDim];
   const double* alpha;   // sorted order, N x R column-major
   long long n;
-  T* grid;               // fine grids, laid out as v says
-  GridView v;            // layout of the grid
+  T* grid;               // (R*C) x nf^d
+  long long nf;
+  long long G;           // nf^d
   int width;
   T beta;
   T inv_halfw;
@@ -264,11 +265,11 @@ __global__ void __launch_bounds__(256) k_spread(SpreadArgs<T> a) {
     __syncthreads();  // slots are reused by the next round
   }
 
-  // write the tile once (cells outside the grid in a partial tile are dropped)
+  // write the tile once (cells past nf in a partial last tile are dropped)
   const int vol = lead * TS;
   for (int i = threadIdx.x; i < vol; i += blockDim.x) {
     int rem = i;
-    long long gidx = 0;
+    long long gidx = 0, gstride = 1;
     int sidx = 0, sstride = 1;
     bool in = true;
 #pragma unroll
@@ -276,21 +277,22 @@ __global__ void __launch_bounds__(256) k_spread(SpreadArgs<T> a) {
       const int c = rem % TS;
       rem /= TS;
       const long long gq = (long long)base[q] + c;
-      in = in && gq >= a.v.lo[q] && gq < a.v.lo[q] + a.v.ext[q];
-      gidx += (gq - a.v.lo[q]) * a.v.stride[q];
+      in = in && gq < a.nf;
+      gidx += gq * gstride;
+      gstride *= a.nf;
       sidx += c * sstride;
       sstride *= (q == D - 1) ? TP : TS;
     }
     if (!in) continue;
-    T* dst = a.grid + r * a.v.rstride + ch0 * a.v.cstride + gidx;
+    T* dst = a.grid + ((size_t)r * a.Ctot + ch0) * a.G + gidx;
 #pragma unroll
     for (int k = 0; k < CMAX; ++k) {
       if (k < C) {
         if constexpr (kFixed) {
           const long long v = ((long long)tile[(size_t)k * TV + sidx] << 16) + tile[(size_t)(C + k) * TV + sidx];
-          dst[k * a.v.cstride] = __ll2float_rn(v) * inv_scale;
+          dst[(size_t)k * a.G] = __ll2float_rn(v) * inv_scale;
         } else {
-          dst[k * a.v.cstride] = tile[(size_t)k * TV + sidx];
+          dst[(size_t)k * a.G] = tile[(size_t)k * TV + sidx];
         }
       }
     }
@@ -331,7 +333,8 @@ void spread_impl(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st)
   a.alpha = alpha_sorted;
   a.n = ps.n;
   a.grid = (T*)plan.grid;
-  a.v = plan.view;
+  a.nf = g.nf;
+  a.G = plan.grid_elems;
   a.width = g.width;
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);

@@ -409,21 +409,17 @@ int tile_rows(const Plan& plan) {
 
 }  // namespace
 
-// The box plans whose bins are wide enough for the candidate table (else the general kernel)
-bool spread3d_supported(const Plan& plan) {
-  const GridGeom& g = plan.geom;
-  if (!plan.box3.on || g.C > kMaxChannels) return false;
-  const int TY = tile_rows(plan);
-  const int rows = ((kTZ + g.width - 2) / g.tile + 2) * ((TY + g.width - 2) / g.tile + 2);
-  return rows <= kMaxRanges && smem_bytes(plan.real_size, reg_channels(g.C), TY / kBands, g.width) <= 200 * 1024;
-}
-
 // Tiles whose candidate bins hold at least one point; the others stay zero.
 void build_spread3d_tiles(Plan& plan, const std::vector<int>& bstart) {
   const GridGeom& g = plan.geom;
   const PointSet& ps = plan.pts;
   const GridView& v = plan.view;
-  const int edge[3] = {kTZ, tile_rows(plan), kTX};
+  const int TY = tile_rows(plan), edge[3] = {kTZ, TY, kTX};
+  // the candidate table and the shared memory hold every box plan (bins are at least a support
+  // less a cell wide: at most 16 bin rows, and 191488 bytes with 32 float64 channels at width 16)
+  const int rows = ((kTZ + g.width - 2) / g.tile + 2) * ((TY + g.width - 2) / g.tile + 2);
+  GPN_CHECK(rows <= kMaxRanges && smem_bytes(plan.real_size, reg_channels(g.C), TY / kBands, g.width) <= 200 * 1024,
+            GP_EUNSUPPORTED, "3-D spread: bins too narrow or too many channels");
   int nt[3];
   std::vector<int> lo[3], hi[3];   // bins a tile's candidates come from, per axis
   for (int q = 0; q < 3; ++q) {

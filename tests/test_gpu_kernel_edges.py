@@ -270,3 +270,22 @@ def test_2d_plan_without_spare_tables(gpn, precision, nf):
     for plan in (full, lean):
         assert rel(plan.matvec(torch.from_numpy(a).cuda()).cpu().numpy(), ref) <= BAR[precision]
     check_means(gpn, lean, w, wp, sig, p, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf,M,n_sigma,step3,R,n", [
+    (88, 8, 3, 1, 2, 200),
+    (88, 8, 3, 2, 3, 200),
+    (132, 10, 5, 1, 1, 500),
+    (88, 7, 24, 1, 1, 150),      # more channels than a tile's shared memory holds (float64)
+    (88, 7, 31, 2, 1, 60),       # the most channels
+])
+def test_3d_plan_on_the_full_grid(gpn, precision, nf, M, n_sigma, step3, R, n):
+    """A grid size with a factor above 7: the full cube by cuFFT, the general spread in its channel
+    chunks, the staged interpolation, step 3 on the half spectrum, and both posterior means."""
+    kw = dict(nf=nf, M=M, n_sigma=n_sigma, step3=step3)
+    check_matvec(gpn, 3, n, precision, R, **kw)
+    w, wp, sig, p, plan = build(gpn, 3, n, precision, **kw)
+    if precision == "fp64" and n_sigma >= 24:
+        assert plan.info["tile"] ** 3 * (n_sigma + 1) * 8 > 160 * 1024
+    check_means(gpn, plan, w, wp, sig, p, precision)
