@@ -528,7 +528,7 @@ Plan* build_plan(const double* points, long long N, int d, const double* fa, con
   if (o.diag_correct) build_diag_correction(*plan, w, sig, st);
   GPN_CHECK(o.near_radius >= 0.0 && std::isfinite(o.near_radius), GP_EINVAL, "near_radius must be >= 0");
   if (o.near_radius > 0.0) build_near_field(*plan, o.near_radius, x.ptr, w, sig, st);
-  if (d == 1 && spare) line_points_setup(*plan, st);
+  if (d == 1) line_points_setup(*plan, st);
   build_active_tiles(*plan, bstart);
   if (spread2d_supported(*plan)) build_spread2d_tiles(*plan, bstart);
   GPN_CHECK(o.precision != GP_DF64 || plan->sp2_tiles, GP_EUNSUPPORTED,

@@ -64,7 +64,7 @@ struct Spread1Args {
   const T* xi;
   const T* psi;          // tabulated kernel values [n][width] (null: evaluate)
   const T* wk;           // [n][C]
-  const int* start;      // start[c]: first sorted point with l0 >= c, c <= nf
+  const int* start;      // start[c]: first sorted point with l0 >= c, c <= nf (null: searched for)
   int cell0, cell1;      // cells the points reach
   int cells;             // cells a block
   const double* alpha;   // n x R column-major
@@ -74,6 +74,19 @@ struct Spread1Args {
   int width, C, R;
   T beta, inv_halfw;
 };
+
+// first of the n sorted cells l0 that is >= c
+__device__ __forceinline__ int first_at(const int* __restrict__ l0, int n, int c) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (l0[mid] < c)
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  return lo;
+}
 
 // One thread takes one (cell, channel) pair, one block a run of `cells` cells.  The points that
 // reach the run are one contiguous run of the cell-sorted points; the block stages their kernel
@@ -90,11 +103,12 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread1d(Spread1Args<T> a) {
   T* s_amp = s_psi + kChunk * W;              // [kChunk][RB]: alpha, converted once a point
   int* s_l0 = reinterpret_cast<int*>(s_amp + kChunk * RB);
   const int c0 = a.cell0 + blockIdx.x * a.cells, c1 = min(c0 + a.cells, a.cell1);
-  const int p0 = a.start[max(0, c0 - W + 1)], p1 = a.start[c1];
+  const auto start = [&](int c) { return a.start ? a.start[c] : first_at(a.l0, (int)a.n, c); };
+  const int p0 = start(max(0, c0 - W + 1)), p1 = start(c1);
   const int ci = tid / C, k = tid - ci * C, cell = c0 + ci;
   const int pi = tid / W, j = tid - pi * W, pstep = kSpreadThreads / W;
   const bool on = ci < a.cells && cell < c1;
-  const int q0 = on ? a.start[max(0, cell - W + 1)] : 0, q1 = on ? a.start[cell + 1] : 0;
+  const int q0 = on ? start(max(0, cell - W + 1)) : 0, q1 = on ? start(cell + 1) : 0;
   const double* alpha = a.alpha + (size_t)r0 * a.n;
   T acc[RB];
 #pragma unroll
@@ -184,19 +198,10 @@ void spread_impl(Plan& plan, const double* alpha, const int* perm, int R, cudaSt
   GPN_CUDA(cudaGetLastError());
 }
 
-// start[c], c = 0 .. nf: first sorted point with l0 >= c
+// start[c], c = 0 .. nf
 __global__ void k_line_start(const int* __restrict__ l0, int n, int cells, int* __restrict__ start) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c > cells) return;
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (l0[mid] < c)
-      lo = mid + 1;
-    else
-      hi = mid;
-  }
-  start[c] = lo;
+  if (c <= cells) start[c] = first_at(l0, n, c);
 }
 
 // ---- interpolation ------------------------------------------------------------------------
@@ -672,16 +677,19 @@ bool line_supported(int d, long long nf, int precision, long long pitch) {
   return nf / 2 / kMaxSplit <= (1 << 20) && passes_fit((int)(nf / 2 / kMaxSplit), precision);
 }
 
-// where each cell's points start (every 1-D plan spreads with k_spread1d)
+// the cells the points reach and, with the spare tables, where each cell's points start (every 1-D
+// plan spreads with k_spread1d)
 void line_points_setup(Plan& plan, cudaStream_t st) {
   const PointSet& ps = plan.pts;
   const int n = (int)ps.n, cells = (int)plan.geom.nf;
   int first = 0, last = 0;
   GPN_CUDA(cudaMemcpyAsync(&first, ps.cell0[0], sizeof(int), cudaMemcpyDeviceToHost, st));
   GPN_CUDA(cudaMemcpyAsync(&last, ps.cell0[0] + n - 1, sizeof(int), cudaMemcpyDeviceToHost, st));
-  plan.line_start = (int*)plan.alloc(sizeof(int) * ((size_t)cells + 1));
-  k_line_start<<<blocks_for(cells + 1, 256), 256, 0, st>>>(ps.cell0[0], n, cells, plan.line_start);
-  GPN_CUDA(cudaGetLastError());
+  if (plan.spare) {
+    plan.line_start = (int*)plan.alloc(sizeof(int) * ((size_t)cells + 1));
+    k_line_start<<<blocks_for(cells + 1, 256), 256, 0, st>>>(ps.cell0[0], n, cells, plan.line_start);
+    GPN_CUDA(cudaGetLastError());
+  }
   GPN_CUDA(cudaStreamSynchronize(st));
   plan.line_cell0 = first;
   plan.line_cell1 = last + plan.geom.width;   // at most nf: no support leaves the grid

@@ -309,7 +309,7 @@ void matvec_sorted(Plan& plan, const double* alpha_sorted, double* out_sorted, i
 
 // 1-D plans read and write the caller's order themselves: two launches of nine fewer.
 void matvec_caller(Plan& plan, const double* alpha, double* out, int R, double shift, cudaStream_t st) {
-  if (plan.line_start && plan.near_nnz == 0) return matvec_blocks(plan, alpha, out, plan.pts.perm, R, shift, st);
+  if (plan.geom.d == 1 && plan.near_nnz == 0) return matvec_blocks(plan, alpha, out, plan.pts.perm, R, shift, st);
   gather_sorted(plan.pts, alpha, plan.vec_a, R, st);
   matvec_sorted(plan, plan.vec_a, plan.vec_b, R, shift, st);
   scatter_sorted(plan.pts, plan.vec_b, out, R, st);

@@ -187,11 +187,11 @@ struct Plan {
   void* query_ws = nullptr;
   size_t query_ws_bytes = 0;
   // d = 1 (line1d.cu): where each cell's points start, and the split transforms
-  int* line_start = nullptr;            // first sorted point with l0 >= c, c = 0..nf
+  int* line_start = nullptr;            // first sorted point with l0 >= c, c = 0..nf (spare)
   int line_cell0 = 0, line_cell1 = 0;   // cells the points reach
   // tables that only speed a plan up and are left out where it fits max_bytes (or the device)
-  // without them alone: the 1-D kernels' (then the tiled spread and the row or cuFFT transforms
-  // run), the 2-D column transforms' (then cuFFT's run) and the 3-D box's buffers
+  // without them alone: the 1-D kernels' (then the spread searches and evaluates what they hold, and
+  // the row or cuFFT transforms run), the 2-D column transforms' (then cuFFT's run) and the 3-D box's buffers
   bool spare = true;
   bool line = false;
   void* line_spec = nullptr;            // [r][C][nf/2] complex

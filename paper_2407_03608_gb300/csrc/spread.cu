@@ -2,9 +2,9 @@
 // for all Chebyshev channels k at once (the type-1 NUFFTs of step (2) share the
 // spreading pass).
 //
-// The general kernel, for the plans that the register-sum kernels of spread2d.cu, spread3d.cu
-// and line1d.cu do not take: 3-D plans without the box transforms, 1-D ones without their spare
-// tables, and those whose sums no thread can hold.
+// The general kernel, for the plans that the register-sum kernels of spread2d.cu and spread3d.cu
+// do not take: 3-D plans without the box transforms, and 2-D ones whose sums no thread can hold.
+// (1-D plans spread in line1d.cu.)
 //
 // Output-stationary tiling.  One CTA owns one tile of tile^d fine-grid cells for
 // one right-hand side and accumulates, in shared memory, the contributions of
@@ -15,8 +15,7 @@
 // (compacted through a shared counter) and tabulates their kernel values per axis
 // in shared memory; then a group of lanes works on each point: in 2-D one lane per
 // support row (a "pencil" of `width` cells along the last axis), in 3-D the warp's
-// lanes over the width^2 pencils, in 1-D one lane per point.  The tile is written
-// once with coalesced stores.  Only tiles
+// lanes over the width^2 pencils.  The tile is written once with coalesced stores.  Only tiles
 // some point can reach are launched (the plan's active-tile list): the other
 // cells of the spreading grid are zeroed once when the plan is built, and the
 // forward R2C transform leaves its input untouched.  No global atomics; the
@@ -355,11 +354,10 @@ void spread_impl(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st)
   }
   size_t smem = spread_smem_bytes(g.d, g.tile, cc, sizeof(T), g.width);
   dim3 grid((unsigned)plan.n_active_tiles, (unsigned)R, (unsigned)((g.C + cc - 1) / cc));
-  switch (g.d) {
-    case 1: launch_c<T, 1>(a, grid, smem, st); break;
-    case 2: launch_c<T, 2>(a, grid, smem, st); break;
-    default: launch_c<T, 3>(a, grid, smem, st);
-  }
+  if (g.d == 2)
+    launch_c<T, 2>(a, grid, smem, st);
+  else
+    launch_c<T, 3>(a, grid, smem, st);
   GPN_CUDA(cudaGetLastError());
 }
 
@@ -377,7 +375,7 @@ size_t spread_smem_bytes(int d, int tile, int C, size_t rs, int width) {
 
 void launch_spread(Plan& plan, const double* alpha_sorted, int R, cudaStream_t st) {
   if (plan.sp2_tiles) return launch_spread2d(plan, alpha_sorted, R, st);
-  if (plan.line_start) return launch_spread1d(plan, alpha_sorted, nullptr, R, st);
+  if (plan.geom.d == 1) return launch_spread1d(plan, alpha_sorted, nullptr, R, st);
   if (plan.sp3_tiles) return launch_spread3d(plan, alpha_sorted, R, st);
   if (plan.precision == GP_FP32)
     spread_impl<float>(plan, alpha_sorted, R, st);

@@ -289,3 +289,29 @@ def test_3d_plan_on_the_full_grid(gpn, precision, nf, M, n_sigma, step3, R, n):
     if precision == "fp64" and n_sigma >= 24:
         assert plan.info["tile"] ** 3 * (n_sigma + 1) * 8 > 160 * 1024
     check_means(gpn, plan, w, wp, sig, p, precision)
+
+
+def test_1d_plan_without_spare_tables_is_not_slow(gpn):
+    """1e5 float64 points: the spread searches and evaluates what the tables hold and the row kernels
+    transform, about twice the work in all (the tiled spread with its emulated float64 atomics took
+    80 times as long); ten times is refused."""
+    n = 100000
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.rand((n, 1), generator=g, device="cuda", dtype=torch.float64)
+    s, l = torch.ones(n, device="cuda", dtype=torch.float64), 0.02 + 0.06 * x[:, 0]
+    kw = dict(nu=1.5, eps=1e-5, precision=gpn.GP_FP64)
+    full = gpn.Plan(x, s, l, **kw)
+    lean = gpn.Plan(x, s, l, max_bytes=full.info["bytes_resident"] - 1, **kw)
+    a = torch.randn(n, generator=g, device="cuda", dtype=torch.float64)
+    ms = []
+    for plan in (full, lean):
+        out = plan.matvec(a)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        for _ in range(5):
+            plan.matvec(a, out=out)
+        t1.record()
+        torch.cuda.synchronize()
+        ms.append(t0.elapsed_time(t1))
+    assert ms[1] <= 10 * ms[0], ms
+    assert rel(lean.matvec(a).cpu().numpy(), full.matvec(a).cpu().numpy()) <= SAME["fp64"]
