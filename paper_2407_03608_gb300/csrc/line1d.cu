@@ -52,6 +52,40 @@ __device__ __forceinline__ void store_c(cpx<T>* p, cpx<T> v) {
   *reinterpret_cast<RawC<T>*>(p) = RawC<T>{v.x, v.y};
 }
 
+// The sum of exact products of FP32 values, in three words (about 72 bits): float64's precision on
+// the FP32 pipe (float64 sums run at a sixtieth of its rate, conversions at a sixteenth).  Largest
+// error over 2e5 sums of up to 32 terms, relative to the largest term: 3.1e-16, float64 1.7e-15, two words
+// 4.6e-14.
+struct Sum3 {
+  float a = 0.0f, b = 0.0f, c = 0.0f;
+
+  // + x + y, |y| below |x|'s last place or so
+  __device__ __forceinline__ void add(float x, float y) {
+    const dd s = two_sum(a, x), t = two_sum(b, s.lo), u = two_sum(t.hi, y);
+    a = s.hi;
+    b = u.hi;
+    c = ffops::add(c, ffops::add(t.lo, u.lo));
+  }
+  __device__ __forceinline__ explicit operator double() const { return (double)a + ((double)b + (double)c); }
+};
+__device__ __forceinline__ void add_product(double& sum, double w, double b) { sum += w * b; }
+__device__ __forceinline__ void add_product(Sum3& sum, float w, float b) {
+  const float p = ffops::mul(w, b);
+  sum.add(p, ffops::fma(w, b, -p));
+}
+__device__ __forceinline__ void add_value(double& sum, double x) { sum += x; }
+__device__ __forceinline__ void add_value(Sum3& sum, float x) { sum.add(x, 0.0f); }
+template <typename T>
+using SumOf = typename std::conditional<sizeof(T) == 4, Sum3, double>::type;
+
+// + the same of lane ^ o
+__device__ __forceinline__ void add_lane(double& sum, int o) { sum += shfl_xor_val(sum, o); }
+__device__ __forceinline__ void add_lane(Sum3& sum, int o) {
+  const float x = shfl_xor_val(sum.a, o), y = shfl_xor_val(sum.b, o), z = shfl_xor_val(sum.c, o);
+  sum.add(x, y);
+  sum.c = ffops::add(sum.c, z);
+}
+
 // ---- spreading --------------------------------------------------------------------------
 
 constexpr int kSpreadThreads = 256;
@@ -71,6 +105,7 @@ struct Spread1Args {
   long long n;
   T* grid;               // [r][k][nf]
   long long nf;
+  T* scratch;            // the parts' sums [part][r][k][cell1 - cell0], with more than one part
   int width, C, R;
   T beta, inv_halfw;
 };
@@ -115,11 +150,15 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread1d(Spread1Args<T> a) {
   const bool on = ci < a.cells && cell < c1;
   const int q0 = on ? start(max(0, cell - W + 1)) : 0, q1 = on ? start(cell + 1) : 0;
   const double* alpha = a.alpha + (size_t)r0 * a.n;
+  // this block's part of the run's chunks
+  const int chunks = (p1 - p0 + kChunk - 1) / kChunk, parts = gridDim.z;
+  const int b0 = p0 + (int)((long long)chunks * blockIdx.z / parts) * kChunk;
+  const int b1 = min(p1, p0 + (int)((long long)chunks * (blockIdx.z + 1) / parts) * kChunk);
   T acc[RB];
 #pragma unroll
   for (int r = 0; r < RB; ++r) acc[r] = T(0);
-  for (int base = p0; base < p1; base += kChunk) {
-    const int m = min(kChunk, p1 - base);
+  for (int base = b0; base < b1; base += kChunk) {
+    const int m = min(kChunk, b1 - base);
     for (int i = tid; i < m; i += kSpreadThreads) {
       s_l0[i] = a.l0[base + i];
       const int q = a.perm ? a.perm[base + i] : base + i;
@@ -148,7 +187,9 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread1d(Spread1Args<T> a) {
   }
   // the run's sums leave through shared memory, cells fastest
   T* s_out = reinterpret_cast<T*>(smem_raw);
-  const int nc = c1 - c0;
+  const int nc = c1 - c0, span = a.cell1 - a.cell0;
+  T* out = parts > 1 ? a.scratch + (size_t)blockIdx.z * a.R * C * span + (c0 - a.cell0) : a.grid + c0;
+  const long long pitch = parts > 1 ? span : a.nf;
 #pragma unroll
   for (int r = 0; r < RB; ++r) {
     if (r0 + r >= a.R) break;
@@ -156,19 +197,47 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spread1d(Spread1Args<T> a) {
     __syncthreads();
     for (int i = tid; i < nc * C; i += kSpreadThreads) {
       const int kk = i / nc, c = i - kk * nc;
-      a.grid[((size_t)(r0 + r) * C + kk) * a.nf + c0 + c] = s_out[kk * a.cells + c];
+      out[((size_t)(r0 + r) * C + kk) * pitch + c] = s_out[kk * a.cells + c];
     }
     __syncthreads();
   }
 }
 
+// the parts' sums, in their order: one thread a (right-hand side, channel, cell)
+template <typename T>
+__global__ void __launch_bounds__(256) k_spread1d_sum(Spread1Args<T> a, int parts) {
+  const int span = a.cell1 - a.cell0, total = a.R * a.C * span, i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= total) return;
+  SumOf<T> s{};
+  for (int p = 0; p < parts; ++p) add_value(s, a.scratch[(size_t)p * total + i]);
+  a.grid[(size_t)(i / span) * a.nf + a.cell0 + i % span] = (T)(double)s;
+}
+
+// right-hand sides a block takes, and cells of a block's run
+constexpr int spread_rhs(int R) { return R <= 2 ? R : 4; }
+int spread_cells(int C) { return std::max(1, kSpreadThreads / C); }
+
+// Parts the points of a run are divided into.  A short grid has few runs (64 cells of 4 channels:
+// one), and a thread walks all points of its cell: parts of a chunk or more, up to two blocks an SM.
+// nf = 64, 4 channels, ms a product without / with parts (and with the atomic or tiled spread of
+// before): float64 n = 1e4 1.01 / .056 (.76), 1e5 with 5 right-hand sides 21.1 / .24 (7.6), FP32 1e5
+// 3.71 / .084 (2.9); nf = 1024, 6 channels, n = 1e6: float64 8.80 / .59 (67), FP32 3.04 / .18 (32).
+int spread_parts(const Plan& plan, int R) {
+  const int span = plan.line_cell1 - plan.line_cell0, cells = spread_cells(plan.geom.C);
+  const long long blocks = (long long)((span + cells - 1) / cells) * ((R + spread_rhs(R) - 1) / spread_rhs(R));
+  if (!plan.spare || blocks >= 76) return 1;
+  const double points = (double)plan.pts.n * std::min(1.0, (double)(cells + plan.geom.width - 1) / span);   // a run's
+  return (int)std::max(1.0, std::min((double)((304 + blocks - 1) / blocks), points / kChunk));
+}
+
 template <typename T, int RB>
-void spread_launch(const Spread1Args<T>& a, int R, cudaStream_t st) {
+void spread_launch(const Spread1Args<T>& a, int R, int parts, cudaStream_t st) {
   const size_t smem = kChunk * ((a.C + a.width + RB) * sizeof(T) + sizeof(int));
   void (*k)(Spread1Args<T>) = a.start ? k_spread1d<T, RB, false> : k_spread1d<T, RB, true>;
   GPN_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int blocks = (a.cell1 - a.cell0 + a.cells - 1) / a.cells;
-  k<<<dim3((unsigned)blocks, (unsigned)((R + RB - 1) / RB)), kSpreadThreads, smem, st>>>(a);
+  k<<<dim3((unsigned)blocks, (unsigned)((R + RB - 1) / RB), (unsigned)parts), kSpreadThreads, smem, st>>>(a);
+  if (parts > 1) k_spread1d_sum<T><<<blocks_for((long long)R * a.C * (a.cell1 - a.cell0), 256), 256, 0, st>>>(a, parts);
 }
 
 template <typename T>
@@ -184,7 +253,7 @@ void spread_impl(Plan& plan, const double* alpha, const int* perm, int R, cudaSt
   a.start = plan.line_start;
   a.cell0 = plan.line_cell0;
   a.cell1 = plan.line_cell1;
-  a.cells = std::max(1, kSpreadThreads / g.C);
+  a.cells = spread_cells(g.C);
   a.alpha = alpha;
   a.n = ps.n;
   a.grid = (T*)plan.grid;
@@ -194,13 +263,14 @@ void spread_impl(Plan& plan, const double* alpha, const int* perm, int R, cudaSt
   a.beta = es_beta_arg<T>(g.beta);
   a.inv_halfw = (T)(2.0 / g.width);
   a.R = R;
+  a.scratch = (T*)plan.line_scratch;
+  const int parts = spread_parts(plan, R);
   // several right-hand sides a block share the staged points
-  if (R == 1)
-    spread_launch<T, 1>(a, R, st);
-  else if (R == 2)
-    spread_launch<T, 2>(a, R, st);
-  else
-    spread_launch<T, 4>(a, R, st);
+  switch (spread_rhs(R)) {
+    case 1: spread_launch<T, 1>(a, R, parts, st); break;
+    case 2: spread_launch<T, 2>(a, R, parts, st); break;
+    default: spread_launch<T, 4>(a, R, parts, st);
+  }
   GPN_CUDA(cudaGetLastError());
 }
 
@@ -235,36 +305,6 @@ __device__ __forceinline__ void finish_point(const Interp1Args<T>& a, long long 
   const long long i = (size_t)r * a.n + (a.perm ? a.perm[p] : p);
   if (a.alpha) res += (a.dcorr ? a.shift + a.dcorr[p] : a.shift) * a.alpha[i];
   a.out[i] = res;
-}
-
-// The sum of exact products of FP32 values, in three words (about 72 bits): float64's precision on
-// the FP32 pipe (float64 sums run at a sixtieth of its rate, conversions at a sixteenth).
-struct Sum3 {
-  float a = 0.0f, b = 0.0f, c = 0.0f;
-
-  // + x + y, |y| below |x|'s last place or so
-  __device__ __forceinline__ void add(float x, float y) {
-    const dd s = two_sum(a, x), t = two_sum(b, s.lo), u = two_sum(t.hi, y);
-    a = s.hi;
-    b = u.hi;
-    c = ffops::add(c, ffops::add(t.lo, u.lo));
-  }
-  __device__ __forceinline__ explicit operator double() const { return (double)a + ((double)b + (double)c); }
-};
-__device__ __forceinline__ void add_product(double& sum, double w, double b) { sum += w * b; }
-__device__ __forceinline__ void add_product(Sum3& sum, float w, float b) {
-  const float p = ffops::mul(w, b);
-  sum.add(p, ffops::fma(w, b, -p));
-}
-template <typename T>
-using SumOf = typename std::conditional<sizeof(T) == 4, Sum3, double>::type;
-
-// + the same of lane ^ o
-__device__ __forceinline__ void add_lane(double& sum, int o) { sum += shfl_xor_val(sum, o); }
-__device__ __forceinline__ void add_lane(Sum3& sum, int o) {
-  const float x = shfl_xor_val(sum.a, o), y = shfl_xor_val(sum.b, o), z = shfl_xor_val(sum.c, o);
-  sum.add(x, y);
-  sum.c = ffops::add(sum.c, z);
 }
 
 // Sixteen lanes a point: lane j holds psi(j), lane k sums channel k (k + 16, ...) over the W
@@ -699,6 +739,12 @@ void line_points_setup(Plan& plan, cudaStream_t st) {
   GPN_CUDA(cudaStreamSynchronize(st));
   plan.line_cell0 = first;
   plan.line_cell1 = last + plan.geom.width;   // at most nf: no support leaves the grid
+  size_t sums = 0;   // the most that the parts of any number of right-hand sides hold
+  for (int R = 1; R <= plan.grid_rhs; ++R) {
+    const size_t parts = spread_parts(plan, R);
+    if (parts > 1) sums = std::max(sums, parts * R * plan.geom.C * (plan.line_cell1 - plan.line_cell0));
+  }
+  if (sums) plan.line_scratch = plan.alloc(sums * plan.real_size);
 }
 
 // twiddles, pass tables of every split, and the cells the transforms read and write (the

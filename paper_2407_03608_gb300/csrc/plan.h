@@ -189,6 +189,7 @@ struct Plan {
   // d = 1 (line1d.cu): where each cell's points start, and the split transforms
   int* line_start = nullptr;            // first sorted point with l0 >= c, c = 0..nf (spare)
   int line_cell0 = 0, line_cell1 = 0;   // cells the points reach
+  void* line_scratch = nullptr;         // sums of the parts a spread's points are divided into (spare)
   // tables that only speed a plan up and are left out where it fits max_bytes (or the device)
   // without them alone: the 1-D kernels' (then the spread searches and evaluates what they hold, and
   // the row or cuFFT transforms run), the 2-D column transforms' (then cuFFT's run) and the 3-D box's buffers

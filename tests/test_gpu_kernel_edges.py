@@ -315,3 +315,14 @@ def test_1d_plan_without_spare_tables_is_not_slow(gpn):
         ms.append(t0.elapsed_time(t1))
     assert ms[1] <= 10 * ms[0], ms
     assert rel(lean.matvec(a).cpu().numpy(), full.matvec(a).cpu().numpy()) <= SAME["fp64"]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf,M,n_sigma,R,n", [
+    (64, 12, 3, 5, 20011),       # one run of cells, as many parts as fill the chip
+    (64, 12, 4, 2, 515),         # two parts, the last chunk of three points
+    (256, 40, 6, 1, 3000),       # a few runs and parts
+    (256, 40, 31, 3, 2500),
+])
+def test_1d_spread_in_parts(gpn, precision, nf, M, n_sigma, R, n):
+    check_matvec(gpn, 1, n, precision, R, nf=nf, M=M, n_sigma=n_sigma)
