@@ -27,6 +27,8 @@ namespace {
 // 64 an SM (32 registers, a few spilled outside the loop), above that what the registers allow
 template <int S>
 constexpr int kWarps = S <= 3 ? 16 : 8;
+// points a block takes, at most and where they still give two blocks an SM: 1000 points of 4 channels
+// at width 7 48 us with 64 a block, 18 with as many as warps (the staged kernel 18)
 constexpr int kPointsPerBlock = 64;
 
 template <typename T>
@@ -39,6 +41,7 @@ struct Interp3Args {
   GridView v;
   int width, C, Cp;
   int fold;              // half the power of two that holds C lanes
+  int per;               // points a block
   T beta, inv_halfw;
   const double* alpha;   // sorted order (may be null)
   double shift;
@@ -56,8 +59,8 @@ __global__ void __launch_bounds__(32 * kWarps<S>, S <= 3 ? 4 : 1) k_interp3d(Int
   const int last = W * a.Cp - 32 * (S - 1);   // lanes of the last slot inside the row
   __shared__ T s_sum[kWarps<S>][32 * S];   // a point's sums over z and y, in the order of a row
   T* sums = s_sum[warp];
-  const long long p1 = min(a.n, (long long)(blockIdx.x + 1) * kPointsPerBlock);
-  for (long long p = (long long)blockIdx.x * kPointsPerBlock + warp; p < p1; p += kWarps<S>) {
+  const long long p1 = min(a.n, (long long)(blockIdx.x + 1) * a.per);
+  for (long long p = (long long)blockIdx.x * a.per + warp; p < p1; p += kWarps<S>) {
     const int lz = a.l0[0][p] - a.v.lo[0], ly = a.l0[1][p] - a.v.lo[1], lx = a.l0[2][p] - a.v.lo[2];
     T pz = T(0), py = T(0), px = T(0);
     if (lane < W) {
@@ -102,11 +105,14 @@ __global__ void __launch_bounds__(32 * kWarps<S>, S <= 3 ? 4 : 1) k_interp3d(Int
 }
 
 template <typename T, int S>
-void dispatch(const Interp3Args<T>& a, dim3 grid, cudaStream_t st) {
-  if (a.width * a.Cp <= 32 * S)
-    k_interp3d<T, S><<<grid, 32 * kWarps<S>, 0, st>>>(a);
-  else if constexpr (S < kMaxWidth * kMaxChannels / 32)
-    dispatch<T, S + 1>(a, grid, st);
+void dispatch(Interp3Args<T> a, int R, cudaStream_t st) {
+  if (a.width * a.Cp <= 32 * S) {
+    const long long rounds = a.n / (304 * kWarps<S>);
+    a.per = (int)std::max<long long>(1, std::min<long long>(kPointsPerBlock / kWarps<S>, rounds)) * kWarps<S>;
+    k_interp3d<T, S><<<dim3((unsigned)((a.n + a.per - 1) / a.per), (unsigned)R), 32 * kWarps<S>, 0, st>>>(a);
+  } else if constexpr (S < kMaxWidth * kMaxChannels / 32) {
+    dispatch<T, S + 1>(a, R, st);
+  }
 }
 
 template <typename T>
@@ -132,7 +138,7 @@ void impl(Plan& plan, const PointSet& ps, const double* alpha_sorted, double shi
   a.shift = shift;
   a.dcorr = (&ps == &plan.pts) ? plan.dcorr : nullptr;
   a.out = out_sorted;
-  dispatch<T, 1>(a, dim3((unsigned)((ps.n + kPointsPerBlock - 1) / kPointsPerBlock), (unsigned)R), st);
+  dispatch<T, 1>(a, R, st);
   GPN_CUDA(cudaGetLastError());
 }
 
