@@ -485,9 +485,82 @@ __global__ void __launch_bounds__(kDiagM) k_box_diag_wide(BoxDiagArgs<T> a) {
     }
 }
 
+// Memory-lean FP32 with more channels: NB >= C of them.  A node's factors and the sums stay in
+// registers, the inputs in shared memory; the factors come as vectors.  (With factors, inputs and
+// sums re-read from memory at every node, 15 channels at nf 128 took 1015 us, 25 channels 1520; the
+// full-grid kernel 295 and 1001; this one 200 and 250.  Float64 keeps the form above: 3970 us
+// against 6290 on the full grid.)
+template <int NB>
+__global__ void __launch_bounds__(kDiagM) k_box_lean_wide(BoxDiagArgs<float> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int C = a.C, E = (C + 1) / 2, PITCH = E | 1;
+  cv<f2>* s_b = reinterpret_cast<cv<f2>*>(smem_raw);           // [kDiagM][PITCH]
+  float* s_em = reinterpret_cast<float*>(s_b + kDiagM * PITCH);   // [J][CP]
+  const int ny = blockIdx.y, nz = blockIdx.z, m0 = blockIdx.x * kDiagM, t = threadIdx.x;
+  const int Mp = a.M + 1, nm = min(kDiagM, Mp - m0);
+  long long row[4];
+  const int ns = sign_rows(nz, ny, a.M, row);
+  stage_factors(a, s_em, nz, ny);
+  const float* tm = a.tab + (size_t)(m0 + min(t, nm - 1)) * a.CP;
+  const size_t jstride = (size_t)Mp * a.CP;
+  cv<f2>* b = s_b + t * PITCH;
+  for (int r = 0; r < a.R; ++r)
+    for (int s = 0; s < ns; ++s) {
+      cv<f2>* Xs = a.X + r * a.xr + row[s] * a.Qe + (size_t)m0 * E;
+      for (int e = t; e < nm * E; e += kDiagM) store_v(s_b + e / E * PITCH + e % E, load_v(Xs + e));
+      __syncthreads();
+      if (t < nm) {
+        float ox[NB], oy[NB];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) ox[k] = oy[k] = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < a.J; ++j) {
+          float g[NB];
+#pragma unroll
+          for (int v = 0; v < NB / 4; ++v) {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), e = x;
+            if (4 * v < a.CP) {
+              x = __ldg(reinterpret_cast<const float4*>(tm + j * jstride) + v);
+              e = reinterpret_cast<const float4*>(s_em + j * a.CP)[v];
+            }
+            g[4 * v] = x.x * e.x, g[4 * v + 1] = x.y * e.y, g[4 * v + 2] = x.z * e.z, g[4 * v + 3] = x.w * e.w;
+          }
+          float ux = 0.f, uy = 0.f;
+#pragma unroll
+          for (int e = 0; e < NB / 2; ++e)
+            if (e < E) {
+              const cv<f2> v = load_v(b + e);
+              ux += g[2 * e] * v.x.x + g[2 * e + 1] * v.x.y;
+              uy += g[2 * e] * v.y.x + g[2 * e + 1] * v.y.y;
+            }
+#pragma unroll
+          for (int k = 0; k < NB; ++k) {
+            ox[k] += g[k] * ux;
+            oy[k] += g[k] * uy;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < NB / 2; ++e)
+          if (e < E) store_v(b + e, cv<f2>{{ox[2 * e], ox[2 * e + 1]}, {oy[2 * e], oy[2 * e + 1]}});
+      }
+      __syncthreads();
+      for (int e = t; e < nm * E; e += kDiagM) store_v(Xs + e, load_v(s_b + e / E * PITCH + e % E));
+      __syncthreads();
+    }
+}
+
+void lean_wide_launch(const BoxDiagArgs<float>& a, dim3 grid, cudaStream_t st) {
+  void (*k)(BoxDiagArgs<float>) = a.C <= 16 ? k_box_lean_wide<16> : a.C <= 24 ? k_box_lean_wide<24> : k_box_lean_wide<32>;
+  const size_t smem = 16 * kDiagM * (size_t)((a.C + 1) / 2 | 1) + sizeof(float) * a.J * a.CP;
+  GPN_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k<<<grid, kDiagM, smem, st>>>(a);
+}
+
 template <typename T, int NC, bool LEAN>
 void diag_launch(const BoxDiagArgs<T>& a, dim3 grid, cudaStream_t st) {
-  if constexpr (NC > 12) {
+  if constexpr (NC > 12 && LEAN && sizeof(T) == 4) {
+    lean_wide_launch(a, grid, st);
+  } else if constexpr (NC > 12) {
     const int E = (a.C + kLanes<T> - 1) / kLanes<T>;
     const size_t smem = 2 * 16 * kDiagM * (E | 1) + (LEAN ? sizeof(T) * a.J * a.CP : 0);
     GPN_CUDA(cudaFuncSetAttribute(k_box_diag_wide<T, LEAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -326,3 +326,10 @@ def test_1d_plan_without_spare_tables_is_not_slow(gpn):
 ])
 def test_1d_spread_in_parts(gpn, precision, nf, M, n_sigma, R, n):
     check_matvec(gpn, 1, n, precision, R, nf=nf, M=M, n_sigma=n_sigma)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("n_sigma,M", [(14, 8), (15, 8), (16, 10), (22, 8), (23, 5), (24, 8)])
+def test_box_memory_lean_with_many_channels(gpn, precision, n_sigma, M):
+    """Channel counts around the register blocks of 16, 24 and 32, two right-hand sides."""
+    check_matvec(gpn, 3, 80, precision, 2, nf=64, M=M, n_sigma=n_sigma, step3=2)
