@@ -685,12 +685,18 @@ constexpr size_t kRowSmemMaxDD = size_t(215) << 10;
 template <typename T>
 constexpr size_t row_smem_max() { return is_dd<T>::value ? kRowSmemMaxDD : kRowSmemMax; }
 
+// FP32 inverse rows of few short grids: a row a block instead of packed pairs (rows2d.cu), whose
+// longer chains show where the launch is short.  us without / with pairs: 5 grids nf 32 6.3 / 10.2, 256
+// and 512 8.2 / 10.2, 1024 17.0 / 14.5; 40 grids nf 32 10.2 / 10.2, 64 14.3 / 12.2, 256 20.3 / 12.1.
+constexpr int kShortRows = 8;       // nf / 2 = 2^8
+constexpr long long kShortGrids = 8;
+
 template <typename T, int L, int RB>
 void rows_launch(bool inv, const RowsArgs<T>& a, cudaStream_t st) {
   const size_t smem = inv ? row_smem<T, true>(L, RB) : row_smem<T, false>(L, RB);
   const int threads = RB * (1 << L) / 16;
   void (*k)(RowsArgs<T>) = k_rows_fwd<T, L, RB>;
-  if constexpr (sizeof(T) == 8) {   // (FP32 inverse rows: rows2d.cu)
+  if constexpr (sizeof(T) == 8 || L <= kShortRows) {   // (other FP32 inverse rows: rows2d.cu)
     if (inv) k = k_rows_inv<T, L, RB>;
   }
   GPN_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -764,7 +770,7 @@ void rows_run(Plan& plan, bool inv, const void* X, int R, cudaStream_t st) {
   a.nitems = a.npairs * plan.geom.C * R;
   const int L = log2_exact(plan.geom.nf / 2);
   if constexpr (sizeof(T) == 4) {
-    if (inv) {
+    if (inv && (L > kShortRows || (long long)plan.geom.C * R > kShortGrids)) {
       rows_pairs_inv(L, a, plan.row_lo, plan.geom.C * R, st);
       GPN_CUDA(cudaGetLastError());
       return;

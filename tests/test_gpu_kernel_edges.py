@@ -333,3 +333,10 @@ def test_1d_spread_in_parts(gpn, precision, nf, M, n_sigma, R, n):
 def test_box_memory_lean_with_many_channels(gpn, precision, n_sigma, M):
     """Channel counts around the register blocks of 16, 24 and 32, two right-hand sides."""
     check_matvec(gpn, 3, 80, precision, 2, nf=64, M=M, n_sigma=n_sigma, step3=2)
+
+
+@pytest.mark.parametrize("nf,M,R", [(64, 16, 2), (64, 16, 3), (512, 30, 2), (512, 30, 3), (1024, 30, 1)])
+def test_fp32_inverse_rows_of_few_and_of_many_grids(gpn, nf, M, R):
+    """Three channels: up to 8 grids of nf <= 512 take a row a block, more (or longer rows) packed
+    pairs of rows."""
+    check_matvec(gpn, 2, 97, "fp32", R, nf=nf, M=M, n_sigma=2, transform=3)
