@@ -625,6 +625,7 @@ LinePlan line_passes(int n, int precision) {
   return m;
 }
 bool passes_fit(int n, int precision) { return line_passes(n, precision).N > 0; }
+constexpr long long kMaxLine = 1 << 17;   // eight blocks of 8192 points (512 threads)
 
 // the pass twiddles W_{Ns R}^{r k}, [r - 1][k], k < Ns, as interleaved (re, im)
 std::vector<double> line_tables(const LinePlan& m) {
@@ -643,8 +644,9 @@ std::vector<double> line_tables(const LinePlan& m) {
 
 // Blocks a transform is split over: the fewest that give kLineBlocks blocks (every block reads
 // the whole sequence, so S multiplies the reads from L2), more where the sub-transform would
-// not fit a block, fewer where it would drop below 64 points.  Measured at N = 1e5 FP32 with
-// 40 sequences of 32768: 29 us with S = 8.
+// not fit a block, fewer where it would drop below 64 points.  40 FP32 sequences of 32768 (N = 1e5, four
+// right-hand sides) take S = 4, 36 us forward and 34 back; with S = 8 30 and 29; 40 of 16384 S = 4, 19
+// and 18 (S = 8 19 and 16); 80 of 32768 S = 4, 50 and 47.
 int line_split(const Plan& plan, int CR) {
   const int h = (int)(plan.geom.nf / 2);
   int S = 1;
@@ -720,7 +722,7 @@ void* upload(Plan& plan, const std::vector<double>& v) {
 // values per channel of the buffer the spectra can live in.
 bool line_supported(int d, long long nf, int precision, long long pitch) {
   if (d != 1 || nf < 64 || (nf & (nf - 1)) || nf / 2 > pitch || precision == GP_DF64) return false;
-  return nf / 2 / kMaxSplit <= (1 << 20) && passes_fit((int)(nf / 2 / kMaxSplit), precision);
+  return nf <= kMaxLine && passes_fit((int)(nf / 2 / kMaxSplit), precision);
 }
 
 // the cells the points reach and, with the spare tables, where each cell's points start (every 1-D

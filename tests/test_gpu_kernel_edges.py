@@ -340,3 +340,11 @@ def test_fp32_inverse_rows_of_few_and_of_many_grids(gpn, nf, M, R):
     """Three channels: up to 8 grids of nf <= 512 take a row a block, more (or longer rows) packed
     pairs of rows."""
     check_matvec(gpn, 2, 97, "fp32", R, nf=nf, M=M, n_sigma=2, transform=3)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nf,M,R", [(1 << 17, 400, 1), (1 << 17, 700, 10), (1 << 18, 300, 1)])
+def test_longest_split_transforms_1d(gpn, precision, nf, M, R):
+    """nf = 2^17: eight blocks of 8192 points a sequence (the most a block takes); 2^18: the first
+    length that is left to the full-grid transform."""
+    check_matvec(gpn, 1, 257, precision, R, nf=nf, M=M, n_sigma=3, transform=1)
