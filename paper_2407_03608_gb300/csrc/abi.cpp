@@ -241,7 +241,9 @@ void build_active_tiles(Plan& plan, const std::vector<int>& bstart) {
 }
 
 // Rows (first axis) and columns (last axis) of the fine grid that hold spread data
-// or that the interpolation reads: the active tiles' extent plus one kernel width.
+// or that the interpolation reads: the active tiles' extent plus one kernel width, and the
+// cells the support of any query in the plan's box can cover (a given box may reach far beyond
+// the points).
 void set_data_extent(Plan& plan) {
   const int d = plan.h.d, TS = plan.h.tile;
   const long long nf = plan.h.nf;
@@ -260,6 +262,14 @@ void set_data_extent(Plan& plan) {
   }
   if (t.empty())
     for (int q = 0; q < d; ++q) lo[q] = hi[q] = 0;
+  for (int q = 0; q < d; ++q) {
+    const Hyper& h = plan.h;
+    const double half = 0.5 * (h.box_hi[q] - h.box_lo[q]) * h.nf * h.dw;
+    const long long first = (long long)std::ceil(0.5 * nf - half - 0.5 * h.width) - 1;
+    const long long last = (long long)std::ceil(0.5 * nf + half - 0.5 * h.width) + h.width + 1;
+    lo[q] = std::min(lo[q], std::max(0ll, first) / TS * TS);
+    hi[q] = std::max(hi[q], std::min(nf, last));
+  }
   plan.col_lo = (int)lo[d - 1];
   plan.col_hi = (int)hi[d - 1];
   plan.row_lo = d == 2 ? (int)lo[0] : 0;

@@ -348,3 +348,27 @@ def test_longest_split_transforms_1d(gpn, precision, nf, M, R):
     """nf = 2^17: eight blocks of 8192 points a sequence (the most a block takes); 2^18: the first
     length that is left to the full-grid transform."""
     check_matvec(gpn, 1, 257, precision, R, nf=nf, M=M, n_sigma=3, transform=1)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "df64"])
+@pytest.mark.parametrize("d,transform", [(1, 0), (1, 2), (2, 3), (2, 2), (2, 1), (3, 0)])
+def test_posterior_mean_outside_the_points_in_a_given_box(gpn, precision, d, transform):
+    """The box may be given larger than the points; queries anywhere in it read cells that no
+    point reaches.  Against the dense kernel, at ten times the accuracy the plan is asked for."""
+    if precision == "df64" and transform != 3:
+        pytest.skip("float-float plans take transform 3 alone")
+    g = np.random.default_rng(103)
+    n, m = 400, 300
+    x, q = 0.48 + 0.04 * g.random((n, d)), 0.05 + 0.9 * g.random((m, d))
+    s, l, sq, lq = np.ones(n), np.full(n, 0.1), np.ones(m), np.full(m, 0.1)
+    alpha = g.random(n)
+    plan = gpn.Plan(x, s, l, nu=2.5, eps=1e-4, precision={"fp64": gpn.GP_FP64, "fp32": gpn.GP_FP32, "df64": gpn.GP_DF64}[precision],
+                    box_lo=[0.0] * d, box_hi=[1.0] * d, transform=transform, **({"nf": 512} if d < 3 else {}))
+    wx, sx = okern.paper_fields(s, l, d)
+    wq, sgq = okern.paper_fields(sq, lq, d)
+    ref = okern.kernel_dense(np.concatenate([q, x]), np.concatenate([wq, wx]), np.concatenate([sgq, sx]), 2.5)[:m, m:] @ alpha
+    dev = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in (alpha, q, sq, lq)]
+    assert rel(plan.posterior_mean(*dev).cpu().numpy(), ref) <= 1e-3
+    mu = torch.empty(m, dtype=torch.float64, device="cuda")
+    gpn.abi.gp_posterior_mean_noalloc(plan.handle, *dev, mu)
+    assert rel(mu.cpu().numpy(), ref) <= 1e-3
