@@ -68,6 +68,12 @@ struct Sum3 {
   }
   __device__ __forceinline__ explicit operator double() const { return (double)a + ((double)b + (double)c); }
 };
+__device__ __forceinline__ void set_product(double& sum, double w, double b) { sum = w * b; }
+__device__ __forceinline__ void set_product(Sum3& sum, float w, float b) {
+  sum.a = ffops::mul(w, b);
+  sum.b = ffops::fma(w, b, -sum.a);
+  sum.c = 0.0f;
+}
 __device__ __forceinline__ void add_product(double& sum, double w, double b) { sum += w * b; }
 __device__ __forceinline__ void add_product(Sum3& sum, float w, float b) {
   const float p = ffops::mul(w, b);
@@ -331,7 +337,10 @@ __global__ void __launch_bounds__(128) k_interp1d_lanes(Interp1Args<T> a) {
 #pragma unroll
     for (int j = 0; j < kMaxWidth; ++j)
       if (j < W) s += __shfl_sync(0xffffffffu, pj, j, 16) * v[j];
-    add_product(part, w, s);
+    if (k0 == 0)
+      set_product(part, w, s);
+    else
+      add_product(part, w, s);
   }
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) add_lane(part, o);
