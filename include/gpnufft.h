@@ -103,8 +103,9 @@ typedef struct gp_plan_opts {
                                library's own transforms over the box of cells the
                                plan's points and queries can reach, and from them to
                                the modes |n_a| <= M (then info.bytes_resident is well
-                               below gp_plan_params' estimate); d = 1 with nf = 2^a:
-                               the library's own split transforms;
+                               below gp_plan_params' estimate, which counts the full
+                               grid, except with a single channel); d = 1 with
+                               nf = 2^a <= 2^17: the library's own split transforms;
                              2 pruned (d <= 2, nf = 2^a): d = 2 custom shared-memory row
                                FFTs keeping modes 0..M, cuFFT along the first axis;
                                d = 1 the split transforms, or the row FFTs where the

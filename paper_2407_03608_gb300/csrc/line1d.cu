@@ -23,7 +23,7 @@
 // Bound: latency (five launches of 7 to 15 us), the FP64 pipe in the float64 transforms.  A matvec,
 // against the tiled or atomic spread, row or cuFFT transforms and a lane-a-point interpolation:
 // N = 2000 float64 (15 channels, nf 8192) 235 -> 57 us, N = 1e5 FP32 with 4 right-hand sides (10
-// channels, nf 65536) 217 -> 125 us.
+// channels, nf 65536) 217 -> 127 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

@@ -166,15 +166,23 @@ void interp_impl(const Plan& plan, const PointSet& qs, double* mu, cudaStream_t 
 
 // Query sets evaluated without binning: the 1-D, 2-D and 3-D box plans', up to the sizes where
 // the unsorted reads of the supports cost more than the sort.  A posterior mean without / with
-// binning, ms (1e5 training points, 2e4 in 3-D float64):
-//   1-D FP32         1e5 queries .25 / .68   1e6 1.21 / 1.71
-//   2-D FP32         1e5 1.36 / 1.79         2.5e5 1.82 / 2.18     1e6 4.25 / 2.73
-//   2-D float-float  1e5 4.28 / 4.66         2.5e5 5.16 / 5.14     1e6 9.73 / 6.19
-//   2-D float64      1e5 4.70 / 4.74         2.5e5 5.89 / 5.41     1e6 11.9 / 7.28
-//   3-D FP32         2e3 1.54 / 1.71         2e5 2.08 / 2.75
-//   3-D float64      2e3 11.4 / 11.6         2e5 16.8 / 17.8
-// (2-D float64: the kernel values of an unbinned query are not tabulated, and their float64
-// arithmetic sets the line.)
+// binning, ms (training points, grid, channels in brackets):
+//   1-D FP32         [1e5, nf 32768, 8]       1e5 queries .19 / .65   1e6 .83 / 1.48   4e6 2.4 / 2.9
+//   1-D float64      [1e5, nf 32768, 8]       1e5 .43 / .84           1e6 1.4 / 2.4    4e6 4.4 / 5.8
+//   2-D FP32         [1e6, nf 8192, 8]        1e4 4.41 / 4.92         1e5 4.73 / 5.63  2.6e5 5.31 / 5.96
+//                    [1e4, nf 512, 5]         1e4 .14 / .29           1e5 .25 / .74    2.6e5 .43 / 1.09
+//                    [1e5, nf 4096, 8]        1e5 1.36 / 1.79         2.5e5 1.82 / 2.18   1e6 4.25 / 2.73
+//   2-D float-float  [1e6, nf 4096, 7]        1e5 4.41 / 4.95         2.6e5 5.20 / 5.25
+//                    [1e5, nf 4096]           1e5 4.28 / 4.66         2.5e5 5.16 / 5.14   1e6 9.73 / 6.19
+//   2-D float64      [1e5, nf 2048, 6]        1e4 3.10 / 3.27         1.3e5 3.97 / 4.08
+//                    [1e5, nf 4096]           1e5 4.70 / 4.74         2.5e5 5.89 / 5.41   1e6 11.9 / 7.28
+//   3-D FP32         [2e6, nf 540, 7]         1e4 9.43 / 9.99         1e5 9.77 / 10.7     2.6e5 10.4 / 11.4
+//                    [2e6, nf 800, 8]         1e4 27.3 / 28.2         1e5 27.8 / 29.4     2.6e5 28.7 / 30.2
+//                    [2e4, nf 140, 5]         1e4 .37 / .55           1e5 .54 / 1.18      2.6e5 .87 / 1.72
+//   3-D float64      [2e4, nf 256, 6]         1e4 9.28 / 9.47         1e5 11.0 / 11.8     2.6e5 14.2 / 15.2
+// So the grids' size against the L2 moves the line little, and in 3-D nothing lost up to the count
+// that was measured, where the line is drawn.  (2-D float64: the kernel values of an unbinned query
+// are not tabulated, and their float64 arithmetic sets the line.  The 3-D interpolation has gained since.)
 bool query_unbinned(const Plan& plan, long long n) {
   if (plan.geom.d == 1) return n < (1ll << 31);   // (more are refused by the binning, as ever)
   if (plan.geom.d == 3) return plan.box3.on && n <= (1 << 18);
