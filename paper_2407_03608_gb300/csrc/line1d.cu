@@ -227,11 +227,13 @@ int spread_cells(int C) { return std::max(1, kSpreadThreads / C); }
 // one), and a thread walks all points of its cell: parts of a chunk or more, up to two blocks an SM.
 // nf = 64, 4 channels, ms a product without / with parts (and with the atomic or tiled spread of
 // before): float64 n = 1e4 1.01 / .056 (.76), 1e5 with 5 right-hand sides 21.1 / .24 (7.6), FP32 1e5
-// 3.71 / .084 (2.9); nf = 1024, 6 channels, n = 1e6: float64 8.80 / .59 (67), FP32 3.04 / .18 (32).
+// 3.71 / .084 (2.9); nf = 1024, 6 channels, n = 1e6: float64 8.80 / .59 (67), FP32 3.04 / .18 (32).  The
+// spread alone at n = 1e6, us, FP32 / float64: 94 runs 439 / 1630 whole and 138 / 600 in parts, 154 runs
+// 365 / 1330 and 215 / 956, 187 runs 240 / 914 and 138 / 579; 307 runs (whole by the rule) 206 / 977.
 int spread_parts(const Plan& plan, int R) {
   const int span = plan.line_cell1 - plan.line_cell0, cells = spread_cells(plan.geom.C);
   const long long blocks = (long long)((span + cells - 1) / cells) * ((R + spread_rhs(R) - 1) / spread_rhs(R));
-  if (!plan.spare || blocks >= 76) return 1;
+  if (!plan.spare || blocks >= 304) return 1;
   const double points = (double)plan.pts.n * std::min(1.0, (double)(cells + plan.geom.width - 1) / span);   // a run's
   return (int)std::max(1.0, std::min((double)((304 + blocks - 1) / blocks), points / kChunk));
 }

@@ -323,6 +323,7 @@ def test_1d_plan_without_spare_tables_is_not_slow(gpn):
     (64, 12, 4, 2, 515),         # two parts, the last chunk of three points
     (256, 40, 6, 1, 3000),       # a few runs and parts
     (256, 40, 31, 3, 2500),
+    (4096, 200, 8, 1, 30011),    # a hundred runs, two parts
 ])
 def test_1d_spread_in_parts(gpn, precision, nf, M, n_sigma, R, n):
     check_matvec(gpn, 1, n, precision, R, nf=nf, M=M, n_sigma=n_sigma)
